@@ -298,6 +298,25 @@ void refresh_group_terms(art_portfolio* p) {
     }
 }
 
+// Whether a layer's FP32 occurrence losses are whole numbers below 2^32 of
+// some unit 2^e (see ylt_fixed.cu): multiples of ulp(OccR) (and of ulp(OccL),
+// the finer of the two), at most min(OccL, the sum of the ELT limits).
+bool whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units) {
+    if (!(occ_ret >= 0x1p-60f) || !(occ_ret <= 0x1p100f)) return false;
+    int er, el;
+    std::frexp(occ_ret, &er);  // occ_ret in [2^(er - 1), 2^er): its ulp is 2^(er - 24)
+    *e = er - 24;
+    double bound = elt_lim_sum * 1.0001;  // the FP32 sum may round up
+    if (std::isfinite(occ_lim)) {
+        if (!(occ_lim >= 0x1p-60f)) return false;
+        std::frexp(occ_lim, &el);
+        *e = std::min(*e, el - 24);
+        bound = std::min(bound, (double)occ_lim);
+    }
+    *max_units = std::ldexp(bound, -*e);
+    return *max_units <= 4294967295.0;
+}
+
 // Terms of every layer as the occurrence-table build reads them, and the
 // aggregate terms of the occurrence groups (kernel parameters).
 cudaError_t upload_layer_build(art_portfolio* p) {
@@ -316,7 +335,24 @@ cudaError_t upload_layer_build(art_portfolio* p) {
         a.occ_ret = p->occ_ret[j];
         a.occ_lim = p->occ_lim[j];
         a.np = p->layer_np[j];
-        a.pad_ = 0;
+        a.fix_scale = 0.0f;
+    }
+    // a skip group's X holds whole numbers where every layer's losses allow it
+    for (OccGroupArgs& g : p->ogroups) {
+        int e[kMaxOccLayers];
+        double top = 1.0;
+        g.sum_fits = 1;
+        for (int s = 0; s < g.n_layers && g.sum_fits; ++s) {
+            const int32_t j = g.layer[s];
+            double lims = 0.0, units;
+            for (int c = p->loff[j]; c < p->loff[j + 1]; ++c) lims += p->lim[p->lids[c]];
+            if (whole_losses(p->occ_ret[j], p->occ_lim[j], lims, &e[s], &units)) top = std::max(top, units);
+            else g.sum_fits = 0;
+        }
+        for (int s = 0; s < kMaxOccLayers; ++s) g.unit[s] = g.sum_fits && s < g.n_layers ? std::ldexp(1.0, e[s]) : 0.0;
+        if (!g.sum_fits) continue;
+        g.sum_fits = (int32_t)std::min(4294967295.0 / top, 64.0);
+        for (int s = 0; s < g.n_layers; ++s) lb[g.layer[s]].fix_scale = (float)std::ldexp(1.0, -e[s]);
     }
     for (std::vector<OccGroupArgs>* v : {&p->ogroups, &p->ogroups64})
         for (OccGroupArgs& g : *v)
@@ -1161,6 +1197,7 @@ art_status art_get_device_status(art_portfolio* p, cudaStream_t stream) {
     if (!e) e = cudaMemcpy(flags, p->d_flags, sizeof(flags), cudaMemcpyDeviceToHost);
     if (!e) e = cudaMemset(p->d_flags, 0, sizeof(flags));
     if (e) return fail(e);
+    if (flags[kFlagTimeout]) return ART_ETIMEOUT;
     if (flags[kFlagIdRange]) return ART_EID_RANGE;
     if (flags[kFlagBadOffsets]) return ART_EINVAL;
     return ART_OK;

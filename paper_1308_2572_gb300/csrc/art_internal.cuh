@@ -21,7 +21,7 @@ constexpr int kMaxPoolElts = 512;   // widest pool row the batched kernel reads
 constexpr int kMaxProbs = 8;        // probabilities per art_metrics call
 
 // Error flag slots in the portfolio's device flag array.
-enum { kFlagIdRange = 0, kFlagBadOffsets = 1, kNumFlags = 4 };
+enum { kFlagIdRange = 0, kFlagBadOffsets = 1, kFlagTimeout = 2, kNumFlags = 4 };
 
 // XL(v; R, L) = min(max(v - R, 0), L), the excess-of-loss form of the
 // occurrence (Algorithm 1 step 3) and aggregate (step 4) terms.
@@ -280,6 +280,10 @@ struct OccGroupArgs {
     int32_t layer[kMaxOccLayers];
     double agg_ret[kMaxOccLayers], agg_lim[kMaxOccLayers];
     int32_t n_layers;
+    // X holds whole numbers: slot s counts units of unit[s] (a power of two);
+    // sum_fits of the group's largest entry fit in 32 bits (0: X is FP32)
+    int32_t sum_fits;
+    double unit[kMaxOccLayers];
 };
 
 // One layer as the occurrence-table build reads it (device array, one entry
@@ -291,7 +295,7 @@ struct LayerBuildArgs {
     float lim[kMaxLayerElts];
     float occ_ret, occ_lim;
     int32_t np;
-    int32_t pad_;
+    float fix_scale;           // units per unit of loss where the group's X holds whole numbers, else 0
 };
 
 // One occurrence group as the build reads it (device array).
@@ -416,11 +420,15 @@ cudaError_t build_sparse(art_portfolio* p, const float* src, cudaStream_t s);
 // call on this stream wrote with the same terms)
 cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                         bool build = true);
+// One occurrence group's trial pass over an X of whole numbers (lp slots per row).
+cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, int num_sms, bool early, double* ylt,
+                               uint8_t* branch, int* flags, cudaStream_t s);
 cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                           bool build = true);
 cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap, cudaStream_t s);
-// Write every occurrence group's X and bitmap (one launch) from the layer tables.
-cudaError_t build_occurrence(art_portfolio* p, cudaStream_t s);
+// Write every occurrence group's X and bitmap (one launch); whole: as whole
+// numbers in the groups whose losses allow it.
+cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s);
 cudaError_t launch_batched(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, bool fp64,
                            cudaStream_t s);
 cudaError_t launch_adjoint(art_portfolio* p, const YetArgs& y, const uint8_t* branch, const double* g,

@@ -1,0 +1,599 @@
+// ylt_fixed.cu -- the skip variant's trial pass over occurrence tables held
+// as whole numbers (Section II, Algorithm 1).
+//
+// An FP32 occurrence loss o = min(max(x - OccR, 0), OccL) > 0 needs x > OccR,
+// and an FP32 x >= OccR is a multiple of u = ulp(OccR), OccR too; so their
+// FP32 difference is a multiple of u, and o is one whenever OccL is. With o
+// bounded by OccL (or by the sum of the layer's ELT limits) every entry of X
+// is then a whole number of units below 2^32 for most real covers (OccL up to
+// 255 times OccR), stored as that number in the same 4 bytes. The trial pass
+// adds entries as 64-bit integers: the sum is exact, takes 1-2 integer
+// operations per entry instead of the seven of a compensated FP32 add, and
+// reduces across the warp in two 32-bit REDUX steps instead of five rounds of
+// compensated shuffles. It is rounded to FP64 once. On c1 (1,000,000 trials x
+// 1,000 events, one layer) the forward takes 0.90 ms against 1.27 with the
+// compensated pass, on a group of 8 of c4's layers 3.3 against 3.95 ms per
+// 1,000,000 trials, on c3 (8 layers, few events with a loss) 1.80 against 2.07. Groups with a layer that
+// does not fit (OccR = 0, very wide covers) keep the FP32 table and the
+// compensated pass of ylt_skip.cu.
+//
+// The rest of the mapping is that of ylt_skip.cu: persistent 1024-thread
+// CTAs, the bitmap folded into shared memory, a warp per trial streaming its
+// ids, the next chunk requested before the current one is processed. A trial
+// that starts off a 16-byte boundary is copied from the boundary before it,
+// and the ids of its neighbours are masked; a trial whose copies would leave
+// the id array (at its very start or end) is read id by id.
+//
+// What bounds it (ncu, c1): the L1 data path (72% of its wavefronts: 3.2-3.5
+// per 32 random bit tests, one per gathered row, one per 32 ids) and the bytes
+// in flight (32 KB per SM); issue is 56%.
+#include <algorithm>
+
+#include "art_internal.cuh"
+
+namespace art {
+
+namespace {
+
+constexpr int kFxThreads = 1024;
+constexpr int kFxWarps = kFxThreads / 32;
+constexpr int kFxIds = 8;     // ids per lane and chunk: 1 KB in flight per warp, 32 KB per SM
+constexpr int kFxQueue = 64;  // per-warp ring of queued ids (wide groups)
+constexpr unsigned kFull = 0xffffffffu;
+constexpr uint64_t kWaitNs = 4000000000ULL;  // longest wait for a copy
+
+__device__ __forceinline__ uint64_t now_ns() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ uint32_t ld_bits(const uint32_t* p) {
+    uint32_t v;
+    asm("ld.global.nc.L1::evict_last.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+
+// Row id of X: LP (1, 2, 4 or 8) whole numbers in one load, not kept in L1.
+template <int LP>
+__device__ __forceinline__ void ld_units(const float* x, uint32_t id, uint32_t (&o)[LP]) {
+    const float* p = x + (size_t)id * LP;
+    if constexpr (LP == 1) {
+        asm("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(o[0]) : "l"(p));
+    } else if constexpr (LP == 2) {
+        asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(o[0]), "=r"(o[1]) : "l"(p));
+    } else if constexpr (LP == 4) {
+        asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+            : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3])
+            : "l"(p));
+    } else {
+        asm("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]), "=r"(o[4]), "=r"(o[5]), "=r"(o[6]), "=r"(o[7])
+            : "l"(p));
+    }
+}
+
+// The ids of one trial as the warp reads them: n positions from a 16-byte
+// boundary, of which the first `head` belong to the trial before. VEC: every
+// trial starts and ends on a 16-byte boundary.
+template <bool VEC>
+struct Span {
+    const int32_t* p = nullptr;  // 16-byte aligned (position 0)
+    uint32_t n = 0, head_ = 0;
+    bool edge_ = false;          // a vector of it leaves the id array: read id by id
+    __device__ __forceinline__ uint32_t head() const { return VEC ? 0u : head_; }
+    __device__ __forceinline__ bool edge() const { return VEC ? false : edge_; }
+};
+
+// The trials of one warp, in its order: t, t + n_warps, ...
+template <bool VEC>
+struct Trials {
+    int64_t lo, hi, stride;  // reads of [lo, hi) stay in the id array (for a CSR every index between the
+                             // first and the last offset lies in some trial); VEC: ids from trial to trial
+    uint32_t mis;            // ids between the 16-byte boundary before y.ids and y.ids
+    bool bad = false;        // a decreasing pair of offsets was seen
+
+    __device__ __forceinline__ Trials(const YetArgs& y, int64_t n_warps) {
+        if constexpr (VEC) {
+            stride = n_warps * (int64_t)y.k;
+        } else {
+            lo = y.off ? y.off[0] : 0;
+            hi = y.off ? y.off[y.n_trials] : y.n_trials * (int64_t)y.k;
+            mis = (uint32_t)(reinterpret_cast<uintptr_t>(y.ids) >> 2) & 3u;
+        }
+    }
+    __device__ __forceinline__ Span<VEC> first(const YetArgs& y, int64_t t) {
+        Span<VEC> s;
+        if (t >= y.n_trials) return s;
+        if constexpr (VEC) {
+            s.p = y.ids + t * (int64_t)y.k;
+            s.n = (uint32_t)y.k;
+        } else {
+            int64_t b, e;
+            bool bo;
+            trial_range(y, t, b, e, bo);
+            bad |= bo;
+            s.head_ = ((uint32_t)b + mis) & 3u;
+            const int64_t a = b - s.head_;
+            s.p = y.ids + a;
+            s.n = e > b ? (uint32_t)(e - a) : 0u;
+            s.edge_ = a < lo || a + (int64_t)((s.n + 3u) & ~3u) > hi;
+        }
+        return s;
+    }
+    // the span of trial t, whose predecessor in the warp's order is s
+    __device__ __forceinline__ Span<VEC> next(const YetArgs& y, const Span<VEC>& s, int64_t t) {
+        if constexpr (VEC) {
+            Span<VEC> r;
+            r.p = s.p + stride;
+            r.n = t < y.n_trials ? s.n : 0u;
+            return r;
+        }
+        return first(y, t);
+    }
+};
+
+// A warp's id stream: chunks of 32 * E positions brought to its buffer in
+// shared memory by bulk copies (TMA), one in flight while the chunk before it
+// is processed from registers. Loads of the ids through L1 would share its
+// in-order return path with the gathers, which then wait for DRAM instead of
+// L2 (c1 forward 1.27 ms with 16-byte loads of the ids, XX with the copies).
+template <int E>
+struct IdStream {
+    uint32_t bar, buf;  // shared-memory addresses of the warp's barrier and buffer
+    uint32_t phase;
+    uint64_t policy;    // evict-first in L2: the stream must not push out X
+
+    __device__ __forceinline__ void init(void* bars, void* bufs, int wib, int lane) {
+        bar = (uint32_t)__cvta_generic_to_shared(bars) + 8u * wib;
+        buf = (uint32_t)__cvta_generic_to_shared(bufs) + 128u * E * wib;
+        phase = 0;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+        if (lane == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncwarp();
+    }
+    // Request the chunk from position c0, once every lane has the ids of the
+    // chunk before it.
+    template <bool VEC>
+    __device__ __forceinline__ void request(const Span<VEC>& s, uint32_t c0, int lane) {
+        if (lane == 0 && c0 < s.n && !s.edge()) {
+            const uint32_t bytes = 4u * min(32u * E, ((s.n + 3u) & ~3u) - c0);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(buf),
+                "l"(s.p + c0), "r"(bytes), "r"(bar), "l"(policy)
+                : "memory");
+        }
+    }
+    __device__ __forceinline__ bool arrived() const {
+        uint32_t ok;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(bar), "r"(phase)
+            : "memory");
+        return ok != 0;
+    }
+    // Wait for the requested chunk; false when it has not come in time.
+    __device__ __forceinline__ bool wait() {
+        bool ok = arrived();
+        if (!ok) {
+            const uint64_t t0 = now_ns();
+            while (!(ok = arrived()) && now_ns() - t0 < kWaitNs) {
+            }
+        }
+        phase ^= 1u;
+        return ok;
+    }
+    // The ids of the chunk from position c0 of a span with c0 < n: slot
+    // 4 h + i of a lane is position c0 + 128 h + 4 lane + i. What positions
+    // outside the trial hold is undefined (the caller masks them).
+    template <bool VEC>
+    __device__ __forceinline__ bool take(const Span<VEC>& s, uint32_t c0, int lane, uint32_t (&v)[E]) {
+        bool ok = true;
+        if (!s.edge()) {
+            ok = wait();
+#pragma unroll
+            for (int h = 0; h < E / 4; ++h)
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(v[4 * h]), "=r"(v[4 * h + 1]), "=r"(v[4 * h + 2]), "=r"(v[4 * h + 3])
+                             : "r"(buf + 512u * h + 16u * lane)
+                             : "memory");
+        } else {
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                const uint32_t d = c0 + 128u * (k >> 2) + 4u * lane + (k & 3);
+                v[k] = d >= s.head() && d < s.n ? (uint32_t)ld_stream(s.p + d) : 0u;
+            }
+        }
+        return ok;
+    }
+};
+
+// A chunk's ids as the tests below take them, at most C: positions outside
+// the trial and ids outside the catalogue become the sentinel C (its row of X
+// is zero). max_id keeps the largest id of the trial's own. The warp's vote
+// needs every id of the chunk in its register, so after it the buffer that
+// they came from may be written again (loads from shared memory only issued
+// may still read it).
+template <int E, bool VEC>
+__device__ __forceinline__ void clean_ids(const Span<VEC>& s, uint32_t c0, int lane, uint32_t C, uint32_t (&v)[E],
+                                          uint32_t& max_id) {
+    uint32_t m = 0;
+    if ((c0 != 0 || s.head() == 0) && c0 + 32u * E <= s.n) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) m = max(m, v[k]);
+    } else if constexpr (VEC) {  // the trial's end: whole vectors are in or out
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const bool live = c0 + 128u * (k >> 2) + 4u * lane < s.n;
+            m = max(m, live ? v[k] : 0u);
+            v[k] = live ? v[k] : C;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const uint32_t d = c0 + 128u * (k >> 2) + 4u * lane + (k & 3);
+            const bool live = d - s.head() < s.n - s.head();
+            m = max(m, live ? v[k] : 0u);
+            v[k] = live ? v[k] : C;
+        }
+    }
+    if (__any_sync(kFull, m >= C)) {  // some id lies outside the catalogue
+        max_id = max(max_id, m);
+#pragma unroll
+        for (int k = 0; k < E; ++k) v[k] = min(v[k], C);
+    }
+}
+
+// The event's bit: word w of shared memory holds bitmap words w and w + S
+// OR-ed together (FOLD: a superset test, a fold-only hit gathers zeros).
+template <bool FOLD>
+__device__ __forceinline__ bool bit_of(const uint32_t* s_bits, const uint32_t* gbits, uint32_t id, uint32_t S) {
+    uint32_t wi = id >> 5, w;
+    if constexpr (FOLD) {
+        wi = __viaddmin_u32(wi, 0u - S, wi);  // wi - S wraps when wi < S
+        w = s_bits[wi];
+    } else {
+        w = wi < S ? s_bits[wi] : ld_bits(gbits + wi);
+    }
+    return __funnelshift_r(w, 0u, id) & 1u;
+}
+
+template <bool FOLD>
+__device__ __forceinline__ void stage_bits(uint32_t* s_bits, const uint32_t* gbits, int32_t smem_words, int32_t words) {
+    const uint4* src = reinterpret_cast<const uint4*>(gbits);
+    uint4* dst = reinterpret_cast<uint4*>(s_bits);
+    for (int i = threadIdx.x; i < smem_words / 4; i += blockDim.x) {
+        uint4 v = src[i];
+        if (FOLD && 4 * i + smem_words < words) {  // the bitmap is zero-padded to whole uint4
+            const uint4 u = src[i + smem_words / 4];
+            v.x |= u.x;
+            v.y |= u.y;
+            v.z |= u.z;
+            v.w |= u.w;
+        }
+        dst[i] = v;
+    }
+}
+
+// The warp's total of a 64-bit count (valid in every lane). Entries are
+// below 2^32, so for trials shorter than 2^20 the lanes' counts stay below
+// 2^47: 20 low and 27 high bits, each summed in one 32-bit reduction.
+__device__ __forceinline__ unsigned long long warp_total(unsigned long long v, bool is_short) {
+    if (is_short) {
+        const uint32_t lo = __reduce_add_sync(kFull, (uint32_t)v & 0xfffffu);
+        const uint32_t hi = __reduce_add_sync(kFull, (uint32_t)(v >> 20));
+        return ((unsigned long long)hi << 20) + lo;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+
+// True when every layer of the group has reached its aggregate cap.
+template <int LP>
+__device__ __forceinline__ bool capped(const OccGroupArgs& g, const unsigned long long (&acc)[LP], bool is_short) {
+    bool all = true;
+#pragma unroll
+    for (int j = 0; j < LP; ++j) {
+        const double v = (double)warp_total(acc[j], is_short) * g.unit[j];
+        if (j < g.n_layers) all = all && (v - g.agg_ret[j] >= g.agg_lim[j]);
+    }
+    return all;
+}
+
+// Groups of 1-2 layers: every lane gathers X for its own events whose bit is
+// set, 8 loads in flight. PRE entries are summed in 32 bits before the 64-bit
+// add (the host picks 4 when four of the largest entry fit).
+template <int LP, bool VEC, bool FOLD, int PRE>
+__global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGroupArgs g, const YetArgs y,
+                                                                    const int32_t smem_words, const bool early_exit,
+                                                                    double* __restrict__ ylt,
+                                                                    uint8_t* __restrict__ branch,
+                                                                    int* __restrict__ flags) {
+    constexpr int E = kFxIds;
+    extern __shared__ __align__(128) uint32_t s_dyn[];
+    uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
+    uint32_t* s_bits = s_ids + kFxWarps * 32 * E;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    IdStream<E> ids;
+    ids.init(s_dyn, s_ids, wib, lane);
+    stage_bits<FOLD>(s_bits, g.occ_bits, smem_words, (y.catalogue >> 5) + 1);
+    __syncthreads();
+    // neighbouring CTAs take neighbouring trials, so that few trials still
+    // spread over every SM
+    const int64_t n_warps = (int64_t)gridDim.x * kFxWarps;
+    int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
+    uint32_t max_id = 0;
+    // results of up to 32 trials, lane s holding the s-th: the FP64 steps run
+    // once per 32 trials
+    unsigned long long res[LP];
+    int64_t rt = -1;
+    bool rcap = false;
+    int slot = 0;
+    auto flush = [&]() {
+        if (rt >= 0) {
+#pragma unroll
+            for (int j = 0; j < LP; ++j)
+                if (j < g.n_layers) {
+                    const double sum = (double)res[j] * g.unit[j];
+                    const size_t wi = (size_t)g.layer[j] * (size_t)y.n_trials + (size_t)rt;
+                    ylt[wi] = rcap ? g.agg_lim[j] : xl_f64(sum, g.agg_ret[j], g.agg_lim[j]);
+                    if (branch) branch[wi] = rcap ? (uint8_t)2 : agg_branch(sum, g.agg_ret[j], g.agg_lim[j]);
+                }
+        }
+        rt = -1;
+    };
+    Trials<VEC> trials(y, n_warps);
+    bool lost = false;  // a wait gave up
+    Span<VEC> cur = trials.first(y, t);
+    ids.request(cur, 0, lane);
+    while (t < y.n_trials && !lost) {
+        const int64_t tn = t + n_warps;
+        const Span<VEC> nxt = trials.next(y, cur, tn);
+        unsigned long long acc[LP];
+#pragma unroll
+        for (int j = 0; j < LP; ++j) acc[j] = 0;
+        const bool is_short = cur.n < (1u << 20);
+        bool cap = false;
+        if (cur.n == 0) ids.request(nxt, 0, lane);
+        for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
+            uint32_t id[E];
+            if (!ids.take(cur, c0, lane, id)) {
+                lost = true;
+                break;
+            }
+            clean_ids<E>(cur, c0, lane, C, id, max_id);
+            // request the next chunk (this trial's, or the next trial's first) now
+            const bool last = c0 + 32 * E >= cur.n;
+            if (last) ids.request(nxt, 0, lane);
+            else ids.request(cur, c0 + 32 * E, lane);
+            bool nz[E];
+#pragma unroll
+            for (int k = 0; k < E; ++k) nz[k] = bit_of<FOLD>(s_bits, g.occ_bits, id[k], S);
+            uint32_t o[E][LP];
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+#pragma unroll
+                for (int j = 0; j < LP; ++j) o[k][j] = 0;
+                if (nz[k]) ld_units<LP>(g.occ, id[k], o[k]);
+            }
+#pragma unroll
+            for (int j = 0; j < LP; ++j)
+#pragma unroll
+                for (int k = 0; k < E; k += PRE) {
+                    uint32_t p = o[k][j];
+#pragma unroll
+                    for (int i = 1; i < PRE; ++i) p += o[k + i][j];
+                    acc[j] += p;
+                }
+            if (early_exit && capped<LP>(g, acc, is_short)) {
+                if (!last) {  // the trial's next chunk is on its way: let it come
+                    lost = !cur.edge() && !ids.wait();
+                    if (!lost) ids.request(nxt, 0, lane);
+                }
+                cap = true;
+                break;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < LP; ++j) {
+            const unsigned long long v = warp_total(acc[j], is_short);
+            if (lane == slot) res[j] = v;
+        }
+        if (lane == slot) {
+            rt = t;
+            rcap = cap;
+        }
+        if (++slot == 32) {
+            flush();
+            slot = 0;
+        }
+        t = tn;
+        cur = nxt;
+    }
+    flush();
+    if (lost) {
+        ids.phase ^= 1u;
+        ids.wait();  // the copy in flight may still come: shared memory stays until then
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
+    }
+    if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
+    if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
+}
+
+// Groups of 3-8 layers: the ids whose bit is set go to a per-warp ring in
+// shared memory; each time 32 are queued every lane takes one row. A lane
+// adds the row of the flush before, then requests this flush's, so a gather's
+// latency runs beside the next chunk's tests.
+template <int LP, bool VEC, bool FOLD>
+__global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_constant__ OccGroupArgs g, const YetArgs y,
+                                                                  const int32_t smem_words, const bool early_exit,
+                                                                  double* __restrict__ ylt,
+                                                                  uint8_t* __restrict__ branch,
+                                                                  int* __restrict__ flags) {
+    constexpr int E = kFxIds;
+    extern __shared__ __align__(128) uint32_t s_dyn[];
+    uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
+    uint32_t* s_queue = s_ids + kFxWarps * 32 * E;
+    uint32_t* s_bits = s_queue + kFxWarps * kFxQueue;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    IdStream<E> ids;
+    ids.init(s_dyn, s_ids, wib, lane);
+    stage_bits<FOLD>(s_bits, g.occ_bits, smem_words, (y.catalogue >> 5) + 1);
+    __syncthreads();
+    uint32_t* q = s_queue + wib * kFxQueue;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int64_t n_warps = (int64_t)gridDim.x * kFxWarps;
+    int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
+    uint32_t max_id = 0;
+    Trials<VEC> trials(y, n_warps);
+    bool lost = false;  // a wait gave up
+    Span<VEC> cur = trials.first(y, t);
+    ids.request(cur, 0, lane);
+    while (t < y.n_trials && !lost) {
+        const int64_t tn = t + n_warps;
+        const Span<VEC> nxt = trials.next(y, cur, tn);
+        unsigned long long acc[LP];
+        uint32_t o[LP];
+#pragma unroll
+        for (int j = 0; j < LP; ++j) {
+            acc[j] = 0;
+            o[j] = 0;
+        }
+        const bool is_short = cur.n < (1u << 20);
+        bool cap = false;
+        uint32_t head = 0, tail = 0;  // warp-uniform ring positions, tail - head < 32 between slots
+        if (cur.n == 0) ids.request(nxt, 0, lane);
+        for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
+            uint32_t id[E];
+            if (!ids.take(cur, c0, lane, id)) {
+                lost = true;
+                break;
+            }
+            clean_ids<E>(cur, c0, lane, C, id, max_id);
+            const bool last = c0 + 32 * E >= cur.n;
+            if (last) ids.request(nxt, 0, lane);
+            else ids.request(cur, c0 + 32 * E, lane);
+            bool nz[E];
+#pragma unroll
+            for (int k = 0; k < E; ++k) nz[k] = bit_of<FOLD>(s_bits, g.occ_bits, id[k], S);
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                const unsigned m = __ballot_sync(kFull, nz[k]);
+                if (nz[k]) q[(tail + __popc(m & lt_mask)) & (kFxQueue - 1)] = id[k];
+                tail += __popc(m);
+                if (tail - head >= 32) {
+                    __syncwarp();
+                    const uint32_t mine = q[(head + lane) & (kFxQueue - 1)];
+                    head += 32;
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < LP; ++j) acc[j] += o[j];
+                    ld_units<LP>(g.occ, mine, o);
+                }
+            }
+            if (early_exit) {
+#pragma unroll
+                for (int j = 0; j < LP; ++j) {
+                    acc[j] += o[j];
+                    o[j] = 0;
+                }
+                if (capped<LP>(g, acc, is_short)) {
+                    if (!last) {
+                        lost = !cur.edge() && !ids.wait();
+                        if (!lost) ids.request(nxt, 0, lane);
+                    }
+                    head = tail;
+                    cap = true;
+                    break;
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < LP; ++j) acc[j] += o[j];
+        if (head + lane < tail) {
+            ld_units<LP>(g.occ, q[(head + lane) & (kFxQueue - 1)], o);
+#pragma unroll
+            for (int j = 0; j < LP; ++j) acc[j] += o[j];
+        }
+        __syncwarp();
+        unsigned long long mine = 0;
+#pragma unroll
+        for (int j = 0; j < LP; ++j) {
+            const unsigned long long v = warp_total(acc[j], is_short);
+            if (lane == j) mine = v;
+        }
+        if (lane < g.n_layers) {
+            const double sum = (double)mine * g.unit[lane], ret = g.agg_ret[lane], lim = g.agg_lim[lane];
+            const size_t wi = (size_t)g.layer[lane] * (size_t)y.n_trials + (size_t)t;
+            ylt[wi] = cap ? lim : xl_f64(sum, ret, lim);
+            if (branch) branch[wi] = cap ? (uint8_t)2 : agg_branch(sum, ret, lim);
+        }
+        t = tn;
+        cur = nxt;
+    }
+    if (lost) {
+        ids.phase ^= 1u;
+        ids.wait();  // the copy in flight may still come: shared memory stays until then
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
+    }
+    if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
+    if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
+}
+
+typedef void (*FixedKernel)(const OccGroupArgs, const YetArgs, const int32_t, const bool, double*, uint8_t*, int*);
+
+template <bool VEC, bool FOLD>
+FixedKernel pick_kernel(int lp, bool pre4) {
+    switch (lp) {
+        case 1: return pre4 ? fixed_narrow_kernel<1, VEC, FOLD, 4> : fixed_narrow_kernel<1, VEC, FOLD, 1>;
+        case 2: return pre4 ? fixed_narrow_kernel<2, VEC, FOLD, 4> : fixed_narrow_kernel<2, VEC, FOLD, 1>;
+        case 4: return fixed_wide_kernel<4, VEC, FOLD>;
+        case 8: return fixed_wide_kernel<8, VEC, FOLD>;
+        default: return nullptr;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, int num_sms, bool early, double* ylt,
+                               uint8_t* branch, int* flags, cudaStream_t s) {
+    int dev = 0, max_optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+    // the warps' barriers (256 bytes), id buffers and queues, then the bitmap
+    const int fixed_bytes = 256 + kFxWarps * (32 * kFxIds + (lp >= 4 ? kFxQueue : 0)) * 4;
+    // Loads of up to 16 bytes hold an L1 line each while they are in flight:
+    // with all 227 KB taken as shared memory the 28 KB of L1 left carry 0.5-0.6
+    // of them per cycle and SM, with 195 KB (60 KB of L1) 0.8-1.0 (probed; 32-byte
+    // loads reach 0.95 with either). So the narrow rows leave that L1 free and
+    // fold more of the bitmap (c1 1.009 -> 0.898 ms; the 32-byte rows of c4
+    // 1.71 ms with 195 KB, 1.65 with all).
+    if (lp <= 4) max_optin = std::min(max_optin, 195 * 1024);
+    const int words = (y.catalogue >> 5) + 1;  // bits 0 .. C (C: the sentinel)
+    // whole 16-byte groups of words that fit next to the queues
+    const int smem_words = std::max(4, std::min((words + 3) & ~3, (max_optin - fixed_bytes) / 4) & ~3);
+    const int smem = fixed_bytes + smem_words * 4;
+    const bool fold = words <= 2 * smem_words;  // it folds once when at most twice as long
+    // every trial starts and ends on a 16-byte boundary
+    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
+    const bool pre4 = g.sum_fits >= 4;
+    const FixedKernel kern = vec ? (fold ? pick_kernel<true, true>(lp, pre4) : pick_kernel<true, false>(lp, pre4))
+                                 : (fold ? pick_kernel<false, true>(lp, pre4) : pick_kernel<false, false>(lp, pre4));
+    if (!kern) return cudaErrorInvalidValue;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(num_sms, y.n_trials));
+    kern<<<(unsigned)grid, kFxThreads, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
+    return cudaGetLastError();
+}
+
+}  // namespace art

@@ -428,6 +428,13 @@ __global__ void __launch_bounds__(kSkipThreads, 1) ylt_skip_kernel(const OccGrou
     if (lane == 0 && bad_off_seen) atomicOr(flags + kFlagBadOffsets, 1);
 }
 
+// An occurrence loss as X holds it: the FP32 value, or (scale > 0) the bits
+// of the whole number o * scale, exactly (scale is a power of two and the
+// product a whole number below 2^32; see ylt_fixed.cu).
+__device__ __forceinline__ float table_entry(float o, float scale) {
+    return scale > 0.0f ? __uint_as_float(__float2uint_rz(o * scale)) : o;
+}
+
 // Occurrence-loss tables (steps 2-3 once per catalogue event): block
 // (x, y) covers 256 events of occurrence group y; thread i sums F_e over row
 // i of each of the group's layer tables in the layer's ELT order (padding
@@ -437,7 +444,7 @@ __global__ void __launch_bounds__(kSkipThreads, 1) ylt_skip_kernel(const OccGrou
 template <int LP>
 __global__ void __launch_bounds__(256) build_occ_kernel(const LayerBuildArgs* __restrict__ lbuild,
                                                         const OccBuildGroup* __restrict__ groups, int32_t catalogue,
-                                                        int32_t words) {
+                                                        int32_t words, const bool whole) {
     __shared__ LayerBuildArgs s_lb[LP];
     const OccBuildGroup& grp = groups[blockIdx.y];
     const int nl = grp.n_layers;
@@ -475,6 +482,7 @@ __global__ void __launch_bounds__(256) build_occ_kernel(const LayerBuildArgs* __
                 }
                 o[s] = xl_f32(x, a.occ_ret, a.occ_lim);
                 nz |= o[s] > 0.0f;
+                o[s] = table_entry(o[s], whole ? a.fix_scale : 0.0f);
             }
         }
         float* dst = grp.occ + i * LP;
@@ -507,7 +515,7 @@ __global__ void __launch_bounds__(256) build_occ_csr_kernel(const uint32_t* __re
                                                             const float* __restrict__ occ_terms,
                                                             const LayerBuildArgs* __restrict__ lbuild,
                                                             const OccBuildGroup* __restrict__ groups, int32_t catalogue,
-                                                            int32_t words) {
+                                                            int32_t words, const bool whole) {
     const OccBuildGroup& grp = groups[blockIdx.y];
     const uint8_t* sm = slotmask + (size_t)blockIdx.y * np;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -549,6 +557,7 @@ __global__ void __launch_bounds__(256) build_occ_csr_kernel(const uint32_t* __re
                 }
                 o[s] = xl_f32(x[s], occ_terms[2 * j], occ_terms[2 * j + 1]);
                 nz |= o[s] > 0.0f;
+                o[s] = table_entry(o[s], whole ? lbuild[j].fix_scale : 0.0f);
             }
         }
         float* dst = grp.occ + i * LP;
@@ -609,7 +618,7 @@ cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np
     return cudaGetLastError();
 }
 
-cudaError_t build_occurrence(art_portfolio* p, cudaStream_t s) {
+cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s) {
     const int32_t words = (int32_t)(((int64_t)p->catalogue + 31) / 32);
     const dim3 grid((unsigned)(((int64_t)words * 32 + 255) / 256), (unsigned)p->ogroups.size());
     // from the CSR of the non-zero losses where the portfolio holds it (see
@@ -617,29 +626,45 @@ cudaError_t build_occurrence(art_portfolio* p, cudaStream_t s) {
     if (p->d_slotmask && p->sp_ptr && p->d_elt_terms && p->d_occ && p->d_lbuild) {
         const SparseEntry* en = reinterpret_cast<const SparseEntry*>(p->sp_entries);
         switch (p->og_lp) {
-            case 1: build_occ_csr_kernel<1><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-            case 2: build_occ_csr_kernel<2><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-            case 4: build_occ_csr_kernel<4><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-            case 8: build_occ_csr_kernel<8><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
+            case 1: build_occ_csr_kernel<1><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+            case 2: build_occ_csr_kernel<2><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+            case 4: build_occ_csr_kernel<4><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+            case 8: build_occ_csr_kernel<8><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
             default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
     }
     switch (p->og_lp) {
-        case 1: build_occ_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-        case 2: build_occ_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-        case 4: build_occ_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
-        case 8: build_occ_kernel<8><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words); break;
+        case 1: build_occ_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+        case 2: build_occ_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+        case 4: build_occ_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+        case 8: build_occ_kernel<8><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
+// Whether a YET's ids lie in a device's own memory (NULL: no ids, a build
+// ahead of staged chunks, which are on the device).
+static bool ids_on_device(const int32_t* ids) {
+    if (!ids) return true;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, ids) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
 cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                         bool build) {
     const bool early = (p->flags & ART_FLAG_EARLY_EXIT) != 0;
+    // tables of whole numbers where the ids lie in device memory (the pass
+    // over them brings the ids by bulk copies); ids read in place from host
+    // memory keep the FP32 tables and the loads of the pass below
+    const bool whole = ids_on_device(y.ids);
     // steps 2-3 once per catalogue event, with the terms as they are now
-    cudaError_t err = build ? build_occurrence(p, s) : cudaSuccess;
+    cudaError_t err = build ? build_occurrence(p, whole, s) : cudaSuccess;
     if (err != cudaSuccess || y.n_trials == 0) return err;
     // ART_FLAG_L2_PERSIST: a persisting window over the table each group
     // pass gathers from, so that the id stream does not evict it
@@ -647,6 +672,10 @@ cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t
     const size_t table_bytes = sizeof(float) * ((size_t)p->catalogue + 1) * (size_t)p->og_lp;
     for (const OccGroupArgs& g : p->ogroups) {
         if (window && (err = set_window(s, g.occ, table_bytes))) return err;
+        if (whole && g.sum_fits) {  // X holds whole numbers
+            if ((err = launch_fixed_group(g, y, p->og_lp, p->num_sms, early, ylt, branch, p->d_flags, s))) return err;
+            continue;
+        }
         switch (p->og_lp) {
             case 1: err = launch_group<1, 1>(g, y, p->num_sms, p->catalogue, early, ylt, branch, p->d_flags, s); break;
             case 2: err = launch_group<2, 2>(g, y, p->num_sms, p->catalogue, early, ylt, branch, p->d_flags, s); break;
