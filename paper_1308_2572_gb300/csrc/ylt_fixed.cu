@@ -213,15 +213,15 @@ struct IdStream {
     }
 };
 
-// A chunk's ids as the tests below take them, at most C: positions outside
-// the trial and ids outside the catalogue become the sentinel C (its row of X
-// is zero). max_id keeps the largest id of the trial's own. The warp's vote
+// A chunk's ids as the tests below take them: positions outside the trial and
+// ids outside the catalogue become `none`, an id whose bit is clear. max_id
+// keeps the largest id of the trial's own. The warp's vote
 // needs every id of the chunk in its register, so after it the buffer that
 // they came from may be written again (loads from shared memory only issued
 // may still read it).
 template <int E, bool VEC>
-__device__ __forceinline__ void clean_ids(const Span<VEC>& s, uint32_t c0, int lane, uint32_t C, uint32_t (&v)[E],
-                                          uint32_t& max_id) {
+__device__ __forceinline__ void clean_ids(const Span<VEC>& s, uint32_t c0, int lane, uint32_t C, uint32_t none,
+                                          uint32_t (&v)[E], uint32_t& max_id) {
     uint32_t m = 0;
     if ((c0 != 0 || s.head() == 0) && c0 + 32u * E <= s.n) {
 #pragma unroll
@@ -231,7 +231,7 @@ __device__ __forceinline__ void clean_ids(const Span<VEC>& s, uint32_t c0, int l
         for (int k = 0; k < E; ++k) {
             const bool live = c0 + 128u * (k >> 2) + 4u * lane < s.n;
             m = max(m, live ? v[k] : 0u);
-            v[k] = live ? v[k] : C;
+            v[k] = live ? v[k] : none;
         }
     } else {
 #pragma unroll
@@ -239,14 +239,24 @@ __device__ __forceinline__ void clean_ids(const Span<VEC>& s, uint32_t c0, int l
             const uint32_t d = c0 + 128u * (k >> 2) + 4u * lane + (k & 3);
             const bool live = d - s.head() < s.n - s.head();
             m = max(m, live ? v[k] : 0u);
-            v[k] = live ? v[k] : C;
+            v[k] = live ? v[k] : none;
         }
     }
     if (__any_sync(kFull, m >= C)) {  // some id lies outside the catalogue
         max_id = max(max_id, m);
 #pragma unroll
-        for (int k = 0; k < E; ++k) v[k] = min(v[k], C);
+        for (int k = 0; k < E; ++k) v[k] = v[k] < C ? v[k] : none;
     }
+}
+
+// The id that stands for no event. Folded, the sentinel C shares its bit with
+// an event's; if that one is set, the empty slots of every trial's last chunk
+// gather row C, and one hot row slows the whole chip's gathers (c1 with 24
+// empty slots per trial: 1.26 against 0.90 ms). So it is an id whose word,
+// 2 S - S, is the always-zero word after the bitmap.
+template <bool FOLD>
+__device__ __forceinline__ uint32_t no_event(uint32_t C, uint32_t S) {
+    return FOLD ? 64u * S : C;
 }
 
 // The event's bit: word w of shared memory holds bitmap words w and w + S
@@ -278,6 +288,7 @@ __device__ __forceinline__ void stage_bits(uint32_t* s_bits, const uint32_t* gbi
         }
         dst[i] = v;
     }
+    if (threadIdx.x == 0) s_bits[smem_words] = 0u;  // no_event's word
 }
 
 // The warp's total of a 64-bit count (valid in every lane). Entries are
@@ -319,7 +330,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGr
     extern __shared__ __align__(128) uint32_t s_dyn[];
     uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
     uint32_t* s_bits = s_ids + kFxWarps * 32 * E;
-    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     IdStream<E> ids;
     ids.init(s_dyn, s_ids, wib, lane);
@@ -368,7 +379,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGr
                 lost = true;
                 break;
             }
-            clean_ids<E>(cur, c0, lane, C, id, max_id);
+            clean_ids<E>(cur, c0, lane, C, none, id, max_id);
             // request the next chunk (this trial's, or the next trial's first) now
             const bool last = c0 + 32 * E >= cur.n;
             if (last) ids.request(nxt, 0, lane);
@@ -442,7 +453,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
     uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
     uint32_t* s_queue = s_ids + kFxWarps * 32 * E;
     uint32_t* s_bits = s_queue + kFxWarps * kFxQueue;
-    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     IdStream<E> ids;
     ids.init(s_dyn, s_ids, wib, lane);
@@ -477,7 +488,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
                 lost = true;
                 break;
             }
-            clean_ids<E>(cur, c0, lane, C, id, max_id);
+            clean_ids<E>(cur, c0, lane, C, none, id, max_id);
             const bool last = c0 + 32 * E >= cur.n;
             if (last) ids.request(nxt, 0, lane);
             else ids.request(cur, c0 + 32 * E, lane);
@@ -571,7 +582,8 @@ cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, 
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
     // the warps' barriers (256 bytes), id buffers and queues, then the bitmap
-    const int fixed_bytes = 256 + kFxWarps * (32 * kFxIds + (lp >= 4 ? kFxQueue : 0)) * 4;
+    // and its zero word
+    const int fixed_bytes = 256 + 16 + kFxWarps * (32 * kFxIds + (lp >= 4 ? kFxQueue : 0)) * 4;
     // Loads of up to 16 bytes hold an L1 line each while they are in flight:
     // with all 227 KB taken as shared memory the 28 KB of L1 left carry 0.5-0.6
     // of them per cycle and SM, with 195 KB (60 KB of L1) 0.8-1.0 (probed; 32-byte
