@@ -192,7 +192,7 @@ cudaError_t launch_adjoint(art_portfolio* p, const YetArgs& y, const uint8_t* br
     const size_t lg_bytes = sizeof(double) * (size_t)p->n_layers * (4 + kMaxLayerElts);
     const size_t part_bytes = sizeof(double) * (size_t)nblk * (4 + kMaxLayerElts);
     char* w = nullptr;
-    cudaError_t err = cudaMallocAsync((void**)&w, lg_bytes + part_bytes + 256, s);
+    cudaError_t err = scratch_alloc((void**)&w, lg_bytes + part_bytes + 256, s);
     if (err) return err;
     double* layer_grad = (double*)w;
     double* partial = (double*)(w + ((lg_bytes + 255) & ~(size_t)255));

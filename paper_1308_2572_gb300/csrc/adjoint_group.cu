@@ -480,7 +480,7 @@ cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& y, const uint
     const size_t part_bytes = sizeof(double) * (size_t)p->num_sms * (4 * kMaxGroupLayers + kMaxLayerElts);
     const size_t a1 = (mask_bytes + 255) & ~(size_t)255, a2 = (bit_bytes + 255) & ~(size_t)255;
     char* w = nullptr;
-    cudaError_t err = cudaMallocAsync((void**)&w, a1 + a2 + part_bytes, s);
+    cudaError_t err = scratch_alloc((void**)&w, a1 + a2 + part_bytes, s);
     if (err) return err;
     Scratch sc{reinterpret_cast<uint2*>(w), reinterpret_cast<uint32_t*>(w + a1), reinterpret_cast<double*>(w + a1 + a2)};
     do {

@@ -144,6 +144,25 @@ cudaError_t upload_batched_terms(art_portfolio* p) {
 
 }  // namespace
 
+// Whether a layer's FP32 occurrence losses are whole numbers below 2^32 of
+// some unit 2^e (see ylt_fixed.cu): multiples of ulp(OccR) (and of ulp(OccL),
+// the finer of the two), at most min(OccL, the sum of the ELT limits).
+bool art::whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units) {
+    if (!(occ_ret >= 0x1p-60f) || !(occ_ret <= 0x1p100f)) return false;
+    int er, el;
+    std::frexp(occ_ret, &er);  // occ_ret in [2^(er - 1), 2^er): its ulp is 2^(er - 24)
+    *e = er - 24;
+    double bound = elt_lim_sum * 1.0001;  // the FP32 sum may round up
+    if (std::isfinite(occ_lim)) {
+        if (!(occ_lim >= 0x1p-60f)) return false;
+        std::frexp(occ_lim, &el);
+        *e = std::min(*e, el - 24);
+        bound = std::min(bound, (double)occ_lim);
+    }
+    *max_units = std::ldexp(bound, -*e);
+    return *max_units <= 4294967295.0;
+}
+
 // Layer tile of the persistent kernels: layer j sits at (tile, slot, lane)
 // with 32 * slots layers per tile; memb holds, per (tile, ELT, lane), the
 // bits of the lane's slots whose layer covers the ELT.
@@ -296,25 +315,6 @@ void refresh_group_terms(art_portfolio* p) {
             g.layer[s] = real ? j : 0;
         }
     }
-}
-
-// Whether a layer's FP32 occurrence losses are whole numbers below 2^32 of
-// some unit 2^e (see ylt_fixed.cu): multiples of ulp(OccR) (and of ulp(OccL),
-// the finer of the two), at most min(OccL, the sum of the ELT limits).
-bool whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units) {
-    if (!(occ_ret >= 0x1p-60f) || !(occ_ret <= 0x1p100f)) return false;
-    int er, el;
-    std::frexp(occ_ret, &er);  // occ_ret in [2^(er - 1), 2^er): its ulp is 2^(er - 24)
-    *e = er - 24;
-    double bound = elt_lim_sum * 1.0001;  // the FP32 sum may round up
-    if (std::isfinite(occ_lim)) {
-        if (!(occ_lim >= 0x1p-60f)) return false;
-        std::frexp(occ_lim, &el);
-        *e = std::min(*e, el - 24);
-        bound = std::min(bound, (double)occ_lim);
-    }
-    *max_units = std::ldexp(bound, -*e);
-    return *max_units <= 4294967295.0;
 }
 
 // Terms of every layer as the occurrence-table build reads them, and the
@@ -580,6 +580,7 @@ void free_portfolio(art_portfolio* p) {
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
     delete p;
+    scratch_user(-1);
 }
 
 int resolve_variant(const art_portfolio* p) {
@@ -690,6 +691,7 @@ art_status art_create_portfolio(int32_t catalogue_size, int32_t n_elt, const flo
         delete p;
         return ART_EINVAL;
     }
+    scratch_user(+1);
 
     cudaError_t e;
     art_status st = ART_OK;

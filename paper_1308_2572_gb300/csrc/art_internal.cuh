@@ -420,6 +420,10 @@ cudaError_t build_sparse(art_portfolio* p, const float* src, cudaStream_t s);
 // call on this stream wrote with the same terms)
 cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                         bool build = true);
+// Whether a layer's FP32 occurrence losses are whole numbers below 2^32 of a
+// unit 2^e; the largest they can be, in units.
+bool whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units);
+bool ids_on_device(const int32_t* ids);
 // One occurrence group's trial pass over an X of whole numbers (lp slots per row).
 cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, int num_sms, bool early, double* ylt,
                                uint8_t* branch, int* flags, cudaStream_t s);
@@ -462,6 +466,15 @@ cudaError_t set_layer_tile(art_portfolio* p, int32_t slots);
 int64_t tail_count(double p, int64_t n);
 
 void set_last_error(cudaError_t e);
+
+// Stream-ordered scratch of one call (release it with cudaFreeAsync), from a
+// pool that keeps a bounded amount between calls (scratch.cu).
+cudaError_t scratch_alloc(void** out, size_t bytes, cudaStream_t s);
+// A portfolio was made (+1) or destroyed (-1): the last one's end trims the
+// current device's pool.
+void scratch_user(int delta);
+// Id of the current device's context; 0 if the driver cannot tell.
+unsigned long long current_context_id();
 
 // Set (bytes > 0) or clear (bytes == 0) a persisting L2 access-policy window
 // over a hot table on a stream.

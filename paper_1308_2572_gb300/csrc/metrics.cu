@@ -901,7 +901,7 @@ cudaError_t metrics_run_k(const double* ylt, int64_t n, int32_t n_layers, const 
     const MetricsLayout m = metrics_layout(n_layers, n_p, nblk, slots);
     char* w = static_cast<char*>(scratch);
     const bool own = !w || scratch_bytes < m.total;
-    cudaError_t err = own ? cudaMallocAsync((void**)&w, m.total, s) : cudaSuccess;
+    cudaError_t err = own ? scratch_alloc((void**)&w, m.total, s) : cudaSuccess;
     if (err != cudaSuccess) return err;
     KParams kq = {};
     for (int q = 0; q < n_p; ++q) kq.k[q] = std::min<int64_t>(n, std::max<int64_t>(1, k[q]));
@@ -929,7 +929,7 @@ cudaError_t metrics_backward_run(const double* ylt, int64_t n, int32_t n_layers,
     const size_t o_we = align256(o_wg + sizeof(double) * n_prob);
     const size_t total = align256(o_we + sizeof(double) * n_prob);
     char* w = nullptr;
-    cudaError_t err = cudaMallocAsync((void**)&w, total, s);
+    cudaError_t err = scratch_alloc((void**)&w, total, s);
     if (err != cudaSuccess) return err;
     KParams kq = {};
     for (int q = 0; q < n_p; ++q) kq.k[q] = tail_count(probs[q], n);
@@ -980,33 +980,6 @@ struct NoAllocAddr {
     unsigned long long ctx_id = 0;  // the context the address belongs to
 };
 NoAllocAddr g_noalloc[kNoAllocMaxDevices];
-
-// Id of the current device's context (unique over the process's life, so a
-// context recreated after cudaDeviceReset gets a new one); 0 if the driver
-// cannot tell. Taken from the driver through the runtime's entry-point
-// lookup, without linking the driver library.
-unsigned long long current_context_id() {
-    typedef int (*GetCurrent)(void**);
-    typedef int (*GetId)(void*, unsigned long long*);
-    static GetCurrent get_current = nullptr;
-    static GetId get_id = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_current = reinterpret_cast<GetCurrent>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            get_id = reinterpret_cast<GetId>(f);
-    });
-    void* ctx = nullptr;
-    unsigned long long id = 0;
-    if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
-    return id;
-}
 
 // Device address of the scratch array on the current device: looked up with
 // the device current on the first call, and again whenever the device's

@@ -133,7 +133,7 @@ extern "C" art_status art_topk(const double* ylt_dev, int64_t n_trials, int32_t 
     double* thr = nullptr;
     unsigned long long* cnt = nullptr;
     const size_t thr_bytes = (sizeof(double) * (size_t)n_layers + 255) & ~(size_t)255;
-    if ((e = cudaMallocAsync((void**)&thr, thr_bytes + sizeof(unsigned long long) * (size_t)n_layers * nblk, stream))) {
+    if ((e = scratch_alloc((void**)&thr, thr_bytes + sizeof(unsigned long long) * (size_t)n_layers * nblk, stream))) {
         set_last_error(e);
         return ART_ECUDA;
     }

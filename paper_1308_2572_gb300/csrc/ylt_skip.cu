@@ -646,7 +646,7 @@ cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s) {
 
 // Whether a YET's ids lie in a device's own memory (NULL: no ids, a build
 // ahead of staged chunks, which are on the device).
-static bool ids_on_device(const int32_t* ids) {
+bool ids_on_device(const int32_t* ids) {
     if (!ids) return true;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, ids) != cudaSuccess) {
