@@ -12,11 +12,26 @@
 // the warp scans o_d in FP64 (an inclusive shuffle scan) on top of the carry
 // from the previous step, applies the aggregate terms to each C_d in FP64 and
 // takes the difference with the previous event's value (the previous lane's,
-// or the carried one). This path runs FP64 per event: it is a reporting path,
-// not the throughput path.
+// or the carried one). It evaluates the layer per occurrence in FP64 and
+// serves short YETs and layers whose losses are not whole numbers.
+//
+// Otherwise (payouts_fixed_kernel) the layer's occurrence losses are evaluated
+// once per catalogue event into a table of whole numbers (see ylt_fixed.cu)
+// with its bitmap, and the pass streams the ids as the skip variant's does.
+// C_d is then an exact 64-bit integer: a lane adds its four consecutive events,
+// the warp scans the lanes' totals, and the branch of A(C_d) is a comparison
+// of integers (the host finds, once per call, the smallest C whose FP64 value
+// passes the retention and the smallest that reaches the limit). Between the
+// two the payout is the event's own occurrence loss, exactly; below and above
+// it is 0; only the events that cross one of them take FP64 arithmetic, at
+// most two per trial. What bounds it: HBM (4 bytes of ids read, 8 of payouts
+// written per event); 100,000 trials x 1,000 events of a 16-ELT layer take
+// 0.35 ms against 2.40 with a warp scan in FP64 over 64-byte rows.
+#include <algorithm>
+#include <cmath>
 #include <limits>
 
-#include "art_internal.cuh"
+#include "id_stream.cuh"
 
 namespace art {
 namespace {
@@ -90,6 +105,250 @@ cudaError_t launch(const LayerArgs& la, const YetArgs& y, double* payouts, int32
     return cudaGetLastError();
 }
 
+constexpr int kPayThreads = 1024;
+constexpr int kPayWarps = kPayThreads / 32;
+constexpr int kPayIds = 8;  // ids per lane and chunk
+
+// One layer as the whole-number pass reads it.
+struct PayArgs {
+    const uint32_t* x;        // [C] occurrence losses in units
+    const uint32_t* bits;     // bit i set when x[i] > 0, zero-padded to whole 16-byte groups
+    double unit, agg_ret, agg_lim;
+    float unit_f;
+    unsigned long long pass;  // smallest C with XL(C) > 0
+    unsigned long long full;  // smallest C with C - AggR >= AggL (all ones: none)
+};
+
+// The layer's table: thread i evaluates event i (steps 2-3, FP32, the layer's
+// ELT order) as the forward does.
+template <int NP>
+__global__ void __launch_bounds__(256) payouts_table_kernel(const LayerArgs la, int32_t catalogue, float scale,
+                                                            int32_t words, uint32_t* __restrict__ x,
+                                                            uint32_t* __restrict__ bits) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t u = 0;
+    if (i < catalogue) {
+        const float4* row = reinterpret_cast<const float4*>(la.table) + i * (NP / 4);
+        float s = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NP / 4; ++q) {
+            const float4 r = __ldcs(row + q);
+            s += fin_f32(r.x, la.m[4 * q + 0], la.d[4 * q + 0], la.lim[4 * q + 0]);
+            s += fin_f32(r.y, la.m[4 * q + 1], la.d[4 * q + 1], la.lim[4 * q + 1]);
+            s += fin_f32(r.z, la.m[4 * q + 2], la.d[4 * q + 2], la.lim[4 * q + 2]);
+            s += fin_f32(r.w, la.m[4 * q + 3], la.d[4 * q + 3], la.lim[4 * q + 3]);
+        }
+        u = __float2uint_rz(xl_f32(s, la.occ_ret, la.occ_lim) * scale);
+        x[i] = u;
+    }
+    const unsigned m = __ballot_sync(kFull, u != 0);
+    if ((threadIdx.x & 31) == 0 && (i >> 5) < words) bits[i >> 5] = m;  // the padding too
+}
+
+__device__ __forceinline__ double agg_of(const PayArgs& a, unsigned long long c) {
+    return xl_f64((double)c * a.unit, a.agg_ret, a.agg_lim);
+}
+
+// u units as FP64, exactly: an FP32 value (the units hold at most 24
+// significant bits) widened by its bit pattern, without the FP64 pipe.
+__device__ __forceinline__ double units_f64(uint32_t u, float unit) {
+    const uint32_t f = __float_as_uint((float)u * unit);
+    return u ? __hiloint2double((int)((f >> 3) + 0x38000000u), (int)(f << 29)) : 0.0;
+}
+
+__device__ __forceinline__ void st_payouts4(double* p, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+                 : "memory");
+}
+
+// pay_vec: the payouts of a 16-byte group of ids start on a 32-byte boundary.
+template <bool VEC, bool FOLD>
+__global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const PayArgs a, const YetArgs y,
+                                                                      const int32_t smem_words, const bool pay_vec,
+                                                                      double* __restrict__ payouts,
+                                                                      int32_t* __restrict__ exhaust,
+                                                                      double* __restrict__ ylt,
+                                                                      int* __restrict__ flags) {
+    constexpr int E = kPayIds;
+    extern __shared__ __align__(128) uint32_t s_dyn[];
+    uint32_t* s_ids = s_dyn + 64;  // [kPayWarps][32 * E], after the warps' barriers
+    uint32_t* s_bits = s_ids + kPayWarps * 32 * E;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    IdStream<E> ids;
+    ids.init(s_dyn, s_ids, wib, lane);
+    stage_bits<FOLD>(s_bits, a.bits, smem_words, (y.catalogue >> 5) + 1);
+    __syncthreads();
+    const int64_t n_warps = (int64_t)gridDim.x * kPayWarps;
+    int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
+    uint32_t max_id = 0;
+    bool lost = false;
+    Trials<VEC> trials(y, n_warps);
+    Span<VEC> cur = trials.first(y, t);
+    ids.request(cur, 0, lane);
+    while (t < y.n_trials && !lost) {
+        const int64_t tn = t + n_warps;
+        const Span<VEC> nxt = trials.next(y, cur, tn);
+        unsigned long long carry = 0;  // C before the step, the same in every lane
+        int32_t first_full = -1;
+        double* pay = payouts ? payouts + (cur.p - y.ids) : nullptr;  // the payout of position 0
+        if (cur.n == 0) ids.request(nxt, 0, lane);
+        for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
+            uint32_t id[E];
+            if (!ids.take(cur, c0, lane, id)) {
+                lost = true;
+                break;
+            }
+            clean_ids<E>(cur, c0, lane, C, none, id, max_id);
+            if (c0 + 32 * E >= cur.n) ids.request(nxt, 0, lane);
+            else ids.request(cur, c0 + 32 * E, lane);
+            uint32_t o[E];
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                const bool nz = bit_of<FOLD>(s_bits, a.bits, id[k], S);
+                o[k] = 0;
+                if (nz) asm("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(o[k]) : "l"(a.x + id[k]));
+            }
+#pragma unroll
+            for (int h = 0; h < E / 4; ++h) {
+                const uint32_t d = c0 + 128u * h + 4u * lane;  // the lane's four consecutive positions
+                if (c0 + 128u * h >= cur.n) break;
+                const uint32_t* oh = o + 4 * h;
+                const unsigned long long total = (unsigned long long)oh[0] + oh[1] + oh[2] + oh[3];
+                unsigned long long run = total;
+#pragma unroll
+                for (int k = 1; k < 32; k <<= 1) {
+                    const unsigned long long v = __shfl_up_sync(kFull, run, k);
+                    if (lane >= k) run += v;
+                }
+                const unsigned long long after = carry + __shfl_sync(kFull, run, 31);
+                double v[4] = {0.0, 0.0, 0.0, 0.0};
+                if (after >= a.pass && carry < a.full) {  // the same for the whole warp
+                    if (carry >= a.pass && after < a.full) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i] = units_f64(oh[i], a.unit_f);
+                    } else {  // some event crosses the retention or the limit
+                        unsigned long long c = carry + run - total;
+                        int32_t at = -1;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const unsigned long long before = c;
+                            c += oh[i];
+                            if (before >= a.pass && c < a.full) v[i] = units_f64(oh[i], a.unit_f);
+                            else if (c >= a.pass && before < a.full) v[i] = agg_of(a, c) - agg_of(a, before);
+                            if (before < a.full && c >= a.full) at = (int32_t)(d + i - cur.head());
+                        }
+                        const unsigned m = __ballot_sync(kFull, at >= 0);
+                        if (m) first_full = __shfl_sync(kFull, at, __ffs(m) - 1);
+                    }
+                }
+                carry = after;
+                if (pay) {
+                    if (pay_vec && d >= cur.head() && d + 4 <= cur.n) {
+                        st_payouts4(pay + d, v);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (d + i >= cur.head() && d + i < cur.n) pay[d + i] = v[i];
+                    }
+                }
+            }
+        }
+        if (lane == 0 && !lost) {
+            if (exhaust) exhaust[t] = first_full;
+            if (ylt) ylt[t] = agg_of(a, carry);  // A(C_K): the telescoped sum of the payouts
+        }
+        t = tn;
+        cur = nxt;
+    }
+    if (lost) {
+        ids.phase ^= 1u;
+        ids.wait();  // the copy in flight may still come: shared memory stays until then
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
+    }
+    if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
+    if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
+}
+
+// The smallest N for which f(N * unit) holds (f never turns false again), or
+// all ones when it does not below 2^63.
+template <class F>
+unsigned long long first_units(double unit, F f) {
+    unsigned long long lo = 0, hi = 1ULL << 63;
+    if (!f((double)hi * unit)) return ~0ULL;
+    while (lo < hi) {
+        const unsigned long long mid = lo + (hi - lo) / 2;
+        if (f((double)mid * unit)) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
+// The whole-number form of the call. The table costs one read of the layer's
+// rows, an occurrence evaluated by itself about a row's gather (24 us per
+// million against 3): it is built from C / 2 events on (a CSR's trials are
+// taken as 500 events each, its length being on the device). done: false where
+// the call keeps the other form.
+cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double lims, const YetArgs& y, double* payouts,
+                         int32_t* exhaust, double* ylt, cudaStream_t s, bool* done) {
+    *done = false;
+    int e2;
+    double top;
+    const double events = (double)y.n_trials * (y.off ? 500.0 : (double)y.k);
+    if (events < 0.5 * p->catalogue || !ids_on_device(y.ids) ||
+        !whole_losses(la.occ_ret, la.occ_lim, lims, &e2, &top))
+        return cudaSuccess;
+    PayArgs a;
+    a.unit = std::ldexp(1.0, e2);
+    a.unit_f = (float)a.unit;
+    a.agg_ret = la.agg_ret;
+    a.agg_lim = la.agg_lim;
+    a.pass = first_units(a.unit, [&](double c) { return c - la.agg_ret > 0.0; });
+    a.full = first_units(a.unit, [&](double c) { return c - la.agg_ret >= la.agg_lim; });
+    const int32_t C = p->catalogue;
+    const int words = (C >> 5) + 1;
+    const size_t padded = (size_t)(words + 3) & ~(size_t)3;  // whole 16-byte groups
+    const size_t xb = (sizeof(uint32_t) * (size_t)C + 255) & ~(size_t)255;
+    int dev = 0, max_optin = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev))) return e;
+    if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+    max_optin = std::min(max_optin, 195 * 1024);  // L1 for the gathers in flight, as in ylt_fixed.cu
+    const int fixed_bytes = 256 + 16 + kPayWarps * 32 * kPayIds * 4;
+    const int smem_words = std::max(4, std::min((int)padded, (max_optin - fixed_bytes) / 4) & ~3);
+    const int smem = fixed_bytes + smem_words * 4;
+    const bool fold = words <= 2 * smem_words;
+    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
+    const bool pay_vec =
+        ((reinterpret_cast<uintptr_t>(payouts) >> 3) - (reinterpret_cast<uintptr_t>(y.ids) >> 2)) % 4 == 0;
+    auto kern = vec ? (fold ? payouts_fixed_kernel<true, true> : payouts_fixed_kernel<true, false>)
+                    : (fold ? payouts_fixed_kernel<false, true> : payouts_fixed_kernel<false, false>);
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    char* w = nullptr;
+    if ((e = scratch_alloc((void**)&w, xb + sizeof(uint32_t) * padded, s))) return e;
+    uint32_t* x = reinterpret_cast<uint32_t*>(w);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(w + xb);
+    a.x = x;
+    a.bits = bits;
+    const float scale = (float)std::ldexp(1.0, -e2);
+    const unsigned blocks = (unsigned)((padded * 32 + 255) / 256);
+    switch (np) {
+        case 4: payouts_table_kernel<4><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+        case 8: payouts_table_kernel<8><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+        case 16: payouts_table_kernel<16><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+        case 24: payouts_table_kernel<24><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+        default: payouts_table_kernel<32><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+    }
+    if (!(e = cudaGetLastError())) {
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(p->num_sms, y.n_trials));
+        kern<<<(unsigned)grid, kPayThreads, smem, s>>>(a, y, smem_words, pay_vec, payouts, exhaust, ylt, p->d_flags);
+        e = cudaGetLastError();
+    }
+    const cudaError_t e3 = cudaFreeAsync(w, s);
+    *done = true;
+    return e ? e : e3;
+}
+
 }  // namespace
 
 cudaError_t launch_payouts(art_portfolio* p, int32_t j, const YetArgs& y, double* payouts, int32_t* exhaust,
@@ -110,6 +369,11 @@ cudaError_t launch_payouts(art_portfolio* p, int32_t j, const YetArgs& y, double
     la.agg_ret = p->agg_ret[j];
     la.agg_lim = p->agg_lim[j];
     la.layer = j;
+    double lims = 0.0;
+    for (int k = 0; k < n; ++k) lims += la.lim[k];
+    bool done = false;
+    const cudaError_t err = launch_whole(p, la, p->layer_np[j], lims, y, payouts, exhaust, ylt, s, &done);
+    if (err || done) return err;
     switch (p->layer_np[j]) {
         case 4: return launch<4>(la, y, payouts, exhaust, ylt, p->d_flags, s);
         case 8: return launch<8>(la, y, payouts, exhaust, ylt, p->d_flags, s);

@@ -1,0 +1,151 @@
+"""The passes over occurrence tables of whole numbers (skip variant, payouts):
+sums are exact, so the YLT equals the FP64 sum of the FP32 occurrence losses
+(every partial sum is a multiple of one unit below 2^53) bit for bit, at the
+edges of chunks, vectors, layers per group and alignments of the id array."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1308_2572_gb300 import art, workloads
+
+pytestmark = pytest.mark.gpu
+
+# around a warp's vector (4), a half chunk (128) and a chunk (256) of ids
+LENGTHS = [0, 1, 3, 4, 5, 31, 127, 128, 129, 252, 255, 256, 257, 260, 511, 513, 1000, 2049]
+
+
+def _case(n_layers, catalogue, seed=5, unlimited=False):
+    rng = np.random.default_rng(seed)
+    w = workloads.random_case(seed, catalogue=catalogue, n_elt=12, n_layers=n_layers, n_trials=1, dense_k=4,
+                              max_elts_per_layer=6, nnz_frac=0.2)
+    p = w.portfolio
+    if unlimited:
+        p.occ_lim[0] = np.inf
+        p.elt_lim[:] = np.inf  # nothing bounds the first layer's losses: its group keeps FP32 tables
+    return w, rng
+
+
+def _occ_losses(p):
+    """o[j][i] in FP32 as the library forms them (m = 1), widened to FP64."""
+    out = np.zeros((p.n_layers, p.catalogue_size))
+    for j in range(p.n_layers):
+        x = np.zeros(p.catalogue_size, np.float32)
+        for e in p.layer_elt_ids[p.layer_elt_off[j]:p.layer_elt_off[j + 1]]:
+            f = np.minimum(np.maximum(p.elt_losses[e] - p.elt_ded[e], np.float32(0)), p.elt_lim[e])
+            x = x + f.astype(np.float32)
+        o = np.minimum(np.maximum(x - np.float32(p.occ_ret[j]), np.float32(0)), np.float32(p.occ_lim[j]))
+        out[j] = o.astype(np.float64)
+    return out
+
+
+def _yet(rng, catalogue, lengths, shift):
+    """A ragged YET whose id array starts `shift` ids past a 16-byte boundary."""
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    ids = rng.integers(0, catalogue, size=int(off[-1]), dtype=np.int32)
+    buf = torch.zeros(ids.size + 8, dtype=torch.int32, device="cuda")
+    dev = buf[shift:shift + ids.size]
+    dev.copy_(torch.from_numpy(ids))
+    return ids, off, dev, torch.from_numpy(off).cuda()
+
+
+def _expected(o, p, ids, off):
+    s = np.stack([np.add.reduceat(np.append(o[j][ids], 0.0), off[:-1].clip(max=max(0, ids.size))) for j in range(len(o))])
+    s[:, np.diff(off) == 0] = 0.0
+    return np.minimum(np.maximum(s - p.agg_ret[:, None], 0.0), p.agg_lim[:, None])
+
+
+# catalogues whose bitmap fits, folds once and needs more than one fold
+@pytest.mark.parametrize("n_layers,catalogue", [(1, 97), (2, 5000), (3, 5000), (8, 97), (9, 5000), (17, 5000),
+                                                (1, 1_999_999), (8, 1_999_999), (1, 4_000_037), (3, 4_000_037)])
+def test_skip_sums_are_exact(n_layers, catalogue):
+    w, rng = _case(n_layers, catalogue)
+    p = w.portfolio
+    o = _occ_losses(p)
+    lengths = np.array(LENGTHS * 4 + [1000] * 90)
+    rng.shuffle(lengths)
+    port = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER, variant=art.ART_VARIANT_SKIP)
+    try:
+        for shift in range(4):
+            ids, off, dev, doff = _yet(rng, catalogue, lengths, shift)
+            want = _expected(o, p, ids, off)
+            y = torch.full((n_layers, lengths.size), -1.0, dtype=torch.float64, device="cuda")
+            br = torch.full((n_layers, lengths.size), 9, dtype=torch.uint8, device="cuda")
+            art.art_run_ylt(port, lengths.size, dev, doff, 0, y, br)
+            assert art.art_get_device_status(port) == art.ART_OK
+            np.testing.assert_array_equal(y.cpu().numpy(), want)
+            s = want + 0.0
+            b = br.cpu().numpy()
+            assert np.all(b[s == 0] == 0) and np.all((b == 1) == ((s > 0) & (s < p.agg_lim[:, None])))
+        for k in (1, 4, 6, 256, 1000):  # dense
+            t = 61
+            ids = rng.integers(0, catalogue, size=t * k, dtype=np.int32)
+            y = torch.full((n_layers, t), -1.0, dtype=torch.float64, device="cuda")
+            art.art_run_ylt(port, t, torch.from_numpy(ids).cuda(), None, k, y)
+            np.testing.assert_array_equal(y.cpu().numpy(), _expected(o, p, ids, np.arange(t + 1) * k))
+        # ids outside the catalogue count as no loss and are reported
+        ids, off, dev, doff = _yet(rng, catalogue, lengths, 1)
+        bad = ids.copy()
+        bad[::97] = np.where(np.arange(bad[::97].size) % 2 == 0, catalogue, -5)
+        dev.copy_(torch.from_numpy(bad))
+        art.art_run_ylt(port, lengths.size, dev, doff, 0, torch.empty((n_layers, lengths.size), dtype=torch.float64, device="cuda"))
+        assert art.art_get_device_status(port) == art.ART_EID_RANGE
+    finally:
+        port.close()
+
+
+def test_unbounded_losses_keep_the_fp32_tables():
+    """A group with a layer whose losses are not bounded takes the compensated
+    pass; the other groups' results stay exact."""
+    w, rng = _case(9, 5000, unlimited=True)
+    p = w.portfolio
+    o = _occ_losses(p)
+    lengths = np.array(LENGTHS * 3)
+    ids, off, dev, doff = _yet(rng, 5000, lengths, 3)
+    port = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER, variant=art.ART_VARIANT_SKIP)
+    try:
+        y = torch.empty((9, lengths.size), dtype=torch.float64, device="cuda")
+        art.art_run_ylt(port, lengths.size, dev, doff, 0, y)
+        want = _expected(o, p, ids, off)
+        got = y.cpu().numpy()
+        np.testing.assert_array_equal(got[8], want[8])
+        # the compensated sums: an error of order n u^2 of the sum
+        np.testing.assert_allclose(got, want, rtol=1e-11, atol=1e-11 * float(o.max()))
+    finally:
+        port.close()
+
+
+@pytest.mark.parametrize("catalogue", [97, 1_999_999])
+def test_payouts_are_exact(catalogue):
+    w, rng = _case(2, catalogue, seed=11)
+    p = w.portfolio
+    o = _occ_losses(p)
+    lengths = np.array(LENGTHS * 4 + [1000] * (1100 if catalogue > 1000 else 60))
+    rng.shuffle(lengths)
+    port = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER)
+    try:
+        for j, shift, pshift in [(0, 0, 0), (1, 1, 1), (0, 3, 0), (1, 2, 3)]:
+            ids, off, dev, doff = _yet(rng, catalogue, lengths, shift)
+            buf = torch.full((ids.size + 8,), -7.0, dtype=torch.float64, device="cuda")
+            pay = buf[pshift:pshift + ids.size]
+            ex = torch.full((lengths.size,), -9, dtype=torch.int32, device="cuda")
+            y = torch.full((lengths.size,), -1.0, dtype=torch.float64, device="cuda")
+            art.art_run_payouts(port, j, lengths.size, dev, doff, 0, pay, ex, y)
+            assert art.art_get_device_status(port) == art.ART_OK
+            np.testing.assert_array_equal(y.cpu().numpy(), _expected(o[j:j + 1], _Layer(p, j), ids, off)[0])
+            got, exh = pay.cpu().numpy(), ex.cpu().numpy()
+            assert torch.all(buf[:pshift] == -7.0) and torch.all(buf[pshift + ids.size:] == -7.0)
+            for t in range(lengths.size):
+                c = np.cumsum(o[j][ids[off[t]:off[t + 1]]])
+                a = np.minimum(np.maximum(c - p.agg_ret[j], 0.0), p.agg_lim[j])
+                full = np.nonzero(c - p.agg_ret[j] >= p.agg_lim[j])[0]
+                assert exh[t] == (full[0] if full.size else -1)
+                # a payout of the exact difference against one of rounded values: an ulp of each
+                np.testing.assert_allclose(got[off[t]:off[t + 1]], np.diff(np.concatenate([[0.0], a])), rtol=0,
+                                           atol=4e-16 * max(1.0, float(c[-1]) if c.size else 1.0))
+    finally:
+        port.close()
+
+
+class _Layer:
+    def __init__(self, p, j):
+        self.agg_ret, self.agg_lim = p.agg_ret[j:j + 1], p.agg_lim[j:j + 1]
