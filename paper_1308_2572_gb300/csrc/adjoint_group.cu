@@ -12,76 +12,84 @@
 //
 // Which occurrence branch each layer takes, and which ELT terms are on their
 // middle branch, depend on the event id alone. So each call first evaluates
-// them once per catalogue event i (the group table row, F_e and the layer
-// sums x_ij in FP32, in the group's ELT order): M_i, the layers on the middle
-// branch; K_i, the layers on the capped branch; and U_i, the ELT columns on
-// their middle branch; plus a bitmap of the events with M_i or K_i non-zero
-// (only those contribute). The trial pass is then shaped like the forward's:
-// a persistent CTA per SM with the bitmap in shared memory (folded once when
-// it does not fit), a warp per trial streaming its ids, and a per-warp queue
-// of the events whose bit is set, evaluated 32 at a time (lane = event):
+// them once per catalogue event i (F_e and the layer sums x_ij in FP32, in the
+// group's ELT order): M_i, the layers on the middle branch; K_i, the layers on
+// the capped branch; and U_i, the ELT columns on their middle branch, plus a
+// bitmap of the events with M_i or K_i non-zero (only those contribute). What
+// the trial pass needs of such an event is one 32-byte record: M_i spread to
+// byte counters, K_i, and up to three (column, layers covering it with a
+// middle branch, loss); the few events with more columns are evaluated from
+// their table row. Records come from the CSR of the non-zero losses where the
+// portfolio holds it (an event with three or more of the group's losses from
+// its table row, in the group's order), else from the table rows; the same
+// values either way.
+//
+// The trial pass is shaped like the forward's (ylt_fixed.cu): a persistent CTA
+// per SM, the bitmap folded into shared memory, a warp per trial streaming its
+// ids by bulk copies, and a per-warp ring of the events whose bit is set,
+// evaluated 32 at a time (lane = event), each gather running beside the tests
+// that follow it:
 //   - the layer counts: per lane, 8-bit counters for the 8 layers packed in
-//     a 64-bit word, incremented by a table lookup of M (and K); reduced
-//     across the warp with integer reductions at the end of the trial (and
-//     every 255 batches), then lane j adds layer j's counts times g_j (g_j
-//     rounded to FP32, the product exact) to a compensated FP32 pair;
-//   - the multipliers: for each column k in U_i with M_i non-zero, the lane
-//     adds l_ik * W[M_i & C_k] to its FP32 partial of column k, where C_k is
-//     the set of layers covering column k and W[S] = sum_{j in S} g_j a_j is
-//     a 2^LT-entry table of the trial's weights (FP32, per warp, built per
-//     trial); at the end of the trial the partials are summed across the
-//     warp (recursive halving: 31 shuffles for every column at once) and
-//     lane k adds column k's total to its compensated FP32 pair.
-// A trial with no layer on the middle branch costs only its branch codes.
-// The lane values are reduced warp -> CTA -> grid in a fixed order (no
-// atomics: deterministic); FP64 arithmetic runs only in that final
-// reduction. Rounding: g is rounded to FP32 once per (layer, trial), and the
-// per-event products and the W entries are FP32 (a few units in the last
-// place of FP32 per term); every sum is compensated or FP64.
+//     two words, added from the record; summed across the warp in 16-bit
+//     fields (one REDUX for two layers) at the end of the trial (and every 255
+//     batches), then lane j adds layer j's counts times g_j (g_j rounded to
+//     FP32, the product exact) to a compensated FP32 pair;
+//   - the multipliers: for each (column k, layers S, loss l) of the record the
+//     lane adds l * W[S] to its own FP32 partial of column k in shared memory,
+//     W[S] = sum_{j in S} g_j a_j from two 16-entry tables of the trial's
+//     weights; every kFold batches the partials are summed across the warp
+//     (recursive halving: 31 shuffles for every column at once) and lane k adds
+//     column k's total to its compensated FP32 pair.
+// A trial with no layer on the middle branch costs only its branch codes. The
+// lane values are reduced warp -> CTA -> grid in a fixed order (no atomics:
+// deterministic); FP64 arithmetic runs only in that final reduction. Rounding:
+// g is rounded to FP32 once per (layer, trial), and the per-event products and
+// the W entries are FP32 (a few units in the last place of FP32 per term);
+// every sum is compensated or FP64.
+//
+// What bounds the pass (ncu, c3): issue (58%; 52 instructions per 32 events,
+// of which the two POPC of the ring take 4 of 23 cycles) with 20 warps per SM.
+// c3, 500,000 trials: 1.24 ms, with the records 1.28, against 1.95 for the form
+// that gathered 64-byte rows and tested 16 columns per queued event.
 #include <algorithm>
 #include <limits>
 
-#include "art_internal.cuh"
+#include "id_stream.cuh"
 
 namespace art {
 
 namespace {
 
-// Threads per CTA of the trial pass and ids per lane in flight, by the
-// group's column count. Up to 16 columns the pass needs about 80 registers
-// per thread, and 24 warps per SM with 4 ids each hide more of the gathers'
-// latency than 16 warps with 8 ids (c3 adjoint 3.88 against 4.18 ms; 1024
-// threads spill); wider groups keep 512 threads with 8 ids (128 registers,
-// no spills).
+// Warps per CTA: each holds a column partial per lane (4 * 32 * NP bytes of
+// shared memory), which the bitmap competes with; 20 warps leave 96 registers
+// a thread, so that nothing is spilled in the chunk loop (24 warps with spills
+// take the same time, 16 warps 8% more).
 template <int NP>
-constexpr int kAgThreadsFor = NP <= 16 ? 768 : 512;
-template <int NP>
-constexpr int kAgIdsFor = NP <= 16 ? 4 : 8;
-constexpr int kAgQueue = 64;  // per-warp queue entries
+constexpr int kAgWarpsFor = NP <= 16 ? 20 : 16;
+constexpr int kAgIds = 8;     // ids per lane and chunk
+constexpr int kFold = 32;     // batches between the folds of the column partials
+constexpr uint32_t kOverflow = 7u;  // more than three columns: evaluated from the table row
 
-__device__ __forceinline__ uint32_t ld_bits_global(const uint32_t* p) {
-    uint32_t v;
-    asm("ld.global.nc.L1::evict_last.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
+// What the trial pass reads of an event.
+struct alignas(32) AdjRecord {
+    uint32_t mid_lo, mid_hi;  // byte j (mid_hi: 4 + j): layer j on its middle branch
+    uint32_t meta;            // columns (5 bits each), their number (bits 15-17), K (bits 20-27)
+    uint32_t sets;            // per column, the layers covering it on their middle branch (kOverflow: M)
+    float loss[3];            // their losses
+    uint32_t u;               // U (kOverflow)
+};
 
-__device__ __forceinline__ uint2 ld_mask(const uint2* p) {
-    uint2 v;
-    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
-
-__device__ __forceinline__ void ld_row8(const float* p, float* v) {
-    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+__device__ __forceinline__ AdjRecord ld_record(const AdjRecord* p) {
+    AdjRecord r;
+    asm("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r.mid_lo), "=r"(r.mid_hi), "=r"(r.meta), "=r"(r.sets), "=f"(r.loss[0]), "=f"(r.loss[1]), "=f"(r.loss[2]),
+          "=r"(r.u)
         : "l"(p));
+    return r;
 }
 
-__device__ __forceinline__ void ld_row4(const float* p, float* v) {
-    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
-        : "l"(p));
-}
+// Bits 0-3 of m to the lowest bits of four bytes.
+__device__ __forceinline__ uint32_t spread4(uint32_t m) { return ((m & 15u) * 0x00204081u) & 0x01010101u; }
 
 // (h, l) += v, keeping the rounding error of the FP32 add (two-sum)
 __device__ __forceinline__ void two_sum_add(float& h, float& l, float v) {
@@ -91,138 +99,195 @@ __device__ __forceinline__ void two_sum_add(float& h, float& l, float v) {
     h = t;
 }
 
-// Per catalogue event i of a group: masks[i] = (M | K << 8, U) and bit i of
-// the bitmap set when M | K is non-zero. Row C (the sentinel for ids outside
-// the catalogue) is never written: it stays zero.
-template <int NP, int LT>
-__global__ void __launch_bounds__(256) adj_masks_kernel(const GroupArgs g, int32_t catalogue, int32_t words,
-                                                        uint2* __restrict__ masks, uint32_t* __restrict__ bits) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool rel = false;
-    if (i < catalogue) {
-        const float4* row = reinterpret_cast<const float4*>(g.table) + i * (NP / 4);
-        float v[NP];
+// The layers covering column k, as the group's membership lists them.
+__device__ __forceinline__ uint32_t layers_of(const GroupArgs& g, int k) {
+    uint32_t c = 0;
+    for (int j = 0; j < g.n_layers; ++j) c |= ((g.member[j] >> k) & 1u) << j;
+    return c;
+}
+
+// Branches of the layers at the sums x.
+template <int LT>
+__device__ __forceinline__ void layer_branches(const GroupArgs& g, const float (&x)[LT], uint32_t& mid, uint32_t& cap) {
+    mid = cap = 0u;
 #pragma unroll
-        for (int q = 0; q < NP / 4; ++q) {
-            const float4 r = __ldcs(row + q);
-            v[4 * q + 0] = r.x;
-            v[4 * q + 1] = r.y;
-            v[4 * q + 2] = r.z;
-            v[4 * q + 3] = r.w;
+    for (int j = 0; j < LT; ++j)
+        if (j < g.n_layers) {
+            const float wo = x[j] - g.occ_ret[j];  // the forward's occurrence subtraction
+            if (wo > 0.0f && wo < g.occ_lim[j]) mid |= 1u << j;
+            if (wo > g.occ_lim[j]) cap |= 1u << j;
         }
-        float f[NP];
-        uint32_t u = 0u;
+}
+
+__device__ __forceinline__ void add_column(AdjRecord& r, uint32_t& n, uint32_t mid, uint32_t cover, int k, float loss) {
+    const uint32_t set = mid & cover;
+    if (!set) return;
+    if (n < 3) {
+        r.meta |= (uint32_t)k << (5 * n);
+        r.sets |= set << (8 * n);
+        if (n == 0) r.loss[0] = loss;
+        if (n == 1) r.loss[1] = loss;
+        if (n == 2) r.loss[2] = loss;
+    }
+    ++n;
+}
+
+__device__ __forceinline__ void finish_record(AdjRecord& r, uint32_t n, uint32_t mid, uint32_t cap, uint32_t u) {
+    r.mid_lo = spread4(mid);
+    r.mid_hi = spread4(mid >> 4);
+    if (n > 3) {
+        r.sets = mid;
+        r.u = u;
+        n = kOverflow;
+    }
+    r.meta |= n << 15 | cap << 20;
+}
+
+// Event i from its table row; false when it is on no branch that counts.
+template <int NP, int LT>
+__device__ bool record_from_row(const GroupArgs& g, const uint32_t* s_cover, int64_t i, AdjRecord& r) {
+    const float4* row = reinterpret_cast<const float4*>(g.table) + i * (NP / 4);
+    float v[NP], f[NP];
+#pragma unroll
+    for (int q = 0; q < NP / 4; ++q) {
+        const float4 w = __ldcs(row + q);
+        v[4 * q + 0] = w.x;
+        v[4 * q + 1] = w.y;
+        v[4 * q + 2] = w.z;
+        v[4 * q + 3] = w.w;
+    }
+    uint32_t u = 0u;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const float wf = __fmaf_rn(g.m[k], v[k], -g.d[k]);
+        f[k] = fminf(fmaxf(wf, 0.0f), g.lim[k]);
+        if (wf > 0.0f && wf < g.lim[k]) u |= 1u << k;
+    }
+    float x[LT];
+#pragma unroll
+    for (int j = 0; j < LT; ++j) {
+        x[j] = 0.0f;
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
-            const float wf = __fmaf_rn(g.m[k], v[k], -g.d[k]);
-            f[k] = fminf(fmaxf(wf, 0.0f), g.lim[k]);
-            if (wf > 0.0f && wf < g.lim[k]) u |= 1u << k;
+            if constexpr (LT == 1) x[j] += f[k];
+            else x[j] = __fmaf_rn(g.coef[j][k], f[k], x[j]);
         }
-        uint32_t mk = 0u;
+    }
+    uint32_t mid, cap, n = 0;
+    layer_branches<LT>(g, x, mid, cap);
+    if (!(mid | cap)) return false;
 #pragma unroll
-        for (int j = 0; j < LT; ++j) {
-            if (j < g.n_layers) {
-                float x = 0.0f;
-#pragma unroll
-                for (int k = 0; k < NP; ++k) {
-                    if constexpr (LT == 1) x += f[k];
-                    else x = __fmaf_rn(g.coef[j][k], f[k], x);
+    for (int k = 0; k < NP; ++k)
+        if ((u >> k) & 1u) add_column(r, n, mid, s_cover[k], k, v[k]);
+    finish_record(r, n, mid, cap, u);
+    return true;
+}
+
+// Records and bitmap of a group, one thread per event. ptr NULL: from the
+// table rows. col: the group's column of a pool ELT, 255 for none.
+template <int NP, int LT>
+__global__ void __launch_bounds__(256) adj_records_kernel(const __grid_constant__ GroupArgs g, int32_t catalogue,
+                                                          int32_t words, const uint32_t* __restrict__ ptr,
+                                                          const SparseEntry* __restrict__ entries,
+                                                          const uint8_t* __restrict__ col,
+                                                          AdjRecord* __restrict__ records,
+                                                          uint32_t* __restrict__ bits) {
+    __shared__ uint32_t s_cover[32];
+    __shared__ float s_m[32], s_d[32], s_lim[32];
+    if (threadIdx.x < 32) {
+        s_cover[threadIdx.x] = layers_of(g, threadIdx.x);
+        s_m[threadIdx.x] = g.m[threadIdx.x];
+        s_d[threadIdx.x] = g.d[threadIdx.x];
+        s_lim[threadIdx.x] = g.lim[threadIdx.x];
+    }
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    bool rel = false;
+    AdjRecord r{};
+    if (i < catalogue) {
+        if (!ptr) {
+            rel = record_from_row<NP, LT>(g, s_cover, i, r);
+        } else {
+            int cnt = 0, ka = 0, kb = 0;
+            float va = 0.0f, vb = 0.0f;
+            const uint32_t q1 = ptr[i + 1];
+            for (uint32_t q = ptr[i]; q < q1; ++q) {
+                const SparseEntry en = entries[q];
+                const int k = col[en.elt];
+                if (k == 255) continue;
+                if (cnt == 0) {
+                    ka = k;
+                    va = en.loss;
+                } else {
+                    kb = k;
+                    vb = en.loss;
                 }
-                const float wo = x - g.occ_ret[j];  // the forward's occurrence subtraction
-                if (wo > 0.0f && wo < g.occ_lim[j]) mk |= 1u << j;
-                if (wo > g.occ_lim[j]) mk |= 1u << (8 + j);
+                ++cnt;
+            }
+            if (cnt > 2) {
+                rel = record_from_row<NP, LT>(g, s_cover, i, r);
+            } else if (cnt) {
+                // one or two losses: their sum is the same in any order
+                const float wa = __fmaf_rn(s_m[ka], va, -s_d[ka]), wb = __fmaf_rn(s_m[kb], vb, -s_d[kb]);
+                const float fa = fminf(fmaxf(wa, 0.0f), s_lim[ka]);
+                const float fb = cnt > 1 ? fminf(fmaxf(wb, 0.0f), s_lim[kb]) : 0.0f;
+                float x[LT];
+#pragma unroll
+                for (int j = 0; j < LT; ++j)
+                    x[j] = ((s_cover[ka] >> j) & 1u ? fa : 0.0f) + (cnt > 1 && ((s_cover[kb] >> j) & 1u) ? fb : 0.0f);
+                uint32_t mid, cap, n = 0;
+                layer_branches<LT>(g, x, mid, cap);
+                rel = (mid | cap) != 0u;
+                if (wa > 0.0f && wa < s_lim[ka]) add_column(r, n, mid, s_cover[ka], ka, va);
+                if (cnt > 1 && wb > 0.0f && wb < s_lim[kb]) add_column(r, n, mid, s_cover[kb], kb, vb);
+                finish_record(r, n, mid, cap, 0u);
             }
         }
-        masks[i] = make_uint2(mk, (mk & 0xffu) ? u : 0u);
-        rel = mk != 0u;
+        {  // an event without its bit too: the folded bitmap may gather it
+            uint4* dst = reinterpret_cast<uint4*>(records + i);
+            dst[0] = make_uint4(r.mid_lo, r.mid_hi, r.meta, r.sets);
+            dst[1] = make_uint4(__float_as_uint(r.loss[0]), __float_as_uint(r.loss[1]), __float_as_uint(r.loss[2]), r.u);
+        }
     }
-    const unsigned m = __ballot_sync(0xffffffffu, rel);
+    const unsigned m = __ballot_sync(kFull, rel);
     if ((threadIdx.x & 31) == 0 && (i >> 5) < words) bits[i >> 5] = m;
 }
 
-// One queued event on one lane: the packed layer counters and, when a layer
-// is on its middle branch, the column partials.
-template <int NP, int LT>
-__device__ __forceinline__ void eval_event(const GroupArgs& g, const uint2* __restrict__ masks, uint32_t id,
-                                           uint32_t last_row, const uint64_t* s_spread, const float* s_w, const uint32_t* s_col,
-                                           uint64_t& cnt_mid, uint64_t& cnt_cap, float (&part)[NP]) {
-    // the row is requested together with the masks (most queued events need
-    // it), so the two gathers overlap; the sentinel C (zero masks) reads the
-    // last row instead, unused
-    const uint2 mk = ld_mask(masks + id);
-    const float* row = g.table + (size_t)min(id, last_row) * NP;
-    float v[NP];
-    if constexpr (NP % 8 == 0) {
-#pragma unroll
-        for (int q = 0; q < NP / 8; ++q) ld_row8(row + 8 * q, v + 8 * q);
-    } else {
-#pragma unroll
-        for (int q = 0; q < NP / 4; ++q) ld_row4(row + 4 * q, v + 4 * q);
-    }
-    const uint32_t m = mk.x & 0xffu;
-    cnt_mid += s_spread[m];
-    cnt_cap += s_spread[(mk.x >> 8) & 0xffu];
-    if (mk.y != 0u) {  // U is stored only where M is non-zero
-#pragma unroll
-        for (int k = 0; k < NP; ++k)
-            if ((mk.y >> k) & 1u) part[k] = __fmaf_rn(v[k], s_w[m & s_col[k]], part[k]);
-    }
-}
+// A trial's branch code and weight as lane j holds them for layer j.
+struct Weight {
+    float g = 0.0f;
+    uint8_t code = 0;
+};
 
 template <int NP, int LT, bool VEC, bool FOLD>
-__global__ void __launch_bounds__(kAgThreadsFor<NP>, 1) adjoint_pass_kernel(const GroupArgs g, const YetArgs y,
-                                                                     const uint2* __restrict__ masks,
-                                                                     const uint32_t* __restrict__ gbits,
-                                                                     const int32_t smem_words,
-                                                                     const uint8_t* __restrict__ branch,
-                                                                     const double* __restrict__ gw,
-                                                                     double* __restrict__ partial) {
-    constexpr unsigned FULL = 0xffffffffu;
-    constexpr int E = kAgIdsFor<NP>;
-    constexpr int kAgWarps = kAgThreadsFor<NP> / 32;
-    constexpr int NW = 1 << LT;      // entries of a warp's weight table
+__global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
+    adjoint_pass_kernel(const __grid_constant__ GroupArgs g, const YetArgs y, const AdjRecord* __restrict__ records,
+                        const uint32_t* __restrict__ gbits, const int32_t smem_words, const int64_t warp_step,
+                        const int64_t cta_step, const uint8_t* __restrict__ branch, const double* __restrict__ gw,
+                        double* __restrict__ partial, int* __restrict__ flags) {
+    constexpr int E = kAgIds;
+    constexpr int NWARP = kAgWarpsFor<NP>;
     constexpr int W = 4 * LT + NP;   // OccR[LT], OccL[LT], AggR[LT], AggL[LT], then the columns
-    extern __shared__ __align__(16) uint32_t s_dyn[];
-    uint64_t* s_spread = reinterpret_cast<uint64_t*>(s_dyn);            // [256]
-    double* s_red = reinterpret_cast<double*>(s_dyn + 512);              // [kAgWarps][W]
-    uint32_t* s_col = s_dyn + 512 + 2 * kAgWarps * W;                    // [32]
-    float* s_wt = reinterpret_cast<float*>(s_col + 32);                  // [kAgWarps][NW]
-    int32_t* s_queue = reinterpret_cast<int32_t*>(s_wt + kAgWarps * NW); // [kAgWarps][kAgQueue]
-    uint32_t* s_bits = reinterpret_cast<uint32_t*>(s_queue + kAgWarps * kAgQueue);
-    {
-        // s_spread[m]: byte j is bit j of m (adds one to layer j's counter)
-        for (int m = threadIdx.x; m < 256; m += blockDim.x) {
-            uint64_t v = 0;
-            for (int j = 0; j < 8; ++j) v |= (uint64_t)((m >> j) & 1) << (8 * j);
-            s_spread[m] = v;
-        }
-        if (threadIdx.x < 32) {
-            uint32_t c = 0;
-            for (int j = 0; j < LT; ++j)
-                if (j < g.n_layers) c |= ((g.member[j] >> threadIdx.x) & 1u) << j;
-            s_col[threadIdx.x] = c;
-        }
-        const uint4* src = reinterpret_cast<const uint4*>(gbits);
-        uint4* dst = reinterpret_cast<uint4*>(s_bits);
-        const int words = (y.catalogue >> 5) + 1;  // bits 0 .. C (C: the sentinel)
-        for (int i = threadIdx.x; i < smem_words / 4; i += blockDim.x) {
-            uint4 v = src[i];
-            if (FOLD && 4 * i + smem_words < words) {  // the bitmap is zero-padded to whole uint4
-                const uint4 u = src[i + smem_words / 4];
-                v.x |= u.x;
-                v.y |= u.y;
-                v.z |= u.z;
-                v.w |= u.w;
-            }
-            dst[i] = v;
-        }
-    }
-    __syncthreads();
+    extern __shared__ __align__(512) uint32_t s_dyn[];
+    uint32_t* s_bars = s_dyn + NWARP * kRing;                            // after the warps' rings
+    uint32_t* s_ids = s_bars + 64;                                       // [NWARP][32 * E]
+    float* s_part = reinterpret_cast<float*>(s_ids + NWARP * 32 * E);    // [NWARP][NP][32]
+    float* s_wt = s_part + NWARP * NP * 32;                              // [NWARP][32]: low and high layers' sums
+    uint32_t* s_cover = reinterpret_cast<uint32_t*>(s_wt + NWARP * 32);  // [32]
+    uint32_t* s_bits = s_cover + 32;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    int32_t* q = s_queue + wib * kAgQueue;
-    float* s_w = s_wt + wib * NW;
+    IdStream<E> ids;
+    ids.init(s_bars, s_ids, wib, lane);
+    IdRing ring(s_dyn + wib * kRing);
+    float* part = s_part + wib * NP * 32 + lane;  // the lane's partial of column k: part[32 k]
+    for (int k = 0; k < NP; ++k) part[32 * k] = 0.0f;
+    if (threadIdx.x < 32) s_cover[threadIdx.x] = layers_of(g, threadIdx.x);
+    stage_bits<FOLD>(s_bits, gbits, smem_words, (y.catalogue >> 5) + 1);
+    __syncthreads();
+    float* s_w = s_wt + wib * 32;
     const unsigned lt_mask = (1u << lane) - 1u;
-    const int64_t n_warps = (int64_t)gridDim.x * kAgWarps;
+    const int64_t n_warps = (int64_t)gridDim.x * NWARP;
 
     // lane j < LT keeps layer j's four term sums, lane k < NP column k's sum,
     // each a compensated FP32 pair (FP64 arithmetic per trial would dominate:
@@ -233,144 +298,210 @@ __global__ void __launch_bounds__(kAgThreadsFor<NP>, 1) adjoint_pass_kernel(cons
 #pragma unroll
     for (int j = 0; j < LT; ++j)
         if (lane == j && j < g.n_layers) my_layer = g.layer[j];
-
-    for (int64_t t = (int64_t)blockIdx.x * kAgWarps + wib; t < y.n_trials; t += n_warps) {
-        float gt = 0.0f;  // the layer's weight, rounded to FP32 once
-        uint8_t code = 0;
-        if (my_layer >= 0) {
+    auto load_weight = [&](int64_t t) {
+        Weight w;
+        if (my_layer >= 0 && t < y.n_trials) {
             const size_t wi = (size_t)my_layer * (size_t)y.n_trials + (size_t)t;
-            code = branch[wi];
-            gt = (float)gw[wi];
+            w.code = branch[wi];
+            w.g = (float)gw[wi];  // the layer's weight, rounded to FP32 once
         }
-        if (code == 1) two_sum_add(ar_h, ar_l, -gt);
-        if (code == 2) two_sum_add(al_h, al_l, gt);
-        const bool mid_l = code == 1 && gt != 0.0f;
-        if (!__ballot_sync(FULL, mid_l)) continue;  // no layer of the group has a middle-branch weight
-        // the trial's weight table W[S] = sum_{j in S} g_j a_j, by doubling:
-        // W[S + 2^b] = W[S] + g_b a_b for S < 2^b (the terms in increasing j,
-        // as a direct sum adds them)
+        return w;
+    };
+    // the first trial from t on with a middle-branch weight in the group (the
+    // aggregate terms' sums take every trial passed); w holds trial t's weight
+    auto active_from = [&](int64_t t, Weight& w) {
+        while (t < y.n_trials) {
+            if (w.code == 1) two_sum_add(ar_h, ar_l, -w.g);
+            if (w.code == 2) two_sum_add(al_h, al_l, w.g);
+            if (__ballot_sync(kFull, w.code == 1 && w.g != 0.0f)) break;
+            t += n_warps;
+            w = load_weight(t);
+        }
+        return t;
+    };
+
+    // the lanes' partials summed across the warp by recursive halving (31
+    // shuffles for all columns): at distance o a lane keeps the half of its
+    // columns selected by bit o of its index and adds the partner's copy of
+    // that half; lane k ends with column k
+    auto fold_columns = [&]() {
+        float v[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            v[k] = 0.0f;
+            if (k < NP) {
+                v[k] = part[32 * k];
+                part[32 * k] = 0.0f;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool upper = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const float keep = upper ? v[i + o] : v[i];
+                const float send = upper ? v[i] : v[i + o];
+                v[i] = keep + __shfl_xor_sync(kFull, send, o);
+            }
+        }
+        if (lane < NP) two_sum_add(col_h, col_l, v[0]);
+    };
+
+    int64_t t = (int64_t)wib * warp_step + (int64_t)blockIdx.x * cta_step;
+    Weight cw = load_weight(t);
+    t = active_from(t, cw);
+    Trials<VEC> trials(y, n_warps);
+    Span<VEC> cur = trials.first(y, t);
+    ids.request(cur, 0, lane);
+    bool lost = false;
+    uint32_t unused_max = 0;  // ids outside the catalogue were reported by the forward
+    int folds = 0;            // batches since the partials were folded
+    while (t < y.n_trials && !lost) {
+        const bool mid_l = cw.code == 1 && cw.g != 0.0f;
+        const float gt = cw.g;
+        Weight nw = load_weight(t + n_warps);
+        // the trial's weights: W[s] = sum of g_j a_j over the layers j < 4 in
+        // s, W[16 + s] over the layers 4 + j, in increasing j
         {
-            if (lane == 0) s_w[0] = 0.0f;
+            const float mine = mid_l ? gt : 0.0f;
+            float acc = 0.0f;
+#pragma unroll
+            for (int b = 0; b < (LT < 4 ? LT : 4); ++b) {
+                const float gb = __shfl_sync(kFull, mine, b + (LT > 4 ? (lane & 16) >> 2 : 0));
+                acc += (lane >> b) & 1 ? gb : 0.0f;
+            }
+            s_w[lane] = LT > 4 || lane < 16 ? acc : 0.0f;
             __syncwarp();
-#pragma unroll
-            for (int b = 0; b < LT; ++b) {
-                const float gb = __shfl_sync(FULL, mid_l ? gt : 0.0f, b);
-                for (int s = lane; s < (1 << b); s += 32) s_w[s + (1 << b)] = s_w[s] + gb;
-                __syncwarp();
-            }
         }
-        uint64_t cnt_mid = 0, cnt_cap = 0;
-        float part[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) part[k] = 0.0f;
-        // lane j adds the warp's counts of layer j, scaled by g_j, and clears
-        // them; the products are exact (FMA residual), the sums compensated
+        uint32_t mid0 = 0, mid1 = 0, cap0 = 0, cap1 = 0;  // packed layer counters
         auto flush_counts = [&]() {
-#pragma unroll
-            for (int j = 0; j < LT; ++j) {
-                const uint32_t cm = __reduce_add_sync(FULL, (uint32_t)(cnt_mid >> (8 * j)) & 0xffu);
-                const uint32_t cc = __reduce_add_sync(FULL, (uint32_t)(cnt_cap >> (8 * j)) & 0xffu);
-                if (lane == j && mid_l) {
-                    const float pm = gt * (float)cm, pc = gt * (float)cc;  // counts < 2^24: exact in FP32
-                    two_sum_add(or_h, or_l, -pm);
-                    or_l -= __fmaf_rn(gt, (float)cm, -pm);
-                    two_sum_add(ol_h, ol_l, pc);
-                    ol_l += __fmaf_rn(gt, (float)cc, -pc);
-                }
+            // two layers per reduction, in 16-bit fields
+            const uint32_t e0 = __reduce_add_sync(kFull, mid0 & 0x00ff00ffu);
+            const uint32_t o0 = LT > 1 ? __reduce_add_sync(kFull, (mid0 >> 8) & 0x00ff00ffu) : 0u;
+            const uint32_t e1 = LT > 4 ? __reduce_add_sync(kFull, mid1 & 0x00ff00ffu) : 0u;
+            const uint32_t o1 = LT > 4 ? __reduce_add_sync(kFull, (mid1 >> 8) & 0x00ff00ffu) : 0u;
+            const uint32_t sm = (lane & 4) ? ((lane & 1) ? o1 : e1) : ((lane & 1) ? o0 : e0);
+            const uint32_t cm = (lane & 2) ? sm >> 16 : sm & 0xffffu;
+            uint32_t cc = 0;
+            if (__any_sync(kFull, (cap0 | cap1) != 0u)) {
+                const uint32_t f0 = __reduce_add_sync(kFull, cap0 & 0x00ff00ffu);
+                const uint32_t p0 = __reduce_add_sync(kFull, (cap0 >> 8) & 0x00ff00ffu);
+                const uint32_t f1 = LT > 4 ? __reduce_add_sync(kFull, cap1 & 0x00ff00ffu) : 0u;
+                const uint32_t p1 = LT > 4 ? __reduce_add_sync(kFull, (cap1 >> 8) & 0x00ff00ffu) : 0u;
+                const uint32_t sc = (lane & 4) ? ((lane & 1) ? p1 : f1) : ((lane & 1) ? p0 : f0);
+                cc = (lane & 2) ? sc >> 16 : sc & 0xffffu;
             }
-            cnt_mid = 0;
-            cnt_cap = 0;
+            if (mid_l && lane < LT) {
+                // the products are exact (FMA residual; counts < 2^24), the sums compensated
+                const float pm = gt * (float)cm, pc = gt * (float)cc;
+                two_sum_add(or_h, or_l, -pm);
+                or_l -= __fmaf_rn(gt, (float)cm, -pm);
+                two_sum_add(ol_h, ol_l, pc);
+                ol_l += __fmaf_rn(gt, (float)cc, -pc);
+            }
+            mid0 = mid1 = cap0 = cap1 = 0;
         };
-        int64_t b, e;
-        bool bad_off;
-        trial_range(y, t, b, e, bad_off);
-        int qn = 0;        // warp-uniform, < 32 between chunks
-        int batches = 0;   // batches since the counters were cleared (each lane's byte counters < 256)
-        // ids of a chunk of 32 * E events from c0 (the sentinel C past the end)
-        auto load_ids = [&](int64_t c0, uint32_t (&v)[E]) {
-            if constexpr (VEC) {
-#pragma unroll
-                for (int h = 0; h < E / 4; ++h) {
-                    const int64_t d = c0 + 128 * h + 4 * lane;
-                    int4 w4 = make_int4(-1, -1, -1, -1);
-                    if (d < e) w4 = __ldcs(reinterpret_cast<const int4*>(y.ids + d));  // e and d are multiples of 4
-                    v[4 * h + 0] = (uint32_t)w4.x;
-                    v[4 * h + 1] = (uint32_t)w4.y;
-                    v[4 * h + 2] = (uint32_t)w4.z;
-                    v[4 * h + 3] = (uint32_t)w4.w;
+        auto weight_of = [&](uint32_t set) { return s_w[set & 15u] + s_w[16 + ((set >> 4) & 15u)]; };
+        // one batch: the lane's event (all zero: none)
+        auto add_record = [&](const AdjRecord& r, uint32_t id) {
+            mid0 += r.mid_lo;
+            mid1 += r.mid_hi;
+            const uint32_t kk = (r.meta >> 20) & 255u, n = (r.meta >> 15) & 7u;
+            if (__any_sync(kFull, kk != 0u)) {
+                cap0 += spread4(kk);
+                cap1 += spread4(kk >> 4);
+            }
+            if (n != kOverflow) {
+                float* c0 = part + 32 * (r.meta & 31u);
+                *c0 = __fmaf_rn(r.loss[0], weight_of(r.sets), *c0);  // no column: 0 * W[0]
+                if (n > 1) {
+                    float* c1 = part + 32 * ((r.meta >> 5) & 31u);
+                    *c1 = __fmaf_rn(r.loss[1], weight_of(r.sets >> 8), *c1);
+                }
+                if (n > 2) {
+                    float* c2 = part + 32 * ((r.meta >> 10) & 31u);
+                    *c2 = __fmaf_rn(r.loss[2], weight_of(r.sets >> 16), *c2);
                 }
             } else {
-#pragma unroll
-                for (int k = 0; k < E; ++k) {
-                    const int64_t d = c0 + 32 * k + lane;
-                    v[k] = d < e ? (uint32_t)ld_stream(y.ids + d) : 0xffffffffu;
+                const float* row = g.table + (size_t)id * NP;
+                for (uint32_t u = r.u; u; u &= u - 1) {
+                    const int k = __ffs(u) - 1;
+                    part[32 * k] = __fmaf_rn(row[k], weight_of(r.sets & s_cover[k]), part[32 * k]);
                 }
             }
         };
-        uint32_t pre[E];
-        if (b < e) load_ids(b, pre);
-        for (int64_t c0 = b; c0 < e; c0 += 32 * E) {
-            uint32_t uid[E];
+        AdjRecord rec{};
+        uint32_t rec_id = 0;
+        int batches = 0;              // since the counters were cleared (each lane's byte counters < 256)
+        int64_t tn = t;
+        Span<VEC> nxt;
+        auto next_trial = [&]() {
+            tn = active_from(t + n_warps, nw);
+            nxt = trials.first(y, tn);
+            ids.request(nxt, 0, lane);
+        };
+        if (cur.n == 0) next_trial();
+        for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
+            uint32_t id[E];
+            if (!ids.take(cur, c0, lane, id)) {
+                lost = true;
+                break;
+            }
+            clean_ids<E>(cur, c0, lane, C, none, id, unused_max);
+            if (c0 + 32 * E >= cur.n) next_trial();
+            else ids.request(cur, c0 + 32 * E, lane);
+            uint32_t nz[E];
 #pragma unroll
-            for (int k = 0; k < E; ++k) uid[k] = min(pre[k], (uint32_t)y.catalogue);
-            // request the trial's next chunk before this one is processed
-            if (c0 + 32 * E < e) load_ids(c0 + 32 * E, pre);
+            for (int k = 0; k < E; ++k) nz[k] = bit_of<FOLD>(s_bits, gbits, id[k], S);
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-                uint32_t wi = uid[k] >> 5;
-                uint32_t w;
-                if constexpr (FOLD) {
-                    wi = wi >= (uint32_t)smem_words ? wi - (uint32_t)smem_words : wi;
-                    w = s_bits[wi];
-                } else {
-                    w = wi < (uint32_t)smem_words ? s_bits[wi] : ld_bits_global(gbits + wi);
-                }
-                const bool nz = (w >> (uid[k] & 31)) & 1u;
-                const unsigned mm = __ballot_sync(FULL, nz);
-                if (nz) q[qn + __popc(mm & lt_mask)] = (int32_t)uid[k];
-                qn += __popc(mm);
-                if (qn >= 32) {
+                ring.push(id[k], nz[k], lt_mask);
+                if ((k & 1) && ring.size() >= 32) {  // at most 31 + 64 queued: two batches
+#pragma unroll 1
+                    do {
+                        const uint32_t mine = ring.take32(lane);
+                        add_record(rec, rec_id);
+                        rec = ld_record(records + mine);
+                        rec_id = mine;
+                        ++folds;
+                        if (++batches == 250) {
+                            flush_counts();
+                            batches = 0;
+                        }
+                    } while (ring.size() >= 32);
                     __syncwarp();
-                    const int32_t mine = q[lane];
-                    const int32_t carry = q[32 + lane];
-                    __syncwarp();
-                    q[lane] = carry;  // entries 32 .. qn-1 move to the front
-                    qn -= 32;
-                    eval_event<NP, LT>(g, masks, (uint32_t)mine, (uint32_t)y.catalogue - 1u, s_spread, s_w, s_col, cnt_mid, cnt_cap, part);
-                    if (++batches == 255) {
-                        flush_counts();
-                        batches = 0;
+                    if (folds >= kFold) {
+                        fold_columns();
+                        folds = 0;
                     }
-                    __syncwarp();
                 }
             }
         }
         __syncwarp();
-        if (lane < qn) eval_event<NP, LT>(g, masks, (uint32_t)q[lane], (uint32_t)y.catalogue - 1u, s_spread, s_w, s_col, cnt_mid, cnt_cap, part);
+        add_record(rec, rec_id);
+        rec = AdjRecord{};
+        if (lane < ring.size()) {
+            rec_id = ring.peek(lane);
+            rec = ld_record(records + rec_id);
+        }
+        ring.head = ring.tail;
+        add_record(rec, rec_id);
+        folds += 1;
         __syncwarp();
         flush_counts();
-        // the trial's column partials summed across the warp by recursive
-        // halving (31 shuffles for all columns): at distance o a lane keeps
-        // the half of its columns selected by bit o of its index and adds
-        // the partner's copy of that half; lane k ends with column k
-        {
-            float v[32];
-#pragma unroll
-            for (int k = 0; k < 32; ++k) v[k] = k < NP ? part[k] : 0.0f;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const bool upper = (lane & o) != 0;
-#pragma unroll
-                for (int i = 0; i < o; ++i) {
-                    const float keep = upper ? v[i + o] : v[i];
-                    const float send = upper ? v[i] : v[i + o];
-                    v[i] = keep + __shfl_xor_sync(FULL, send, o);
-                }
-            }
-            if (lane < NP) two_sum_add(col_h, col_l, v[0]);
-        }
-        __syncwarp();  // the weight table is rebuilt by the next trial
+        if (lost) break;
+        t = tn;
+        cur = nxt;
+        cw = nw;
     }
+    fold_columns();
+    if (lost) {
+        ids.phase ^= 1u;
+        ids.wait();  // the copy in flight may still come: shared memory stays until then
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
+    }
+    __syncthreads();
+    double* s_red = reinterpret_cast<double*>(s_part);  // [NWARP][W]
     // the lane values in FP64, reduced warp -> CTA in a fixed order
 #pragma unroll
     for (int i = 0; i < W; ++i) {
@@ -385,13 +516,13 @@ __global__ void __launch_bounds__(kAgThreadsFor<NP>, 1) adjoint_pass_kernel(cons
         } else {
             v = lane == i - 4 * LT ? (double)col_h + (double)col_l : 0.0;
         }
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
         if (lane == 0) s_red[wib * W + i] = v;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < W; i += blockDim.x) {
         double s = 0.0;
-        for (int wv = 0; wv < kAgWarps; ++wv) s += s_red[wv * W + i];
+        for (int wv = 0; wv < NWARP; ++wv) s += s_red[wv * W + i];
         partial[(size_t)blockIdx.x * W + i] = s;
     }
 }
@@ -403,92 +534,104 @@ struct GroupIndex {
     int32_t n_elt, n_layers;
 };
 
-// Sum the CTA partials of one group in block order and add them into the
-// outputs: each layer belongs to one group; an ELT's multiplier gradient sums
-// over the groups that hold it, in group order (groups run in order on one
-// stream).
-__global__ void group_scatter_kernel(const double* __restrict__ partial, int nblk, int lt, int np,
-                                     const GroupIndex gix, double* __restrict__ grad_terms,
-                                     double* __restrict__ grad_mult) {
-    const int w = 4 * lt + np;
-    const int i = threadIdx.x;
-    if (i >= w) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * w + i];
-    if (i < 4 * lt) {
-        const int c = i / lt, j = i % lt;
-        if (j < gix.n_layers) grad_terms[(size_t)gix.layer[j] * 4 + c] = s;
-    } else {
-        const int k = i - 4 * lt;
-        if (k < gix.n_elt) grad_mult[gix.elt[k]] += s;
+// Sum the CTA partials of one group (a warp per value, each lane every 32nd
+// CTA, then the lanes: a fixed order) and add them into the outputs: each
+// layer belongs to one group; an ELT's multiplier gradient sums over the groups
+// that hold it, in group order (groups run in order on one stream).
+__global__ void __launch_bounds__(1024) group_scatter_kernel(const double* __restrict__ partial, int nblk, int lt,
+                                                             int np, const GroupIndex gix,
+                                                             double* __restrict__ grad_terms,
+                                                             double* __restrict__ grad_mult) {
+    const int w = 4 * lt + np, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < w; i += blockDim.x >> 5) {
+        double s = 0.0;
+        for (int b = lane; b < nblk; b += 32) s += partial[(size_t)b * w + i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
+        if (lane) continue;
+        if (i < 4 * lt) {
+            const int c = i / lt, j = i % lt;
+            if (j < gix.n_layers) grad_terms[(size_t)gix.layer[j] * 4 + c] = s;
+        } else {
+            const int k = i - 4 * lt;
+            if (k < gix.n_elt) grad_mult[gix.elt[k]] += s;
+        }
     }
 }
 
 struct Scratch {
-    uint2* masks;     // [C + 1]
-    uint32_t* bits;   // zero-padded to whole 16-byte groups, bits 0 .. C
-    double* partial;  // [num_sms][4 * 8 + 32]
+    AdjRecord* records;  // [C]
+    uint32_t* bits;      // zero-padded to whole 16-byte groups, bits 0 .. C
+    double* partial;     // [num_sms][4 * 8 + 32]
+    uint8_t* col;        // the group's column of each pool ELT (NULL without the CSR)
 };
 
 template <int NP, int LT>
-cudaError_t launch_one(const GroupArgs& g, const GroupIndex& gix, const YetArgs& y, const uint8_t* branch,
-                       const double* gw, const Scratch& sc, int num_sms, double* grad_terms, double* grad_mult,
-                       cudaStream_t s) {
+cudaError_t launch_one(const art_portfolio* p, const GroupArgs& g, const GroupIndex& gix, const YetArgs& y,
+                       const uint8_t* branch, const double* gw, const Scratch& sc, double* grad_terms,
+                       double* grad_mult, cudaStream_t s) {
     const int32_t C = y.catalogue;
-    const int32_t words_w = (int32_t)(((int64_t)C + 31) / 32);  // words the mask kernel writes
-    adj_masks_kernel<NP, LT><<<(unsigned)(((int64_t)words_w * 32 + 255) / 256), 256, 0, s>>>(g, C, words_w, sc.masks,
-                                                                                            sc.bits);
+    const int32_t words_w = (int32_t)(((int64_t)C + 31) / 32);  // words the record kernel writes
+    adj_records_kernel<NP, LT><<<(unsigned)(((int64_t)words_w * 32 + 255) / 256), 256, 0, s>>>(
+        g, C, words_w, sc.col ? p->sp_ptr : nullptr, reinterpret_cast<const SparseEntry*>(p->sp_entries), sc.col,
+        sc.records, sc.bits);
     cudaError_t e = cudaGetLastError();
     if (e || y.n_trials == 0) return e;
     int dev = 0, max_optin = 0;
     if ((e = cudaGetDevice(&dev))) return e;
     if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
-    constexpr int W = 4 * LT + NP;
-    constexpr int kAgWarps = kAgThreadsFor<NP> / 32;
-    const int fixed = 4 * (512 + 2 * kAgWarps * W + 32 + kAgWarps * (1 << LT) + kAgWarps * kAgQueue);
+    constexpr int NWARP = kAgWarpsFor<NP>;
+    const int fixed = 256 + 16 + 4 * (NWARP * (32 * kAgIds + NP * 32 + 32 + (int)kRing) + 32);
     const int words = (C >> 5) + 1;  // bits 0 .. C (C: the sentinel)
     const int smem_words = std::max(4, std::min((words + 3) & ~3, (max_optin - fixed) / 4) & ~3);
     const int smem = fixed + 4 * smem_words;
     const bool fold = words <= 2 * smem_words;
-    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
+    const bool vec = !y.by_id && !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
     auto kern = vec ? (fold ? adjoint_pass_kernel<NP, LT, true, true> : adjoint_pass_kernel<NP, LT, true, false>)
                     : (fold ? adjoint_pass_kernel<NP, LT, false, true> : adjoint_pass_kernel<NP, LT, false, false>);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
-    const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms, (y.n_trials + kAgWarps - 1) / kAgWarps));
-    kern<<<nblk, kAgThreadsFor<NP>, smem, s>>>(g, y, sc.masks, sc.bits, smem_words, branch, gw, sc.partial);
+    // a CTA's warps take neighbouring trials (they share the sectors of the
+    // branch codes and weights); few trials are spread over the SMs instead
+    const bool many = y.n_trials >= (int64_t)p->num_sms * NWARP;
+    const int64_t nblk = many ? p->num_sms : std::max<int64_t>(1, std::min<int64_t>(p->num_sms, y.n_trials));
+    kern<<<(unsigned)nblk, 32 * NWARP, smem, s>>>(g, y, sc.records, sc.bits, smem_words, many ? 1 : nblk,
+                                                  many ? NWARP : 1, branch, gw, sc.partial, p->d_flags);
     if ((e = cudaGetLastError())) return e;
-    group_scatter_kernel<<<1, 128, 0, s>>>(sc.partial, nblk, LT, NP, gix, grad_terms, grad_mult);
+    group_scatter_kernel<<<1, 1024, 0, s>>>(sc.partial, (int)nblk, LT, NP, gix, grad_terms, grad_mult);
     return cudaGetLastError();
 }
 
 template <int NP>
-cudaError_t launch_lt(const GroupArgs& g, const GroupIndex& gix, const YetArgs& y, const uint8_t* branch,
-                      const double* gw, const Scratch& sc, int num_sms, double* gt, double* gm, cudaStream_t s) {
-    if (g.n_layers <= 1) return launch_one<NP, 1>(g, gix, y, branch, gw, sc, num_sms, gt, gm, s);
-    if (g.n_layers <= 2) return launch_one<NP, 2>(g, gix, y, branch, gw, sc, num_sms, gt, gm, s);
-    if (g.n_layers <= 4) return launch_one<NP, 4>(g, gix, y, branch, gw, sc, num_sms, gt, gm, s);
-    return launch_one<NP, 8>(g, gix, y, branch, gw, sc, num_sms, gt, gm, s);
+cudaError_t launch_lt(const art_portfolio* p, const GroupArgs& g, const GroupIndex& gix, const YetArgs& y,
+                      const uint8_t* branch, const double* gw, const Scratch& sc, double* gt, double* gm,
+                      cudaStream_t s) {
+    if (g.n_layers <= 1) return launch_one<NP, 1>(p, g, gix, y, branch, gw, sc, gt, gm, s);
+    if (g.n_layers <= 2) return launch_one<NP, 2>(p, g, gix, y, branch, gw, sc, gt, gm, s);
+    if (g.n_layers <= 4) return launch_one<NP, 4>(p, g, gix, y, branch, gw, sc, gt, gm, s);
+    return launch_one<NP, 8>(p, g, gix, y, branch, gw, sc, gt, gm, s);
 }
 
 }  // namespace
 
-cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& y, const uint8_t* branch, const double* g,
+cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& yet, const uint8_t* branch, const double* g,
                                   double* grad_terms, double* grad_mult, cudaStream_t s) {
+    YetArgs y = yet;
+    y.by_id = !ids_on_device(y.ids);
     const size_t C = (size_t)p->catalogue;
-    const size_t mask_bytes = sizeof(uint2) * (C + 1);
+    const size_t rec_bytes = sizeof(AdjRecord) * C;
     const size_t bit_bytes = 16 * ((C / 32 + 1 + 3) / 4);
     const size_t part_bytes = sizeof(double) * (size_t)p->num_sms * (4 * kMaxGroupLayers + kMaxLayerElts);
-    const size_t a1 = (mask_bytes + 255) & ~(size_t)255, a2 = (bit_bytes + 255) & ~(size_t)255;
+    const size_t a1 = (rec_bytes + 255) & ~(size_t)255, a2 = (bit_bytes + 255) & ~(size_t)255;
     char* w = nullptr;
     cudaError_t err = scratch_alloc((void**)&w, a1 + a2 + part_bytes, s);
     if (err) return err;
-    Scratch sc{reinterpret_cast<uint2*>(w), reinterpret_cast<uint32_t*>(w + a1), reinterpret_cast<double*>(w + a1 + a2)};
+    Scratch sc{reinterpret_cast<AdjRecord*>(w), reinterpret_cast<uint32_t*>(w + a1),
+               reinterpret_cast<double*>(w + a1 + a2), nullptr};
     do {
         if ((err = cudaMemsetAsync(grad_terms, 0, sizeof(double) * 4 * p->n_layers, s))) break;
         if ((err = cudaMemsetAsync(grad_mult, 0, sizeof(double) * p->n_elt, s))) break;
         if (y.n_trials == 0) break;
-        // the sentinel row and the padding words stay zero for every group
-        if ((err = cudaMemsetAsync(w, 0, a1 + a2, s))) break;
+        // the bitmap's padding words stay zero for every group
+        if ((err = cudaMemsetAsync(sc.bits, 0, a2, s))) break;
         for (size_t gi = 0; gi < p->groups.size() && !err; ++gi) {
             const GroupArgs& ga = p->groups[gi];
             GroupIndex gix{};
@@ -496,15 +639,15 @@ cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& y, const uint
             gix.n_layers = (int32_t)p->group_layers[gi].size();
             for (int k = 0; k < gix.n_elt; ++k) gix.elt[k] = p->group_elts[gi][k];
             for (int j = 0; j < gix.n_layers; ++j) gix.layer[j] = p->group_layers[gi][j];
-            const int ns = p->num_sms;
+            sc.col = p->d_group_col ? p->d_group_col + gi * (size_t)p->pool_np : nullptr;
             double* gt = grad_terms;
             double* gm = grad_mult;
             switch (p->group_np[gi]) {
-                case 4: err = launch_lt<4>(ga, gix, y, branch, g, sc, ns, gt, gm, s); break;
-                case 8: err = launch_lt<8>(ga, gix, y, branch, g, sc, ns, gt, gm, s); break;
-                case 16: err = launch_lt<16>(ga, gix, y, branch, g, sc, ns, gt, gm, s); break;
-                case 24: err = launch_lt<24>(ga, gix, y, branch, g, sc, ns, gt, gm, s); break;
-                case 32: err = launch_lt<32>(ga, gix, y, branch, g, sc, ns, gt, gm, s); break;
+                case 4: err = launch_lt<4>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
+                case 8: err = launch_lt<8>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
+                case 16: err = launch_lt<16>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
+                case 24: err = launch_lt<24>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
+                case 32: err = launch_lt<32>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
                 default: err = cudaErrorInvalidValue;
             }
         }

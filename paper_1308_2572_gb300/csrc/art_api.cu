@@ -516,6 +516,14 @@ cudaError_t build_groups(art_portfolio* p, const float* losses, cudaStream_t str
     cudaFree(d_el);
     if (e) return e;
     if (e2) return e2;
+    if (p->sp_ptr) {  // the adjoint's records come from the CSR
+        std::vector<uint8_t> col(ng * p->pool_np, 255);
+        for (size_t gi = 0; gi < ng; ++gi)
+            for (size_t k = 0; k < p->group_elts[gi].size(); ++k)
+                col[gi * p->pool_np + p->group_elts[gi][k]] = (uint8_t)k;
+        if ((e = cudaMalloc(&p->d_group_col, col.size()))) return e;
+        if ((e = cudaMemcpy(p->d_group_col, col.data(), col.size(), cudaMemcpyHostToDevice))) return e;
+    }
     refresh_group_terms(p);
     return cudaSuccess;
 }
@@ -540,6 +548,7 @@ void free_portfolio(art_portfolio* p) {
     for (float* t : p->layer_tab) cudaFree(t);
     for (float* t : p->group_tab) cudaFree(t);
     for (uint32_t* b : p->group_bitmap) cudaFree(b);
+    cudaFree(p->d_group_col);
     for (float* t : p->og_occ) cudaFree(t);
     for (uint32_t* b : p->og_bits) cudaFree(b);
     cudaFree(p->d_lbuild);

@@ -67,6 +67,7 @@ struct YetArgs {
     int64_t n_trials;
     int32_t k;            // events per trial when dense
     int32_t catalogue;
+    bool by_id = false;   // ids to be read one by one (not in device memory: no bulk copies)
 };
 
 __device__ __forceinline__ void trial_range(const YetArgs& y, int64_t t, int64_t& b, int64_t& e, bool& bad) {
@@ -341,6 +342,7 @@ struct art_portfolio {
     std::vector<std::vector<int32_t>> group_layers; // layer ids per group
     std::vector<float*> group_tab;
     std::vector<uint32_t*> group_bitmap;
+    uint8_t* d_group_col = nullptr;             // [n_groups][pool_np]: the group's column of an ELT (255: none)
 
     // skip variant (needs ART_LAYOUT_LAYER): occurrence groups and their
     // per-call occurrence-loss tables and bitmaps

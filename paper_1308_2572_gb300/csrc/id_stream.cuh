@@ -39,19 +39,11 @@ struct Span {
 // The trials of one warp, in its order: t, t + n_warps, ...
 template <bool VEC>
 struct Trials {
-    int64_t lo, hi, stride;  // reads of [lo, hi) stay in the id array (for a CSR every index between the
-                             // first and the last offset lies in some trial); VEC: ids from trial to trial
-    uint32_t mis;            // ids between the 16-byte boundary before y.ids and y.ids
-    bool bad = false;        // a decreasing pair of offsets was seen
+    int64_t stride = 0;  // VEC: ids from trial to trial
+    bool bad = false;    // a decreasing pair of offsets was seen
 
     __device__ __forceinline__ Trials(const YetArgs& y, int64_t n_warps) {
-        if constexpr (VEC) {
-            stride = n_warps * (int64_t)y.k;
-        } else {
-            lo = y.off ? y.off[0] : 0;
-            hi = y.off ? y.off[y.n_trials] : y.n_trials * (int64_t)y.k;
-            mis = (uint32_t)(reinterpret_cast<uintptr_t>(y.ids) >> 2) & 3u;
-        }
+        if constexpr (VEC) stride = n_warps * (int64_t)y.k;
     }
     __device__ __forceinline__ Span<VEC> first(const YetArgs& y, int64_t t) {
         Span<VEC> s;
@@ -64,11 +56,17 @@ struct Trials {
             bool bo;
             trial_range(y, t, b, e, bo);
             bad |= bo;
+            // ids between the 16-byte boundary before y.ids and y.ids
+            const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(y.ids) >> 2) & 3u;
+            // reads of [lo, hi) stay in the id array (for a CSR every index
+            // between the first and the last offset lies in some trial)
+            const int64_t lo = y.off ? y.off[0] : 0;
+            const int64_t hi = y.off ? y.off[y.n_trials] : y.n_trials * (int64_t)y.k;
             s.head_ = ((uint32_t)b + mis) & 3u;
             const int64_t a = b - s.head_;
             s.p = y.ids + a;
             s.n = e > b ? (uint32_t)(e - a) : 0u;
-            s.edge_ = a < lo || a + (int64_t)((s.n + 3u) & ~3u) > hi;
+            s.edge_ = y.by_id || a < lo || a + (int64_t)((s.n + 3u) & ~3u) > hi;
         }
         return s;
     }
@@ -93,13 +91,11 @@ template <int E>
 struct IdStream {
     uint32_t bar, buf;  // shared-memory addresses of the warp's barrier and buffer
     uint32_t phase;
-    uint64_t policy;    // evict-first in L2: the stream must not push out X
 
     __device__ __forceinline__ void init(void* bars, void* bufs, int wib, int lane) {
         bar = (uint32_t)__cvta_generic_to_shared(bars) + 8u * wib;
         buf = (uint32_t)__cvta_generic_to_shared(bufs) + 128u * E * wib;
         phase = 0;
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
         if (lane == 0) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -112,6 +108,8 @@ struct IdStream {
     __device__ __forceinline__ void request(const Span<VEC>& s, uint32_t c0, int lane) {
         if (lane == 0 && c0 < s.n && !s.edge()) {
             const uint32_t bytes = 4u * min(32u * E, ((s.n + 3u) & ~3u) - c0);
+            uint64_t policy;  // evict-first in L2: the stream must not push out X
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
             asm volatile(
                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(buf),
@@ -212,8 +210,9 @@ __device__ __forceinline__ uint32_t no_event(uint32_t C, uint32_t S) {
 
 // The event's bit: word w of shared memory holds bitmap words w and w + S
 // OR-ed together (FOLD: a superset test, a fold-only hit gathers zeros).
+// Returned as bit 0 of a word (its other bits are other events').
 template <bool FOLD>
-__device__ __forceinline__ bool bit_of(const uint32_t* s_bits, const uint32_t* gbits, uint32_t id, uint32_t S) {
+__device__ __forceinline__ uint32_t bit_of(const uint32_t* s_bits, const uint32_t* gbits, uint32_t id, uint32_t S) {
     uint32_t wi = id >> 5, w;
     if constexpr (FOLD) {
         wi = __viaddmin_u32(wi, 0u - S, wi);  // wi - S wraps when wi < S
@@ -221,7 +220,7 @@ __device__ __forceinline__ bool bit_of(const uint32_t* s_bits, const uint32_t* g
     } else {
         w = wi < S ? s_bits[wi] : ld_bits(gbits + wi);
     }
-    return __funnelshift_r(w, 0u, id) & 1u;
+    return __funnelshift_r(w, 0u, id);
 }
 
 template <bool FOLD>
@@ -241,6 +240,50 @@ __device__ __forceinline__ void stage_bits(uint32_t* s_bits, const uint32_t* gbi
     }
     if (threadIdx.x == 0) s_bits[smem_words] = 0u;  // no_event's word
 }
+
+// A warp's ring of queued ids in shared memory. Stores are predicated rather
+// than branched over (a branch region per slot of 32 events costs the skip
+// pass a third of its instructions on the 8-layer groups).
+constexpr uint32_t kRing = 128;  // entries: up to 31 left over and two slots of 32
+
+struct IdRing {
+    uint32_t base;            // shared-memory address, a multiple of the ring's size
+    uint32_t head = 0, tail = 0;  // warp-uniform positions in bytes
+
+    __device__ __forceinline__ explicit IdRing(const uint32_t* ring) : base((uint32_t)__cvta_generic_to_shared(ring)) {}
+    // Queue the ids of the lanes whose word has bit 0 set. One block, so that
+    // one predicate serves the vote and the store.
+    __device__ __forceinline__ void push(uint32_t id, uint32_t word, unsigned lt_mask) {
+        asm volatile(
+            "{\n.reg .pred p;\n.reg .b32 m, a;\n"
+            "and.b32 a, %2, 1;\nsetp.ne.u32 p, a, 0;\n"
+            "vote.sync.ballot.b32 m, p, 0xffffffff;\n"
+            "and.b32 a, m, %3;\npopc.b32 a, a;\nmad.lo.u32 a, a, 4, %0;\n"
+            "and.b32 a, a, %5;\nor.b32 a, a, %4;\n"
+            "@p st.shared.u32 [a], %1;\n"
+            "popc.b32 m, m;\nmad.lo.u32 %0, m, 4, %0;\n}"
+            : "+r"(tail)
+            : "r"(id), "r"(word), "r"(lt_mask), "r"(base), "n"(4u * kRing - 1u)
+            : "memory");
+    }
+    __device__ __forceinline__ uint32_t size() const { return (tail - head) / 4u; }
+    // The entry `lane` places after the head.
+    __device__ __forceinline__ uint32_t peek(int lane) const {
+        uint32_t v;
+        asm volatile("ld.shared.u32 %0, [%1];"
+                     : "=r"(v)
+                     : "r"(base | ((head + 4u * lane) & (4u * kRing - 1u)))
+                     : "memory");
+        return v;
+    }
+    // 32 entries, one per lane.
+    __device__ __forceinline__ uint32_t take32(int lane) {
+        __syncwarp();
+        const uint32_t v = peek(lane);
+        head += 128u;
+        return v;
+    }
+};
 
 }  // namespace
 

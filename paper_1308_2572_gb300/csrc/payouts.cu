@@ -205,9 +205,11 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
             uint32_t o[E];
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-                const bool nz = bit_of<FOLD>(s_bits, a.bits, id[k], S);
-                o[k] = 0;
-                if (nz) asm("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(o[k]) : "l"(a.x + id[k]));
+                // bit 0 clear: 0, without a branch
+                asm("{\n.reg .pred p;\n.reg .b32 w;\nand.b32 w, %2, 1;\nsetp.ne.u32 p, w, 0;\nmov.u32 %0, 0;\n"
+                    "@p ld.global.nc.L1::no_allocate.u32 %0, [%1];\n}"
+                    : "=r"(o[k])
+                    : "l"(a.x + id[k]), "r"(bit_of<FOLD>(s_bits, a.bits, id[k], S)));
             }
 #pragma unroll
             for (int h = 0; h < E / 4; ++h) {

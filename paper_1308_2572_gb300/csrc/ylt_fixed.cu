@@ -35,10 +35,13 @@ namespace art {
 
 namespace {
 
-constexpr int kFxThreads = 1024;
-constexpr int kFxWarps = kFxThreads / 32;
+// Warps per CTA. The 8-layer rows with ragged trials need more than the 64
+// registers a thread of 32 warps gets; a spilled value costs L2's latency per
+// chunk (the gathers leave L1 no room for it): 16 of c2's layers, 250,000
+// trials, 3.05 ms with 32 warps, 1.71 with 24.
+template <int LP, bool VEC>
+constexpr int kFxWarpsFor = LP == 8 && !VEC ? 24 : 32;
 constexpr int kFxIds = 8;     // ids per lane and chunk: 1 KB in flight per warp, 32 KB per SM
-constexpr int kFxQueue = 64;  // per-warp ring of queued ids (wide groups)
 // Row id of X: LP (1, 2, 4 or 8) whole numbers in one load, not kept in L1.
 template <int LP>
 __device__ __forceinline__ void ld_units(const float* x, uint32_t id, uint32_t (&o)[LP]) {
@@ -58,6 +61,24 @@ __device__ __forceinline__ void ld_units(const float* x, uint32_t id, uint32_t (
     }
 }
 
+// The same where the word's bit 0 is set, zeros elsewhere, without a branch
+// (narrow rows).
+template <int LP>
+__device__ __forceinline__ void ld_units_if(const float* x, uint32_t id, uint32_t word, uint32_t (&o)[LP]) {
+    static_assert(LP <= 2, "narrow rows");
+    const float* p = x + (size_t)id * LP;
+    if constexpr (LP == 1) {
+        asm("{\n.reg .pred p;\n.reg .b32 a;\nand.b32 a, %2, 1;\nsetp.ne.u32 p, a, 0;\nmov.u32 %0, 0;\n@p ld.global.nc.L1::no_allocate.u32 %0, [%1];\n}"
+            : "=r"(o[0])
+            : "l"(p), "r"(word));
+    } else {
+        asm("{\n.reg .pred p;\n.reg .b32 a;\nand.b32 a, %3, 1;\nsetp.ne.u32 p, a, 0;\nmov.u32 %0, 0;\nmov.u32 %1, 0;\n"
+            "@p ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];\n}"
+            : "=r"(o[0]), "=r"(o[1])
+            : "l"(p), "r"(word));
+    }
+}
+
 // The warp's total of a 64-bit count (valid in every lane). Entries are
 // below 2^32, so for trials shorter than 2^20 the lanes' counts stay below
 // 2^47: 20 low and 27 high bits, each summed in one 32-bit reduction.
@@ -70,6 +91,29 @@ __device__ __forceinline__ unsigned long long warp_total(unsigned long long v, b
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
+}
+
+// Lane j's share: the warp's total of acc[j] (j < LP).
+template <int LP>
+__device__ __forceinline__ unsigned long long lane_totals(const unsigned long long (&acc)[LP], int lane, bool is_short) {
+    if (is_short) {
+        uint32_t lo = 0, hi = 0;
+#pragma unroll
+        for (int j = 0; j < LP; ++j) {
+            const uint32_t l = __reduce_add_sync(kFull, (uint32_t)acc[j] & 0xfffffu);
+            const uint32_t h = __reduce_add_sync(kFull, (uint32_t)(acc[j] >> 20));
+            lo = lane == j ? l : lo;
+            hi = lane == j ? h : hi;
+        }
+        return ((unsigned long long)hi << 20) + lo;
+    }
+    unsigned long long mine = 0;
+#pragma unroll
+    for (int j = 0; j < LP; ++j) {
+        const unsigned long long v = warp_total(acc[j], false);
+        if (lane == j) mine = v;
+    }
+    return mine;
 }
 
 // True when every layer of the group has reached its aggregate cap.
@@ -88,15 +132,16 @@ __device__ __forceinline__ bool capped(const OccGroupArgs& g, const unsigned lon
 // set, 8 loads in flight. PRE entries are summed in 32 bits before the 64-bit
 // add (the host picks 4 when four of the largest entry fit).
 template <int LP, bool VEC, bool FOLD, int PRE>
-__global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGroupArgs g, const YetArgs y,
+__global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_narrow_kernel(const OccGroupArgs g, const YetArgs y,
                                                                     const int32_t smem_words, const bool early_exit,
                                                                     double* __restrict__ ylt,
                                                                     uint8_t* __restrict__ branch,
                                                                     int* __restrict__ flags) {
     constexpr int E = kFxIds;
-    extern __shared__ __align__(128) uint32_t s_dyn[];
-    uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
-    uint32_t* s_bits = s_ids + kFxWarps * 32 * E;
+    constexpr int NWARP = kFxWarpsFor<LP, VEC>;
+    extern __shared__ __align__(512) uint32_t s_dyn[];
+    uint32_t* s_ids = s_dyn + 64;                 // [NWARP][32 * E], after the warps' barriers
+    uint32_t* s_bits = s_ids + NWARP * 32 * E;
     const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     IdStream<E> ids;
@@ -105,7 +150,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGr
     __syncthreads();
     // neighbouring CTAs take neighbouring trials, so that few trials still
     // spread over every SM
-    const int64_t n_warps = (int64_t)gridDim.x * kFxWarps;
+    const int64_t n_warps = (int64_t)gridDim.x * NWARP;
     int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
     uint32_t max_id = 0;
     // results of up to 32 trials, lane s holding the s-th: the FP64 steps run
@@ -151,15 +196,13 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGr
             const bool last = c0 + 32 * E >= cur.n;
             if (last) ids.request(nxt, 0, lane);
             else ids.request(cur, c0 + 32 * E, lane);
-            bool nz[E];
+            uint32_t nz[E];
 #pragma unroll
             for (int k = 0; k < E; ++k) nz[k] = bit_of<FOLD>(s_bits, g.occ_bits, id[k], S);
             uint32_t o[E][LP];
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-#pragma unroll
-                for (int j = 0; j < LP; ++j) o[k][j] = 0;
-                if (nz[k]) ld_units<LP>(g.occ, id[k], o[k]);
+                ld_units_if<LP>(g.occ, id[k], nz[k], o[k]);
             }
 #pragma unroll
             for (int j = 0; j < LP; ++j)
@@ -210,25 +253,26 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_narrow_kernel(const OccGr
 // adds the row of the flush before, then requests this flush's, so a gather's
 // latency runs beside the next chunk's tests.
 template <int LP, bool VEC, bool FOLD>
-__global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_constant__ OccGroupArgs g, const YetArgs y,
+__global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_wide_kernel(const __grid_constant__ OccGroupArgs g, const YetArgs y,
                                                                   const int32_t smem_words, const bool early_exit,
                                                                   double* __restrict__ ylt,
                                                                   uint8_t* __restrict__ branch,
                                                                   int* __restrict__ flags) {
     constexpr int E = kFxIds;
-    extern __shared__ __align__(128) uint32_t s_dyn[];
-    uint32_t* s_ids = s_dyn + 64;                 // [kFxWarps][32 * E], after the warps' barriers
-    uint32_t* s_queue = s_ids + kFxWarps * 32 * E;
-    uint32_t* s_bits = s_queue + kFxWarps * kFxQueue;
+    constexpr int NWARP = kFxWarpsFor<LP, VEC>;
+    extern __shared__ __align__(512) uint32_t s_dyn[];
+    uint32_t* s_bars = s_dyn + NWARP * kRing;  // after the warps' rings
+    uint32_t* s_ids = s_bars + 64;                // [NWARP][32 * E]
+    uint32_t* s_bits = s_ids + NWARP * 32 * E;
     const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     IdStream<E> ids;
-    ids.init(s_dyn, s_ids, wib, lane);
+    ids.init(s_bars, s_ids, wib, lane);
+    IdRing ring(s_dyn + wib * kRing);
     stage_bits<FOLD>(s_bits, g.occ_bits, smem_words, (y.catalogue >> 5) + 1);
     __syncthreads();
-    uint32_t* q = s_queue + wib * kFxQueue;
     const unsigned lt_mask = (1u << lane) - 1u;
-    const int64_t n_warps = (int64_t)gridDim.x * kFxWarps;
+    const int64_t n_warps = (int64_t)gridDim.x * NWARP;
     int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
     uint32_t max_id = 0;
     Trials<VEC> trials(y, n_warps);
@@ -247,7 +291,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
         }
         const bool is_short = cur.n < (1u << 20);
         bool cap = false;
-        uint32_t head = 0, tail = 0;  // warp-uniform ring positions, tail - head < 32 between slots
         if (cur.n == 0) ids.request(nxt, 0, lane);
         for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
             uint32_t id[E];
@@ -259,22 +302,18 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
             const bool last = c0 + 32 * E >= cur.n;
             if (last) ids.request(nxt, 0, lane);
             else ids.request(cur, c0 + 32 * E, lane);
-            bool nz[E];
-#pragma unroll
-            for (int k = 0; k < E; ++k) nz[k] = bit_of<FOLD>(s_bits, g.occ_bits, id[k], S);
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-                const unsigned m = __ballot_sync(kFull, nz[k]);
-                if (nz[k]) q[(tail + __popc(m & lt_mask)) & (kFxQueue - 1)] = id[k];
-                tail += __popc(m);
-                if (tail - head >= 32) {
-                    __syncwarp();
-                    const uint32_t mine = q[(head + lane) & (kFxQueue - 1)];
-                    head += 32;
-                    __syncwarp();
+                ring.push(id[k], bit_of<FOLD>(s_bits, g.occ_bits, id[k], S), lt_mask);
+                if ((k & 1) && ring.size() >= 32) {  // at most 31 + 64 queued: two batches
+#pragma unroll 1
+                    do {
+                        const uint32_t mine = ring.take32(lane);
 #pragma unroll
-                    for (int j = 0; j < LP; ++j) acc[j] += o[j];
-                    ld_units<LP>(g.occ, mine, o);
+                        for (int j = 0; j < LP; ++j) acc[j] += o[j];
+                        ld_units<LP>(g.occ, mine, o);
+                    } while (ring.size() >= 32);
+                    __syncwarp();
                 }
             }
             if (early_exit) {
@@ -288,7 +327,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
                         lost = !cur.edge() && !ids.wait();
                         if (!lost) ids.request(nxt, 0, lane);
                     }
-                    head = tail;
+                    ring.head = ring.tail;
                     cap = true;
                     break;
                 }
@@ -297,18 +336,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) fixed_wide_kernel(const __grid_
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < LP; ++j) acc[j] += o[j];
-        if (head + lane < tail) {
-            ld_units<LP>(g.occ, q[(head + lane) & (kFxQueue - 1)], o);
+        if (lane < ring.size()) {
+            ld_units<LP>(g.occ, ring.peek(lane), o);
 #pragma unroll
             for (int j = 0; j < LP; ++j) acc[j] += o[j];
         }
+        ring.head = ring.tail;
         __syncwarp();
-        unsigned long long mine = 0;
-#pragma unroll
-        for (int j = 0; j < LP; ++j) {
-            const unsigned long long v = warp_total(acc[j], is_short);
-            if (lane == j) mine = v;
-        }
+        unsigned long long mine = lane_totals<LP>(acc, lane, is_short);
         if (lane < g.n_layers) {
             const double sum = (double)mine * g.unit[lane], ret = g.agg_ret[lane], lim = g.agg_lim[lane];
             const size_t wi = (size_t)g.layer[lane] * (size_t)y.n_trials + (size_t)t;
@@ -348,9 +383,12 @@ cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, 
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
-    // the warps' barriers (256 bytes), id buffers and queues, then the bitmap
+    // every trial starts and ends on a 16-byte boundary
+    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
+    // the warps' rings, barriers (256 bytes) and id buffers, then the bitmap
     // and its zero word
-    const int fixed_bytes = 256 + 16 + kFxWarps * (32 * kFxIds + (lp >= 4 ? kFxQueue : 0)) * 4;
+    const int warps = lp == 8 && !vec ? kFxWarpsFor<8, false> : kFxWarpsFor<8, true>;
+    const int fixed_bytes = 256 + 16 + warps * (32 * kFxIds + (lp >= 4 ? (int)kRing : 0)) * 4;
     // Loads of up to 16 bytes hold an L1 line each while they are in flight:
     // with all 227 KB taken as shared memory the 28 KB of L1 left carry 0.5-0.6
     // of them per cycle and SM, with 195 KB (60 KB of L1) 0.8-1.0 (probed; 32-byte
@@ -363,15 +401,13 @@ cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, 
     const int smem_words = std::max(4, std::min((words + 3) & ~3, (max_optin - fixed_bytes) / 4) & ~3);
     const int smem = fixed_bytes + smem_words * 4;
     const bool fold = words <= 2 * smem_words;  // it folds once when at most twice as long
-    // every trial starts and ends on a 16-byte boundary
-    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
     const bool pre4 = g.sum_fits >= 4;
     const FixedKernel kern = vec ? (fold ? pick_kernel<true, true>(lp, pre4) : pick_kernel<true, false>(lp, pre4))
                                  : (fold ? pick_kernel<false, true>(lp, pre4) : pick_kernel<false, false>(lp, pre4));
     if (!kern) return cudaErrorInvalidValue;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(num_sms, y.n_trials));
-    kern<<<(unsigned)grid, kFxThreads, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
+    kern<<<(unsigned)grid, 32 * warps, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
     return cudaGetLastError();
 }
 

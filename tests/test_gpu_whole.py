@@ -149,3 +149,47 @@ def test_payouts_are_exact(catalogue):
 class _Layer:
     def __init__(self, p, j):
         self.agg_ret, self.agg_lim = p.agg_ret[j:j + 1], p.agg_lim[j:j + 1]
+
+
+@pytest.mark.parametrize("n_elt,n_layers,per,nnz", [(3, 1, 3, 0.3), (8, 2, 8, 0.1), (16, 8, 8, 0.02), (16, 8, 16, 0.5),
+                                                    (24, 5, 12, 0.2), (32, 4, 32, 0.3), (40, 9, 20, 0.1)])
+def test_adjoint_records(n_elt, n_layers, per, nnz):
+    """The group adjoint against the FP64 oracle at the edges of its records:
+    one to 32 columns, events with up to three columns on their middle branch
+    and with more (evaluated from their row), records from the CSR and from
+    the table rows (the same bits), ragged trials of 0 to 2,049 events."""
+    import oracle
+    w = workloads.random_case(31 + n_elt, catalogue=3001, n_elt=n_elt, n_layers=n_layers, n_trials=1, dense_k=4,
+                              max_elts_per_layer=per, nnz_frac=nnz, mult_range=(0.8, 1.2))
+    rng = np.random.default_rng(n_elt)
+    lengths = np.array(LENGTHS * 3 + [700] * 60)
+    rng.shuffle(lengths)
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    ids = rng.integers(0, 3001, size=int(off[-1]), dtype=np.int32)
+    w.yet = workloads.YET(n_trials=lengths.size, event_ids=ids, trial_off=off)
+    s = oracle.ylt(w.oracle_problem(), want_sum=True)[2]
+    w.portfolio.agg_ret[:] = np.median(s, axis=1) * 0.5 + 1.0
+    w.portfolio.agg_lim[:] = np.median(s, axis=1) + 1.0
+    g = rng.uniform(0.5, 1.5, size=(n_layers, lengths.size))
+    ot, om, _, _ = oracle.grad(w.oracle_problem(), g)
+    outs = []
+    for layouts in (art.ART_LAYOUT_LAYER | art.ART_LAYOUT_GROUP,
+                    art.ART_LAYOUT_LAYER | art.ART_LAYOUT_GROUP | art.ART_LAYOUT_SPARSE):
+        p = art.portfolio_from_workload(w, layouts=layouts, variant=art.ART_VARIANT_SKIP)
+        try:
+            d_ids, d_off = torch.from_numpy(ids).cuda(), torch.from_numpy(off).cuda()
+            y = torch.empty((n_layers, lengths.size), dtype=torch.float64, device="cuda")
+            br = torch.empty((n_layers, lengths.size), dtype=torch.uint8, device="cuda")
+            art.art_run_ylt(p, lengths.size, d_ids, d_off, 0, y, br)
+            gt = torch.empty((n_layers, 4), dtype=torch.float64, device="cuda")
+            gm = torch.empty(n_elt, dtype=torch.float64, device="cuda")
+            art.art_run_ylt_backward(p, lengths.size, d_ids, d_off, 0, br, torch.from_numpy(g).cuda(), gt, gm)
+            assert art.art_get_device_status(p) == art.ART_OK
+            outs.append((gt.cpu().numpy(), gm.cpu().numpy()))
+        finally:
+            p.close()
+    np.testing.assert_array_equal(outs[0][0], outs[1][0])
+    np.testing.assert_array_equal(outs[0][1], outs[1][1])
+    # weights and products are FP32 (2^-24 each), the sums compensated
+    np.testing.assert_allclose(outs[1][0], ot, rtol=1e-6, atol=1e-6 * np.abs(ot).max())
+    np.testing.assert_allclose(outs[1][1], om, rtol=2e-6, atol=1e-6 * np.abs(om).max())
