@@ -145,8 +145,10 @@ __global__ void __launch_bounds__(256) payouts_table_kernel(const LayerArgs la, 
     if ((threadIdx.x & 31) == 0 && (i >> 5) < words) bits[i >> 5] = m;  // the padding too
 }
 
+// XL of C = c units (the product is exact, so the FMA rounds as the
+// subtraction alone).
 __device__ __forceinline__ double agg_of(const PayArgs& a, unsigned long long c) {
-    return xl_f64((double)c * a.unit, a.agg_ret, a.agg_lim);
+    return fmin(fmax(fma((double)c, a.unit, -a.agg_ret), 0.0), a.agg_lim);
 }
 
 // u units as FP64, exactly: an FP32 value (the units hold at most 24
@@ -183,6 +185,15 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
     int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
     uint32_t max_id = 0;
     bool lost = false;
+    // the trial losses of up to 32 trials, lane s holding the s-th: their FP64
+    // steps run once per 32 trials
+    unsigned long long held = 0;
+    int64_t held_t = -1;
+    int slot = 0;
+    auto flush = [&]() {
+        if (ylt && held_t >= 0) ylt[held_t] = agg_of(a, held);  // A(C_K): the telescoped sum of the payouts
+        held_t = -1;
+    };
     Trials<VEC> trials(y, n_warps);
     Span<VEC> cur = trials.first(y, t);
     ids.request(cur, 0, lane);
@@ -236,8 +247,15 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
                         for (int i = 0; i < 4; ++i) {
                             const unsigned long long before = c;
                             c += oh[i];
+                            const bool crosses = c >= a.pass && before < a.full && (before < a.pass || c >= a.full);
                             if (before >= a.pass && c < a.full) v[i] = units_f64(oh[i], a.unit_f);
-                            else if (c >= a.pass && before < a.full) v[i] = agg_of(a, c) - agg_of(a, before);
+                            // one evaluation, and only where some lane's event crosses: an FP64
+                            // instruction takes a warp 16 cycles of its SM. From the retention the
+                            // payout is XL(C); to the limit it is what XL(C before) leaves of it.
+                            if (__any_sync(kFull, crosses)) {
+                                const double x = agg_of(a, before < a.pass ? c : before);
+                                if (crosses) v[i] = before < a.pass ? x : a.agg_lim - x;
+                            }
                             if (before < a.full && c >= a.full) at = (int32_t)(d + i - cur.head());
                         }
                         const unsigned m = __ballot_sync(kFull, at >= 0);
@@ -256,13 +274,20 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
                 }
             }
         }
-        if (lane == 0 && !lost) {
-            if (exhaust) exhaust[t] = first_full;
-            if (ylt) ylt[t] = agg_of(a, carry);  // A(C_K): the telescoped sum of the payouts
+        if (lost) break;
+        if (exhaust && lane == 0) exhaust[t] = first_full;
+        if (lane == slot) {
+            held = carry;
+            held_t = t;
+        }
+        if (++slot == 32) {
+            flush();
+            slot = 0;
         }
         t = tn;
         cur = nxt;
     }
+    flush();
     if (lost) {
         ids.phase ^= 1u;
         ids.wait();  // the copy in flight may still come: shared memory stays until then
