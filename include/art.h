@@ -75,7 +75,7 @@ typedef struct {
 
 /* Kernel variants for art_run_ylt. */
 enum {
-    ART_VARIANT_AUTO = 0,     /* batched when the pool layout exists, else plain          */
+    ART_VARIANT_AUTO = 0,     /* by the layouts built, the layers' terms and the YET's size */
     ART_VARIANT_PLAIN = 1,    /* one launch per layer over a per-layer event-major table  */
     ART_VARIANT_BATCHED = 2,  /* one persistent launch over all layers (pool table)       */
     ART_VARIANT_FP64 = 3,     /* all-FP64 arithmetic: per call, FP64 occurrence losses of

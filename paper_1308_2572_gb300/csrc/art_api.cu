@@ -592,8 +592,19 @@ void free_portfolio(art_portfolio* p) {
     scratch_user(-1);
 }
 
-int resolve_variant(const art_portfolio* p) {
+// The variant of a call over n_trials trials of k events (k = 0: a CSR, whose
+// length is on the device: 500 events per trial are assumed). ids NULL: they
+// will be staged on the device.
+int resolve_variant(const art_portfolio* p, int64_t n_trials, const int32_t* ids, int32_t k) {
     if (p->variant != ART_VARIANT_AUTO) return p->variant;
+    // tables of whole numbers: a pass takes about 3.2 ps per event and run of
+    // 8 layers where the sparse variant takes 12 (64 layers over 256 ELTs), after
+    // a build of about 45 ps per catalogue event and run: it pays from five
+    // events per catalogue event on
+    const bool whole = !p->ogroups.empty() && std::all_of(p->ogroups.begin(), p->ogroups.end(),
+                                                          [](const OccGroupArgs& g) { return g.sum_fits > 0; });
+    if (whole && (double)n_trials * (k > 0 ? k : 500) >= 5.0 * p->catalogue && ids_on_device(ids))
+        return ART_VARIANT_SKIP;
     // few groups: the YET is streamed once per group, each event row read
     // only when its bit is set; many groups: one pass over a pool table
     if (!p->groups.empty() && p->groups.size() <= 2) return ART_VARIANT_SKIP;
@@ -864,7 +875,7 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
     if (st) return st;
     if (n_trials == 0) return ART_OK;
     if (!ylt_dev) return ART_EINVAL;
-    const int variant = resolve_variant(p);
+    const int variant = resolve_variant(p, n_trials, event_ids_dev, trial_off_dev ? 0 : events_per_trial);
     if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     YetArgs y{event_ids_dev, trial_off_dev, n_trials, trial_off_dev ? 0 : events_per_trial, p->catalogue};
     cudaError_t e;
@@ -969,7 +980,7 @@ art_status host_run(art_portfolio* p, int64_t n_trials, const int32_t* event_ids
         for (int64_t t = 0; t < n_trials; ++t)
             if (trial_off_host[t + 1] < trial_off_host[t]) return ART_EINVAL;
     }
-    const int variant = resolve_variant(p);
+    const int variant = resolve_variant(p, n_trials, nullptr, trial_off_host ? 0 : events_per_trial);
     if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     if (!(p->flags & ART_FLAG_HOST_STAGED) && one_pass_over_ids(p, variant)) {
         const int32_t* d_ids = device_alias(event_ids_host);
