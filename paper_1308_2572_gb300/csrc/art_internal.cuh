@@ -453,6 +453,12 @@ cudaError_t metrics_run_k(const double* ylt, int64_t n, int32_t n_layers, const 
                           double* mean, double* pml, double* tvar, double* sum_out, cudaStream_t s,
                           void* scratch = nullptr, size_t scratch_bytes = 0);
 size_t metrics_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_p);
+// The one-read form of the metrics (metrics_list.cu): whether it takes ranks
+// up to k_max of n_layers layers of n trials, its scratch, and the call.
+bool metrics_listable(int64_t n, int32_t n_layers, int64_t k_max);
+size_t metrics_list_bytes(int64_t n, int32_t n_layers);
+cudaError_t metrics_list_run(const double* ylt, int64_t n, int32_t n_layers, const int64_t* k, int32_t n_p, double* mean,
+                             double* pml, double* tvar, double* sum_out, cudaStream_t s, void* scratch);
 cudaError_t metrics_backward_run(const double* ylt, int64_t n, int32_t n_layers, const double* probs,
                                  int32_t n_p, const double* pml, const double* gmean, const double* gtvar,
                                  double* gylt, cudaStream_t s);

@@ -890,16 +890,28 @@ int64_t tail_count(double p, int64_t n) {
 }
 
 size_t metrics_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_p) {
-    return metrics_layout(n_layers, n_p, blocks_per_layer(n, n_layers), default_cand_slots(n, n_layers)).total;
+    return std::max(metrics_list_bytes(n, n_layers),
+                    metrics_layout(n_layers, n_p, blocks_per_layer(n, n_layers), default_cand_slots(n, n_layers)).total);
 }
 
 cudaError_t metrics_run_k(const double* ylt, int64_t n, int32_t n_layers, const int64_t* k, int32_t n_p,
                           double* mean, double* pml, double* tvar, double* sum_out, cudaStream_t s,
                           void* scratch, size_t scratch_bytes) {
+    char* w = static_cast<char*>(scratch);
+    int64_t k_max = 1;
+    for (int q = 0; q < n_p; ++q) k_max = std::max(k_max, k[q]);
+    if (metrics_listable(n, n_layers, k_max)) {
+        const size_t bytes = metrics_list_bytes(n, n_layers);
+        const bool own = !w || scratch_bytes < bytes;
+        cudaError_t err = own ? scratch_alloc((void**)&w, bytes, s) : cudaSuccess;
+        if (err != cudaSuccess) return err;
+        err = metrics_list_run(ylt, n, n_layers, k, n_p, mean, pml, tvar, sum_out, s, w);
+        const cudaError_t e2 = own ? cudaFreeAsync(w, s) : cudaSuccess;
+        return err ? err : e2;
+    }
     const int nblk = blocks_per_layer(n, n_layers);
     const uint64_t slots = default_cand_slots(n, n_layers);
     const MetricsLayout m = metrics_layout(n_layers, n_p, nblk, slots);
-    char* w = static_cast<char*>(scratch);
     const bool own = !w || scratch_bytes < m.total;
     cudaError_t err = own ? scratch_alloc((void**)&w, m.total, s) : cudaSuccess;
     if (err != cudaSuccess) return err;
@@ -1035,8 +1047,22 @@ extern "C" art_status art_metrics_noalloc(const double* ylt_dev, int64_t n_trial
         set_last_error(err);
         return ART_ECUDA;
     }
+    int64_t k[kMaxProbs], k_max = 1;
+    for (int q = 0; q < n_p; ++q) {
+        k[q] = tail_count(probs_host[q], n_trials);
+        k_max = std::max(k_max, k[q]);
+    }
+    if (metrics_listable(n_trials, n_layers, k_max) &&
+        metrics_list_bytes(n_trials, n_layers) <= (size_t)ART_METRICS_NOALLOC_SCRATCH_BYTES) {
+        err = metrics_list_run(ylt_dev, n_trials, n_layers, k, n_p, mean_dev, pml_dev, tvar_dev, nullptr, stream, w);
+        if (err != cudaSuccess) {
+            set_last_error(err);
+            return ART_ECUDA;
+        }
+        return ART_OK;
+    }
     KParams kq = {};
-    for (int q = 0; q < n_p; ++q) kq.k[q] = tail_count(probs_host[q], n_trials);
+    for (int q = 0; q < n_p; ++q) kq.k[q] = k[q];
     // the scratch keeps the previous call's contents: the launcher clears
     // what must start at zero
     err = launch_metric_kernels(ylt_dev, n_trials, n_layers, n_p, kq, nblk, reinterpret_cast<char*>(w), m, slots,

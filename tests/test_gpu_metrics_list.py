@@ -1,0 +1,49 @@
+"""The one-read metrics (sample, pass, finish) against a full sort in FP64:
+sizes around the rows that fit shared memory, distributions that make the
+sample's threshold, the tie key and the lists go each way, misaligned rows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1308_2572_gb300 import art
+
+pytestmark = pytest.mark.gpu
+
+
+def _rows(n, rng):
+    ln = rng.lognormal(15.0, 2.0, n)
+    rows = [ln, np.where(ln > np.median(ln), ln, 0.0),             # half the trials without a loss
+            np.minimum(ln, np.quantile(ln, 0.7)),                  # capped in 30% of trials
+            np.minimum(ln, np.quantile(ln, 0.9995)),               # capped in fewer than k
+            np.full(n, 4.0e7), np.zeros(n),                        # constant
+            np.where(np.arange(n) == n // 3, 1e300, ln),           # one loss far above any sample
+            np.where(rng.random(n) < 0.002, ln, 0.0),              # fewer losses than k at 0.99
+            np.floor(ln / 1e6) * 1e6,                              # heavy ties everywhere
+            np.sort(ln), 1e-310 * rng.integers(0, 1000, n),        # ordered; subnormal
+            np.where(rng.random(n) < 0.4, 3.0, np.where(rng.random(n) < 0.5, 2.0, 5.0))]  # the second value repeats
+    return np.stack(rows)
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 1000, 20480, 20481, 50_003, 300_001])
+def test_metrics_match_a_full_sort(n):
+    rng = np.random.default_rng(n)
+    y = _rows(n, rng)
+    dev = torch.from_numpy(y).cuda()
+    for probs in ([0.99], [0.95, 0.999], [0.9, 0.99, 0.996], [0.5, 0.97]):
+        L, n_p = y.shape[0], len(probs)
+        om, op, ot = oracle.metrics(y, probs)
+        outs = []
+        for fn in (art.art_metrics, art.art_metrics_noalloc, art.art_metrics):
+            mean = torch.full((L,), -1.0, dtype=torch.float64, device="cuda")
+            pml = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+            tvar = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+            fn(dev, n, L, probs, mean, pml, tvar)
+            outs.append([t.cpu().numpy() for t in (mean, pml, tvar)])
+        for got in outs:
+            np.testing.assert_array_equal(got[1], op)  # selected exactly
+            # one or two roundings against the oracle's sequential FP64 sums
+            np.testing.assert_allclose(got[0], om, rtol=1e-12, atol=1e-320)
+            np.testing.assert_allclose(got[2], ot, rtol=1e-12, atol=1e-320)
+        for a, b in zip(outs[0], outs[2]):
+            np.testing.assert_array_equal(a, b)  # repeatable bits
