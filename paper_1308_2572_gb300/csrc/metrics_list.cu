@@ -4,7 +4,7 @@
 //
 // PML_p and TVaR_p need only a layer's k largest losses, k = ceil((1 - p) n).
 // Where k is a small part of n, three launches do:
-//   1. sample (one CTA per layer): the r-th largest of 4,096 losses at hashed
+//   1. sample (one CTA per layer): the r-th largest of 8,192 losses at hashed
 //      positions is a threshold T below which the k-th largest lies with
 //      overwhelming probability (r is about six standard deviations past the
 //      sample's share of k); the sample's largest loss, if it repeats, is the
@@ -21,8 +21,9 @@
 //
 // What bounds it: HBM (8 bytes per loss, once); the general path's two full
 // reads and six list passes took 1.04 ms on 128 layers x 1,000,000 trials at
-// three probabilities, this takes 0.47 ms (floor 0.15), and one layer's metrics
-// 43 us against 89 (eight dependent launches).
+// three probabilities, this takes 0.27 ms (floor 0.15: the pass issues 37
+// instructions per 32 losses and runs at 0.73 of the copy rate), and one layer's
+// metrics 40 us against 90 (eight dependent launches).
 #include <algorithm>
 #include <cmath>
 
@@ -35,14 +36,14 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr unsigned kAll = 0xffffffffu;
-constexpr int kSample = 4096;
+constexpr int kSample = 8192;
 constexpr int kFinishThreads = 1024;
-constexpr int kSmall = 20480;        // keys the finish CTA holds in shared memory (160 KB)
+constexpr int kSmall = 26624;        // keys the finish CTA holds in shared memory (208 KB)
 constexpr int kPassThreads = 256;
 constexpr int kPassUnroll = 8;       // values per thread whose loads are in flight together
 constexpr u64 kNoTie = ~0ULL;
 constexpr int kBins = 2048;          // 11-bit digits
-constexpr int kDirect = 512;         // candidates that are ranked by comparison
+constexpr int kDirect = 128;         // candidates that are ranked by comparison
 
 struct Ranks {
     long long k[kMaxProbs];
@@ -51,7 +52,7 @@ struct Ranks {
 
 // Per-layer state, written by the sample.
 struct ListState {
-    u64 threshold;   // T
+    u64 threshold;   // T (its low word is 0)
     u64 tie;         // the tie key (kNoTie: none)
     u64 sum[2];      // fixed-point sum of the row (unit by ref)
     u64 n_tie;
@@ -100,16 +101,43 @@ struct SelectScratch {
     u64 red[64];
     unsigned int hist[kBins];
     u64 cand[kDirect];
+    unsigned int warp_sum[32];
     unsigned int n_cand;
     int bin;
-    u64 above;
+    unsigned int above;
     u64 found;
 };
 
+// The bin of s.hist where the count from the top reaches krem (into s.bin) and
+// the count above it (s.above): two bins per thread, a scan over the block.
+__device__ __forceinline__ void pick_bin(SelectScratch& s, unsigned int krem) {
+    static_assert(kBins == 2 * kFinishThreads, "two bins per thread");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int b1 = kBins - 1 - 2 * (int)threadIdx.x, b0 = b1 - 1;  // from the top
+    const unsigned int c1 = s.hist[b1], c0 = s.hist[b0];
+    unsigned int incl = c1 + c0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int v = __shfl_up_sync(kAll, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) s.warp_sum[w] = incl;
+    __syncthreads();
+    const unsigned int ws = s.warp_sum[lane];
+    incl += __reduce_add_sync(kAll, lane < w ? ws : 0u);
+    const unsigned int excl = incl - c1 - c0;
+    if (excl < krem && krem <= incl) {
+        const bool first = krem <= excl + c1;
+        s.bin = first ? b1 : b0;
+        s.above = first ? excl : excl + c1;
+        s.n_cand = 0;
+    }
+    __syncthreads();
+}
+
 // The k-th largest (k >= 1) of the n keys that get(i) yields, of which tie
 // counts n_tie more times; n + n_tie >= k. Every thread of the block calls it
-// and receives it. MSD radix select over the offsets from the smallest
-// possible key lo; once few candidates are left they are ranked directly.
+// and receives it. MSD radix select over the offsets from the smallest key lo; once few candidates are left they are ranked directly.
 template <class Get>
 __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 hi, long long k, SelectScratch& s) {
     int top = 64 - __clzll((long long)(hi - lo));  // bits of the largest offset
@@ -121,39 +149,14 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
         __syncthreads();
         for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
             const u64 d = get(i) - lo;
-            if (get(i) >= lo && (top >= 64 || (d >> top) == prefix)) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], 1u);
+            if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], 1u);
         }
         if (threadIdx.x == 0 && n_tie) {
             const u64 d = tie - lo;
-            if (tie >= lo && (top >= 64 || (d >> top) == prefix)) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], (unsigned)n_tie);
+            if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], (unsigned)n_tie);
         }
         __syncthreads();
-        // the bin where the count from the top reaches krem: warp 0 scans 64
-        // bins per lane, from the top
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            u64 mine = 0;
-            for (int b = 0; b < kBins / 32; ++b) mine += s.hist[kBins - 1 - (lane * (kBins / 32) + b)];
-            u64 incl = mine;
-            for (int o = 1; o < 32; o <<= 1) {
-                const u64 v = __shfl_up_sync(kAll, incl, o);
-                if (lane >= o) incl += v;
-            }
-            u64 run = incl - mine;
-            if ((long long)run < krem && krem <= (long long)incl)
-                for (int b = 0; b < kBins / 32; ++b) {
-                    const int bin = kBins - 1 - (lane * (kBins / 32) + b);
-                    const unsigned c = s.hist[bin];
-                    if ((long long)(run + c) >= krem) {
-                        s.bin = bin;
-                        s.above = run;
-                        s.n_cand = 0;
-                        break;
-                    }
-                    run += c;
-                }
-        }
-        __syncthreads();
+        pick_bin(s, (unsigned int)krem);
         const u64 in_bin = s.hist[s.bin];
         prefix = prefix << bits | (u64)s.bin;
         krem -= (long long)s.above;
@@ -163,11 +166,11 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
             // against the others
             for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
                 const u64 v = get(i);
-                if (v >= lo && ((v - lo) >> top) == prefix) s.cand[atomicAdd(&s.n_cand, 1u)] = v;
+                if (((v - lo) >> top) == prefix) s.cand[atomicAdd(&s.n_cand, 1u)] = v;
             }
             __syncthreads();
             const int m = (int)s.n_cand;
-            const bool tie_in = n_tie && tie >= lo && ((tie - lo) >> top) == prefix;
+            const bool tie_in = n_tie && ((tie - lo) >> top) == prefix;
             for (int c = threadIdx.x; c < m + (tie_in ? 1 : 0); c += blockDim.x) {
                 const u64 v = c < m ? s.cand[c] : tie;
                 u64 gt = 0, ge = 0;
@@ -198,27 +201,54 @@ __device__ __forceinline__ int64_t sample_pos(int i, int64_t n) {
     return (int64_t)__umul64hi(h ^ (h >> 29), (u64)n);
 }
 
+// The threshold's low word is left 0 (a slightly lower T), so the select works
+// on high words: two 11-bit digits of their offset from the sample's smallest.
 __global__ void __launch_bounds__(kFinishThreads) list_sample_kernel(const double* __restrict__ ylt, int64_t n,
                                                                      int rank, ListState* __restrict__ st) {
-    __shared__ u64 s_keys[kSample];
     __shared__ SelectScratch s;
+    constexpr int PER = kSample / kFinishThreads;
     const u64* row = reinterpret_cast<const u64*>(ylt) + (size_t)blockIdx.x * (size_t)n;
-    u64 mx = 0;
-    for (int i = threadIdx.x; i < kSample; i += kFinishThreads) {
-        const u64 v = row[sample_pos(i, n)] & 0x7fffffffffffffffULL;
-        s_keys[i] = v;
-        mx = max(mx, v);
+    u64 v[PER];
+    u64 mx = 0, mn = ~0ULL;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) v[i] = row[sample_pos(i * kFinishThreads + threadIdx.x, n)] & 0x7fffffffffffffffULL;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        mx = max(mx, v[i]);
+        mn = min(mn, v[i]);
     }
+    for (int i = threadIdx.x; i < kBins; i += kFinishThreads) s.hist[i] = 0;
     mx = block_max(mx, s.red);
-    u64 rep = 0;
-    for (int i = threadIdx.x; i < kSample; i += kFinishThreads) rep += s_keys[i] == mx;
-    rep = block_sum(rep, s.red);
-    const u64 t = kth_largest([&](int64_t i) { return s_keys[i]; }, kSample, 0ULL, 0ULL, 0ULL, mx, rank, s);
+    mn = ~block_max(~mn, s.red);
+    unsigned int rep = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) rep += v[i] == mx;
+    const u64 repeats = block_sum(rep, s.red);
+    const unsigned int lo = (unsigned int)(mn >> 32);
+    const int top = 32 - __clz((int)((unsigned int)(mx >> 32) - lo));
+    const int sh1 = max(top - 11, 0), sh2 = max(top - 22, 0);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) atomicAdd(&s.hist[((unsigned int)(v[i] >> 32) - lo) >> sh1], 1u);
+    __syncthreads();
+    pick_bin(s, (unsigned int)rank);
+    const unsigned int b1 = (unsigned int)s.bin, above = s.above;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBins; i += kFinishThreads) s.hist[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const unsigned int d = (unsigned int)(v[i] >> 32) - lo;
+        if (d >> sh1 == b1) atomicAdd(&s.hist[(d >> sh2) & ((1u << (sh1 - sh2)) - 1u)], 1u);
+    }
+    __syncthreads();
+    pick_bin(s, (unsigned int)rank - above);
     if (threadIdx.x == 0) {
         ListState l{};
-        l.threshold = t;
-        l.tie = rep > 1 && mx ? mx : kNoTie;
+        l.threshold = (u64)(lo + (((b1 << (sh1 - sh2)) | (unsigned int)s.bin) << sh2)) << 32;
+        l.tie = repeats > 1 && mx ? mx : kNoTie;
+        // the pass's short fixed point wants room below the sum's unit
         l.ref = min(ref_exp(mx) + 3, 2046);
+        l.beyond = l.ref < 128 ? 1u : 0u;
         st[blockIdx.x] = l;
     }
 }
@@ -230,29 +260,62 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
     const unsigned lane = threadIdx.x & 31;
     const u64* row = reinterpret_cast<const u64*>(ylt) + (size_t)j * (size_t)n;
     u64* list = lists + (size_t)j * cap;
-    const u64 thr = max(st[j].threshold, 1ULL), tie = st[j].tie;  // zeros are never listed
+    // keys of a high word from thr on are listed; zeros never are
+    const unsigned int thr = max((unsigned int)(st[j].threshold >> 32), 1u);
+    const unsigned int tie_hi = (unsigned int)(st[j].tie >> 32), tie_lo = (unsigned int)st[j].tie;
     const int ref = st[j].ref;
-    Fix sum{0, 0};
+    // The sum as four 32-bit words, the highest a carry: a key within 31
+    // binades below ref is its mantissa at the top of 96 bits, shifted down
+    // (three shifts and four adds; no bit is lost, so the unit is 2^-96 of
+    // ref's upper end, as in the general path). Zeros add nothing; any other
+    // key (rare) goes the long way in `rest`.
+    unsigned int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+    Fix rest{0, 0};
     unsigned int n_tie = 0;
     bool beyond = false;
     for (int64_t i0 = (int64_t)blockIdx.x * kPassThreads * kPassUnroll; i0 < n;
          i0 += (int64_t)gridDim.x * kPassThreads * kPassUnroll) {
-        u64 kv[kPassUnroll];  // 0 past the end
+        unsigned int kh[kPassUnroll], kl[kPassUnroll];  // 0 past the end
+        if (i0 + kPassThreads * kPassUnroll <= n) {
 #pragma unroll
-        for (int u = 0; u < kPassUnroll; ++u) {
-            const int64_t i = i0 + (int64_t)u * kPassThreads + threadIdx.x;
-            kv[u] = i < n ? key_at(row, i) : 0ULL;
+            for (int u = 0; u < kPassUnroll; ++u) {
+                const u64 v = key_at(row, i0 + u * kPassThreads + threadIdx.x);
+                kh[u] = (unsigned int)(v >> 32);
+                kl[u] = (unsigned int)v;
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < kPassUnroll; ++u) {
+                const int64_t i = i0 + (int64_t)u * kPassThreads + threadIdx.x;
+                const u64 v = i < n ? key_at(row, i) : 0ULL;
+                kh[u] = (unsigned int)(v >> 32);
+                kl[u] = (unsigned int)v;
+            }
         }
-        unsigned in = 0;  // bit u: listed
+        unsigned in = 0, odd = 0;  // bit u: listed; summed the long way
 #pragma unroll
         for (int u = 0; u < kPassUnroll; ++u) {
-            const u64 key = kv[u];
-            const int e = (int)(key >> 52);
-            if (e <= ref) fix_add(sum, key, ref);
-            else beyond = true;
-            const bool eq = key == tie;
+            const unsigned int d = (unsigned int)ref - (kh[u] >> 20);
+            const unsigned int hi = __funnelshift_l(kl[u], kh[u], 11) | 0x80000000u, lo = kl[u] << 11;
+            const unsigned int x2 = hi >> (d & 31), x1 = __funnelshift_r(lo, hi, d), x0 = __funnelshift_r(0u, lo, d);
+            asm("{\n.reg .pred p;\nsetp.lt.u32 p, %4, 32;\n"
+                "@p add.cc.u32 %0, %0, %5;\n@p addc.cc.u32 %1, %1, %6;\n"
+                "@p addc.cc.u32 %2, %2, %7;\n@p addc.u32 %3, %3, 0;\n}"
+                : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3)
+                : "r"(d), "r"(x0), "r"(x1), "r"(x2));
+            if (d >= 32u && (kh[u] | kl[u])) odd |= 1u << u;
+            const bool eq = kh[u] == tie_hi && kl[u] == tie_lo;
             n_tie += eq;
-            in |= (unsigned)(key >= thr && !eq) << u;
+            if (kh[u] >= thr && !eq) in |= 1u << u;
+        }
+        if (odd) {
+#pragma unroll
+            for (int u = 0; u < kPassUnroll; ++u)
+                if ((odd >> u) & 1u) {
+                    // a key above ref, or below what the list's threshold can tell from 0
+                    if ((int)(kh[u] >> 20) > ref || kh[u] == 0u) beyond = true;
+                    else fix_add(rest, (u64)kh[u] << 32 | kl[u], ref);
+                }
         }
         if (__any_sync(kAll, in != 0u)) {
             // one counter update per warp and step: a scan of the lanes' counts
@@ -269,11 +332,15 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
 #pragma unroll
             for (int u = 0; u < kPassUnroll; ++u)
                 if ((in >> u) & 1u) {
-                    if (base < cap) list[base] = kv[u];
+                    if (base < cap) list[base] = (u64)kh[u] << 32 | kl[u];
                     ++base;
                 }
         }
     }
+    // the words hold units of 2^(ref - 1075 - 43): twice kFixBits' unit
+    Fix sum{(u64)a1 << 32 | a0, (u64)a3 << 32 | a2};
+    sum = Fix{sum.lo << 1, sum.hi << 1 | sum.lo >> 63};
+    fix_add2(sum, rest.lo, rest.hi);
     fix_block_atomic(st[j].sum, sum);
     n_tie = __reduce_add_sync(kAll, n_tie);
     if (lane == 0 && n_tie) atomicAdd(&st[j].n_tie, (u64)n_tie);
@@ -314,11 +381,23 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     const u64* src = use_list ? lists + (size_t)j * cap : row;
     const bool held = m <= kSmall;
     u64 mx = n_tie ? tie : 0ULL, mn = n_tie ? tie : ~0ULL;
-    for (int64_t i = threadIdx.x; i < m; i += kFinishThreads) {
-        const u64 v = src[i] & 0x7fffffffffffffffULL;
-        if (held) s_keys[i] = v;
-        mx = max(mx, v);
-        mn = min(mn, v);
+    constexpr int U = 8;  // loads in flight per thread
+    for (int64_t i0 = threadIdx.x; i0 < m; i0 += (int64_t)U * kFinishThreads) {
+        u64 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + (int64_t)u * kFinishThreads;
+            v[u] = i < m ? src[i] & 0x7fffffffffffffffULL : 0ULL;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + (int64_t)u * kFinishThreads;
+            if (i < m) {
+                if (held) s_keys[i] = v[u];
+                mx = max(mx, v[u]);
+                mn = min(mn, v[u]);
+            }
+        }
     }
     mx = block_max(mx, s.red);
     mn = ~block_max(~mn, s.red);
@@ -412,9 +491,10 @@ cudaError_t metrics_list_run(const double* ylt, int64_t n, int32_t n_layers, con
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        // about 8 CTAs per SM over all layers, each at least one step
+        // about 32 CTAs per SM over all layers (about five run at a time: more,
+        // shorter CTAs leave less of the last wave empty), each at least one step
         const int64_t steps = (n + kPassThreads * kPassUnroll - 1) / (kPassThreads * kPassUnroll);
-        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(steps, (8LL * sms + n_layers - 1) / n_layers));
+        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(steps, (32LL * sms + n_layers - 1) / n_layers));
         list_pass_kernel<<<dim3((unsigned)blocks, (unsigned)n_layers), kPassThreads, 0, s>>>(ylt, n, st, lists, cap);
         if ((e = cudaGetLastError())) return e;
     }
