@@ -163,6 +163,22 @@ bool art::whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e,
     return *max_units <= 4294967295.0;
 }
 
+// The same for the FP64 tables: multiples of the FP64 ulp of OccR, below 2^64.
+static bool whole_losses64(float occ_ret, float occ_lim, double elt_lim_sum, int* e) {
+    if (!(occ_ret >= 0x1p-60f) || !(occ_ret <= 0x1p100f)) return false;
+    int er, el;
+    std::frexp(occ_ret, &er);
+    *e = er - 53;
+    double bound = elt_lim_sum * 1.0001;
+    if (std::isfinite(occ_lim)) {
+        if (!(occ_lim >= 0x1p-60f)) return false;
+        std::frexp(occ_lim, &el);
+        *e = std::min(*e, el - 24);
+        bound = std::min(bound, (double)occ_lim);
+    }
+    return std::ldexp(bound, -*e) < 0x1.fffp63;
+}
+
 // Layer tile of the persistent kernels: layer j sits at (tile, slot, lane)
 // with 32 * slots layers per tile; memb holds, per (tile, ELT, lane), the
 // bits of the lane's slots whose layer covers the ELT.
@@ -336,7 +352,20 @@ cudaError_t upload_layer_build(art_portfolio* p) {
         a.occ_lim = p->occ_lim[j];
         a.np = p->layer_np[j];
         a.fix_scale = 0.0f;
+        a.unit64 = 0;
+        a.pad_ = 0;
     }
+    p->whole64 = !p->ogroups64.empty();
+    for (OccGroupArgs& g : p->ogroups64)
+        for (int s = 0; s < g.n_layers; ++s) {
+            const int32_t j = g.layer[s];
+            double lims = 0.0;
+            int e = 0;
+            for (int c = p->loff[j]; c < p->loff[j + 1]; ++c) lims += p->lim[p->lids[c]];
+            if (!whole_losses64(p->occ_ret[j], p->occ_lim[j], lims, &e)) p->whole64 = false;
+            lb[j].unit64 = e;
+            g.unit[s] = std::ldexp(1.0, e);
+        }
     // a skip group's X holds whole numbers where every layer's losses allow it
     for (OccGroupArgs& g : p->ogroups) {
         int e[kMaxOccLayers];

@@ -297,6 +297,8 @@ struct LayerBuildArgs {
     float occ_ret, occ_lim;
     int32_t np;
     float fix_scale;           // units per unit of loss where the group's X holds whole numbers, else 0
+    int32_t unit64;            // exponent of the FP64 table's unit where those tables hold whole numbers
+    int32_t pad_;
 };
 
 // One occurrence group as the build reads it (device array).
@@ -361,6 +363,7 @@ struct art_portfolio {
     double** d_occ64_ptrs = nullptr;            // [n_ogroups64]
     unsigned long long* d_occ64_max = nullptr;  // [n_ogroups64]: each FP64 table's largest entry
     int32_t og_lp64 = 0;                        // slots per row of the FP64 tables (1, 2 or 4)
+    bool whole64 = false;                       // every FP64 occurrence loss is a whole number of its layer's unit
     uint8_t* d_slotmask = nullptr;              // [n_ogroups][pool_np]: slots of the skip group holding the ELT
     uint8_t* d_slotmask64 = nullptr;            // [n_ogroups64][pool_np]: slots of the group holding the ELT
     int64_t occ64_bytes = 0;

@@ -30,12 +30,18 @@
 // mantissa and shift of its fixed-point value, so a pass adds an entry with
 // two shifts and a 128-bit add. The lanes' sums are reduced across the warp
 // (xor shuffles: every lane holds every layer's total) and lane j applies
-// layer j's aggregate terms in FP64. Integer adds replace the FP64 adds of a sequential sum, of which this
+// layer j's aggregate terms in FP64.
+//
+// Where every FP64 occurrence loss is a whole number of its layer's unit below
+// 2^64 (o is a multiple of the FP64 ulp of OccR and of OccL's, as in
+// ylt_fixed.cu: covers up to about 2,000 times their retention), the table
+// holds those numbers and the pass of ylt_fixed.cu runs over them: ids by bulk
+// copies, three 32-bit adds per entry, the same exact sums (XXFIG). Integer adds replace the FP64 adds of a sequential sum, of which this
 // part has about 0.53 TFLOP/s.
 #include <algorithm>
 #include <limits>
 
-#include "art_internal.cuh"
+#include "id_stream.cuh"
 
 namespace art {
 
@@ -50,6 +56,28 @@ __device__ __forceinline__ uint32_t ld_bits_global(const uint32_t* p) {
     uint32_t v;
     asm("ld.global.nc.L1::evict_last.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
+}
+
+// An FP64 value that is a multiple of 2^e as that multiple.
+__device__ __forceinline__ unsigned long long units64(double o, int e) {
+    const unsigned long long key = (unsigned long long)__double_as_longlong(o);
+    const unsigned long long m = (key & kMant) | (1ULL << 52);
+    const int sh = (int)(key >> 52) - 1075 - e;
+    return !key ? 0ULL : sh >= 0 ? m << sh : m >> -sh;
+}
+
+// max(v, 0) and min(v, lim) for v > 0 by their bit patterns (the FP64 pipe
+// takes a warp 16 cycles of its SM per instruction).
+__device__ __forceinline__ double clamp_bits(double v, double lim) {
+    const long long b = __double_as_longlong(v), l = __double_as_longlong(lim);
+    return __longlong_as_double(b <= 0 ? 0LL : b < l ? b : l);
+}
+
+// A float >= 0 widened, without the FP64 pipe where it is normal or 0.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f);
+    if (u - 0x00800000u >= 0x7f000000u && u) return (double)f;  // subnormal (or not finite)
+    return u ? __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29)) : 0.0;
 }
 
 // The table's largest entry: a warp maximum of the keys, one atomic per warp.
@@ -84,7 +112,7 @@ template <int LP>
 __global__ void __launch_bounds__(256) build_occ64_kernel(const LayerBuildArgs* __restrict__ lbuild,
                                                           const OccBuildGroup* __restrict__ groups,
                                                           double* const* __restrict__ occ64, int32_t catalogue,
-                                                          int32_t words) {
+                                                          int32_t words, const bool whole) {
     __shared__ LayerBuildArgs s_lb[LP];
     const OccBuildGroup& grp = groups[blockIdx.y];
     const int nl = grp.n_layers;
@@ -128,6 +156,7 @@ __global__ void __launch_bounds__(256) build_occ64_kernel(const LayerBuildArgs* 
                 }
                 o[s] = xl_f64(x, a.occ_ret, a.occ_lim);
                 nz |= o[s] > 0.0;
+                if (whole) o[s] = __longlong_as_double((long long)units64(o[s], a.unit64));
             }
         }
         double* dst = occ64[blockIdx.y] + i * LP;
@@ -201,6 +230,256 @@ __global__ void __launch_bounds__(256) build_occ64_csr_kernel(const uint32_t* __
     if ((threadIdx.x & 31) == 0 && (i >> 5) < words) grp.occ_bits[i >> 5] = m;
 }
 
+// Whole-number tables of up to 16 layers (16 / LP groups) from the CSR: a block
+// takes 128 events. Its entries' F_e are evaluated first, one entry per
+// thread (dense warps: an event has a handful of entries, and a warp that walks
+// 32 events takes as long as the longest), then each thread adds its event's
+// entries, in ELT order, to the sums of the layers that hold them, kept in
+// shared memory; a layer's first loss is stored, not added. c4's FP64 tables
+// for 16 layers: BLD us against 1,625 for a walk per group with every FP64 step
+// in it.
+constexpr int kTileEvents = 128;
+constexpr int kTileSlots = 16;
+constexpr int kTileEntries = 2048;  // entries of a block evaluated ahead; more: in place
+
+template <int LP>
+__global__ void __launch_bounds__(kTileEvents) build_occ64_tile_kernel(
+    const uint32_t* __restrict__ ptr, const SparseEntry* __restrict__ entries, const double* __restrict__ terms64,
+    int32_t np, const uint8_t* __restrict__ slotmask, const LayerBuildArgs* __restrict__ lbuild,
+    const OccBuildGroup* __restrict__ groups, int32_t n_groups, double* const* __restrict__ occ64, int32_t catalogue,
+    int32_t words) {
+    constexpr int GROUPS = kTileSlots / LP;
+    __shared__ double s_x[kTileSlots][kTileEvents];
+    __shared__ double s_f[kTileEntries];
+    __shared__ uint16_t s_elt[kTileEntries];
+    __shared__ uint16_t s_mask[kMaxPoolElts];  // the tile's slots of each ELT
+    const int g0 = blockIdx.y * GROUPS, ng = min(GROUPS, n_groups - g0);
+    const int64_t i0 = (int64_t)blockIdx.x * kTileEvents, i = i0 + threadIdx.x;
+    for (int e = threadIdx.x; e < np; e += kTileEvents) {
+        unsigned m = 0;
+        for (int g = 0; g < ng; ++g) m |= (unsigned)slotmask[(size_t)(g0 + g) * np + e] << (LP * g);
+        s_mask[e] = (uint16_t)m;
+    }
+#pragma unroll
+    for (int s = 0; s < kTileSlots; ++s) s_x[s][threadIdx.x] = 0.0;
+    const uint32_t e0 = ptr[min(i0, (int64_t)catalogue)], e1 = ptr[min(i0 + kTileEvents, (int64_t)catalogue)];
+    auto loss_of = [&](const SparseEntry& en) {
+        return clamp_bits(fma(widen(en.loss), terms64[en.elt], -terms64[np + en.elt]), terms64[2 * np + en.elt]);
+    };
+    const bool ahead = e1 - e0 <= (uint32_t)kTileEntries;
+    if (ahead)
+        for (uint32_t k = threadIdx.x; k < e1 - e0; k += kTileEvents) {
+            const SparseEntry en = entries[e0 + k];
+            s_elt[k] = (uint16_t)en.elt;
+            s_f[k] = loss_of(en);
+        }
+    __syncthreads();
+    if (i < catalogue) {
+        const uint32_t q1 = ptr[i + 1];
+        for (uint32_t q = ptr[i]; q < q1; ++q) {
+            SparseEntry en{};
+            unsigned mask;
+            double f;
+            if (ahead) {
+                mask = s_mask[s_elt[q - e0]];
+                f = s_f[q - e0];
+            } else {
+                en = entries[q];
+                mask = s_mask[en.elt];
+                f = loss_of(en);
+            }
+            for (; mask; mask &= mask - 1) {
+                double* x = &s_x[__ffs(mask) - 1][threadIdx.x];
+                const double v = *x;
+                *x = v == 0.0 ? f : v + f;
+            }
+        }
+    }
+    for (int g = 0; g < ng; ++g) {
+        const OccBuildGroup& grp = groups[g0 + g];
+        unsigned long long o[LP];
+        bool nz = false;
+#pragma unroll
+        for (int s = 0; s < LP; ++s) {
+            o[s] = 0;
+            if (s < grp.n_layers) {
+                const LayerBuildArgs& a = lbuild[grp.layer[s]];
+                const double x = s_x[LP * g + s][threadIdx.x];
+                if (x > 0.0) o[s] = units64(clamp_bits(x - (double)a.occ_ret, (double)a.occ_lim), a.unit64);
+                nz |= o[s] != 0;
+            }
+        }
+        if (i < catalogue) {
+            unsigned long long* dst = reinterpret_cast<unsigned long long*>(occ64[g0 + g]) + i * LP;
+            if constexpr (LP == 1) dst[0] = o[0];
+            else {
+#pragma unroll
+                for (int q = 0; q < LP / 2; ++q)
+                    reinterpret_cast<ulonglong2*>(dst)[q] = make_ulonglong2(o[2 * q], o[2 * q + 1]);
+            }
+        }
+        const unsigned m = __ballot_sync(kFull, i < catalogue && nz);
+        if ((threadIdx.x & 31) == 0 && (i >> 5) < words) grp.occ_bits[i >> 5] = m;
+    }
+}
+
+// The trial pass over whole numbers: that of ylt_fixed.cu's wide rows, with
+// entries of 64 bits and per-layer sums of 96.
+constexpr int k64FxIds = 8;
+template <int LT, bool VEC>
+constexpr int k64FxWarps = LT == 4 && !VEC ? 24 : 32;
+
+template <int LT, bool VEC, bool FOLD>
+__global__ void __launch_bounds__(32 * k64FxWarps<LT, VEC>, 1)
+    fixed64_kernel(const __grid_constant__ OccGroupArgs g, const YetArgs y, const int32_t smem_words,
+                   const bool early_exit, double* __restrict__ ylt, uint8_t* __restrict__ branch,
+                   int* __restrict__ flags) {
+    constexpr int E = k64FxIds;
+    constexpr int NWARP = k64FxWarps<LT, VEC>;
+    extern __shared__ __align__(512) uint32_t s_dyn[];
+    uint32_t* s_bars = s_dyn + NWARP * kRing;  // after the warps' rings
+    uint32_t* s_ids = s_bars + 64;             // [NWARP][32 * E]
+    uint32_t* s_bits = s_ids + NWARP * 32 * E;
+    const uint32_t C = (uint32_t)y.catalogue, S = (uint32_t)smem_words, none = no_event<FOLD>(C, S);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    IdStream<E> ids;
+    ids.init(s_bars, s_ids, wib, lane);
+    IdRing ring(s_dyn + wib * kRing);
+    stage_bits<FOLD>(s_bits, g.occ_bits, smem_words, (y.catalogue >> 5) + 1);
+    __syncthreads();
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int64_t n_warps = (int64_t)gridDim.x * NWARP;
+    int64_t t = (int64_t)wib * gridDim.x + blockIdx.x;
+    uint32_t max_id = 0;
+    bool lost = false;
+    Trials<VEC> trials(y, n_warps);
+    Span<VEC> cur = trials.first(y, t);
+    ids.request(cur, 0, lane);
+    while (t < y.n_trials && !lost) {
+        const int64_t tn = t + n_warps;
+        const Span<VEC> nxt = trials.next(y, cur, tn);
+        uint32_t a0[LT], a1[LT], a2[LT];  // the lane's sums, 96 bits per layer
+        unsigned long long o[LT];         // the row of the flush before
+#pragma unroll
+        for (int j = 0; j < LT; ++j) {
+            a0[j] = a1[j] = a2[j] = 0;
+            o[j] = 0;
+        }
+        auto add_row = [&]() {
+#pragma unroll
+            for (int j = 0; j < LT; ++j)
+                asm("add.cc.u32 %0, %0, %3;\naddc.cc.u32 %1, %1, %4;\naddc.u32 %2, %2, 0;"
+                    : "+r"(a0[j]), "+r"(a1[j]), "+r"(a2[j])
+                    : "r"((uint32_t)o[j]), "r"((uint32_t)(o[j] >> 32)));
+        };
+        // layer j's total over the warp, in every lane
+        auto total = [&](int j) { return fix_warp_sum(Fix{(unsigned long long)a1[j] << 32 | a0[j], a2[j]}); };
+        // a 96-bit count of units: its top 64 bits are below 2^53 unless a
+        // trial holds millions of events, so the FMA rounds once
+        auto value = [&](const Fix& f, int j) {
+            return fma((double)(f.hi << 32 | f.lo >> 32), 4294967296.0, (double)(uint32_t)f.lo) * g.unit[j];
+        };
+        bool cap = false;
+        if (cur.n == 0) ids.request(nxt, 0, lane);
+        for (uint32_t c0 = 0; c0 < cur.n; c0 += 32 * E) {
+            uint32_t id[E];
+            if (!ids.take(cur, c0, lane, id)) {
+                lost = true;
+                break;
+            }
+            clean_ids<E>(cur, c0, lane, C, none, id, max_id);
+            const bool last = c0 + 32 * E >= cur.n;
+            if (last) ids.request(nxt, 0, lane);
+            else ids.request(cur, c0 + 32 * E, lane);
+#pragma unroll
+            for (int k = 0; k < E; ++k) {
+                ring.push(id[k], bit_of<FOLD>(s_bits, g.occ_bits, id[k], S), lt_mask);
+                if ((k & 1) && ring.size() >= 32) {  // at most 31 + 64 queued: two batches
+#pragma unroll 1
+                    do {
+                        const uint32_t mine = ring.take32(lane);
+                        add_row();
+                        ld_row64<LT>(g.occ64, mine, o);
+                    } while (ring.size() >= 32);
+                    __syncwarp();
+                }
+            }
+            if (early_exit) {
+                // every layer capped: the aggregate never decreases, the loss is AggL
+                add_row();
+                bool all = true;
+#pragma unroll
+                for (int j = 0; j < LT; ++j) {
+                    o[j] = 0;
+                    const double v = value(total(j), j);
+                    if (j < g.n_layers) all = all && (v - g.agg_ret[j] >= g.agg_lim[j]);
+                }
+                if (all) {
+                    if (!last) {
+                        lost = !cur.edge() && !ids.wait();
+                        if (!lost) ids.request(nxt, 0, lane);
+                    }
+                    ring.head = ring.tail;
+                    cap = true;
+                    break;
+                }
+            }
+        }
+        __syncwarp();
+        add_row();
+#pragma unroll
+        for (int j = 0; j < LT; ++j) o[j] = 0;
+        if (lane < ring.size()) ld_row64<LT>(g.occ64, ring.peek(lane), o);
+        add_row();
+        ring.head = ring.tail;
+        __syncwarp();
+        Fix mine{0, 0};
+#pragma unroll
+        for (int j = 0; j < LT; ++j) {
+            const Fix f = total(j);
+            if (lane == j) mine = f;
+        }
+        if (lane < g.n_layers) {
+            const double sum = value(mine, lane), ret = g.agg_ret[lane], lim = g.agg_lim[lane];
+            const size_t wi = (size_t)g.layer[lane] * (size_t)y.n_trials + (size_t)t;
+            ylt[wi] = cap ? lim : xl_f64(sum, ret, lim);
+            if (branch) branch[wi] = cap ? (uint8_t)2 : agg_branch(sum, ret, lim);
+        }
+        t = tn;
+        cur = nxt;
+    }
+    if (lost) {
+        ids.phase ^= 1u;
+        ids.wait();  // the copy in flight may still come: shared memory stays until then
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
+    }
+    if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
+    if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
+}
+
+template <int LT>
+cudaError_t launch_fixed64(const OccGroupArgs& g, const YetArgs& y, int num_sms, bool early, double* ylt,
+                           uint8_t* branch, int* flags, cudaStream_t s) {
+    int dev = 0, max_optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+    const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
+    const int warps = vec ? k64FxWarps<LT, true> : k64FxWarps<LT, false>;
+    const int fixed_bytes = 256 + 16 + warps * (32 * k64FxIds + (int)kRing) * 4;
+    if (LT < 4) max_optin = std::min(max_optin, 195 * 1024);  // L1 for the gathers in flight, as in ylt_fixed.cu
+    const int words = (y.catalogue >> 5) + 1;                 // bits 0 .. C (C: the sentinel)
+    const int smem_words = std::max(4, std::min((words + 3) & ~3, (max_optin - fixed_bytes) / 4) & ~3);
+    const int smem = fixed_bytes + smem_words * 4;
+    const bool fold = words <= 2 * smem_words;
+    auto kern = vec ? (fold ? fixed64_kernel<LT, true, true> : fixed64_kernel<LT, true, false>)
+                    : (fold ? fixed64_kernel<LT, false, true> : fixed64_kernel<LT, false, false>);
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(num_sms, y.n_trials));
+    kern<<<(unsigned)grid, 32 * warps, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
+    return cudaGetLastError();
+}
+
 // Packs every entry of group blockIdx.y's table in place (fix_pack against
 // the group's reference exponent, known once the build has recorded the
 // table's largest entry), so that the trial passes add each entry without
@@ -222,7 +501,7 @@ __global__ void __launch_bounds__(k64Threads, 1) ylt_skip64_kernel(const OccGrou
                                                                   int* __restrict__ flags) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int E = k64Ids;
-    extern __shared__ __align__(16) uint32_t s_dyn[];
+    extern __shared__ __align__(512) uint32_t s_dyn[];
     int32_t* s_queue = reinterpret_cast<int32_t*>(s_dyn);  // [k64Warps][k64Queue]
     uint32_t* s_bits = s_dyn + k64Warps * k64Queue;
     {
@@ -403,7 +682,18 @@ cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8
     // per-layer tables
     const bool csr = p->sp_ptr && p->d_slotmask64 && p->d_elt_terms64 && p->d_occ;
     const SparseEntry* en = reinterpret_cast<const SparseEntry*>(p->sp_entries);
-    if (build) {
+    const bool whole = p->whole64 && ids_on_device(y.ids);
+    if (build && whole && csr) {
+        const dim3 tiles((unsigned)(((int64_t)words * 32 + kTileEvents - 1) / kTileEvents),
+                         (unsigned)((p->ogroups64.size() * p->og_lp64 + kTileSlots - 1) / kTileSlots));
+        const int32_t ng = (int32_t)p->ogroups64.size();
+        switch (p->og_lp64) {
+            case 1: build_occ64_tile_kernel<1><<<tiles, kTileEvents, 0, s>>>(p->sp_ptr, en, p->d_elt_terms64, p->pool_np, p->d_slotmask64, p->d_lbuild, p->d_ogroups64, ng, p->d_occ64_ptrs, p->catalogue, words); break;
+            case 2: build_occ64_tile_kernel<2><<<tiles, kTileEvents, 0, s>>>(p->sp_ptr, en, p->d_elt_terms64, p->pool_np, p->d_slotmask64, p->d_lbuild, p->d_ogroups64, ng, p->d_occ64_ptrs, p->catalogue, words); break;
+            case 4: build_occ64_tile_kernel<4><<<tiles, kTileEvents, 0, s>>>(p->sp_ptr, en, p->d_elt_terms64, p->pool_np, p->d_slotmask64, p->d_lbuild, p->d_ogroups64, ng, p->d_occ64_ptrs, p->catalogue, words); break;
+            default: return cudaErrorInvalidValue;
+        }
+    } else if (build) {
         cudaError_t me = cudaMemsetAsync(p->d_occ64_max, 0, sizeof(unsigned long long) * p->ogroups64.size(), s);
         if (me != cudaSuccess) return me;
         if (csr) {
@@ -415,16 +705,16 @@ cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8
             }
         } else {
             switch (p->og_lp64) {
-                case 1: build_occ64_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words); break;
-                case 2: build_occ64_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words); break;
-                case 4: build_occ64_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words); break;
+                case 1: build_occ64_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words, whole); break;
+                case 2: build_occ64_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words, whole); break;
+                case 4: build_occ64_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups64, p->d_occ64_ptrs, p->catalogue, words, whole); break;
                 default: return cudaErrorInvalidValue;
             }
         }
     }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    if (build) {
+    if (build && !whole) {
         // the tables' entries packed against their groups' largest entries
         const int64_t n_entries = ((int64_t)p->catalogue + 1) * p->og_lp64;
         const int64_t blocks = std::min<int64_t>((n_entries + 255) / 256, (int64_t)p->num_sms * 8);
@@ -434,6 +724,16 @@ cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8
     }
     if (y.n_trials == 0) return cudaSuccess;
     for (const OccGroupArgs& g : p->ogroups64) {
+        if (whole) {
+            switch (p->og_lp64) {
+                case 1: err = launch_fixed64<1>(g, y, p->num_sms, early, ylt, branch, p->d_flags, s); break;
+                case 2: err = launch_fixed64<2>(g, y, p->num_sms, early, ylt, branch, p->d_flags, s); break;
+                case 4: err = launch_fixed64<4>(g, y, p->num_sms, early, ylt, branch, p->d_flags, s); break;
+                default: err = cudaErrorInvalidValue;
+            }
+            if (err != cudaSuccess) return err;
+            continue;
+        }
         switch (p->og_lp64) {
             case 1: err = launch_group64<1>(g, y, p->num_sms, p->catalogue, early, ylt, branch, p->d_flags, s); break;
             case 2: err = launch_group64<2>(g, y, p->num_sms, p->catalogue, early, ylt, branch, p->d_flags, s); break;

@@ -114,6 +114,37 @@ def test_unbounded_losses_keep_the_fp32_tables():
         port.close()
 
 
+@pytest.mark.parametrize("n_layers,catalogue,csr", [(1, 97, True), (2, 5000, True), (3, 5000, False), (4, 1_999_999, True),
+                                                    (5, 5000, True), (17, 5000, True), (17, 97, False)])
+def test_all_fp64_rounds_once(n_layers, catalogue, csr):
+    """The all-FP64 variant over whole-number tables: the exact sum of the
+    FP64 occurrence losses, rounded once, then the aggregate terms."""
+    import math
+    w, rng = _case(n_layers, catalogue, seed=23)
+    p = w.portfolio
+    o = np.zeros((n_layers, catalogue))
+    for j in range(n_layers):
+        x = np.zeros(catalogue)
+        for e in p.layer_elt_ids[p.layer_elt_off[j]:p.layer_elt_off[j + 1]]:
+            x += np.minimum(np.maximum(p.elt_losses[e].astype(np.float64) - float(p.elt_ded[e]), 0.0), float(p.elt_lim[e]))
+        o[j] = np.minimum(np.maximum(x - p.occ_ret[j], 0.0), p.occ_lim[j])
+    lengths = np.array(LENGTHS * 2 + [300] * 40)
+    rng.shuffle(lengths)
+    layouts = art.ART_LAYOUT_LAYER | art.ART_LAYOUT_OCC64 | (art.ART_LAYOUT_SPARSE if csr else 0)
+    port = art.portfolio_from_workload(w, layouts=layouts, variant=art.ART_VARIANT_FP64)
+    try:
+        for shift in (0, 3):
+            ids, off, dev, doff = _yet(rng, catalogue, lengths, shift)
+            y = torch.full((n_layers, lengths.size), -1.0, dtype=torch.float64, device="cuda")
+            art.art_run_ylt(port, lengths.size, dev, doff, 0, y)
+            assert art.art_get_device_status(port) == art.ART_OK
+            s = np.array([[math.fsum(o[j][ids[off[t]:off[t + 1]]]) for t in range(lengths.size)] for j in range(n_layers)])
+            want = np.minimum(np.maximum(s - p.agg_ret[:, None], 0.0), p.agg_lim[:, None])
+            np.testing.assert_array_equal(y.cpu().numpy(), want)
+    finally:
+        port.close()
+
+
 @pytest.mark.parametrize("catalogue", [97, 1_999_999])
 def test_payouts_are_exact(catalogue):
     w, rng = _case(2, catalogue, seed=11)
