@@ -441,6 +441,7 @@ cudaError_t build_occ_groups(art_portfolio* p) {
             const int32_t j = p->ogroups[gi].layer[s];
             for (int32_t c = p->loff[j] + 1; c < p->loff[j + 1]; ++c)
                 if (!(p->lids[c - 1] < p->lids[c])) bg[gi].unsorted |= 1 << s;
+            if (bg[gi].unsorted) p->og_unsorted = true;
         }
     if (p->pool_np > 0 && p->sp_ptr) {
         std::vector<uint8_t> sm((size_t)ng * p->pool_np, 0);

@@ -350,6 +350,7 @@ struct art_portfolio {
     // per-call occurrence-loss tables and bitmaps
     std::vector<art::OccGroupArgs> ogroups;
     int32_t og_lp = 0;                          // slots per row of X (1, 2, 4 or 8)
+    bool og_unsorted = false;                   // some layer lists its ELTs out of ascending id order
     std::vector<float*> og_occ;
     std::vector<uint32_t*> og_bits;
     art::LayerBuildArgs* d_lbuild = nullptr;    // [n_layers]

@@ -573,6 +573,87 @@ __global__ void __launch_bounds__(256) build_occ_csr_kernel(const uint32_t* __re
     if ((threadIdx.x & 31) == 0 && (i >> 5) < words) grp.occ_bits[i >> 5] = m;
 }
 
+// The same for several groups of 8 at once (32 layers, each listing its
+// ELTs in ascending order): a block takes 128 events. Its entries' F_e are
+// evaluated first, one entry per thread (a warp that walks 32 events takes as
+// long as the longest), then each thread adds its event's entries, in ELT
+// order, to the sums of the layers that hold them, kept in shared memory. The
+// same additions in the same order as above, so the same bits. 64 layers over
+// 256 ELTs: 330 us against 550 for a walk per group, which visited every entry
+// eight times.
+constexpr int kTileEvents = 128;
+constexpr int kTileGroups = 4;  // 27 KB of shared memory per block: 32 warps per SM
+constexpr int kTileEntries = 1536;  // entries of a block evaluated ahead; more: in place
+
+__global__ void __launch_bounds__(kTileEvents) build_occ_tile_kernel(
+    const uint32_t* __restrict__ ptr, const SparseEntry* __restrict__ entries, const float* __restrict__ terms,
+    int32_t np, const uint8_t* __restrict__ slotmask, const float* __restrict__ occ_terms,
+    const LayerBuildArgs* __restrict__ lbuild, const OccBuildGroup* __restrict__ groups, int32_t n_groups,
+    int32_t catalogue, int32_t words, const bool whole) {
+    __shared__ float s_x[8 * kTileGroups][kTileEvents];
+    __shared__ uint32_t s_mask[kMaxPoolElts];  // the tile's slots of each ELT
+    __shared__ float s_f[kTileEntries];
+    __shared__ uint16_t s_elt[kTileEntries];
+    const int g0 = blockIdx.y * kTileGroups, ng = min(kTileGroups, n_groups - g0);
+    const int64_t i0 = (int64_t)blockIdx.x * kTileEvents, i = i0 + threadIdx.x;
+    for (int e = threadIdx.x; e < np; e += kTileEvents) {
+        uint32_t m = 0;
+        for (int g = 0; g < ng; ++g) m |= (uint32_t)slotmask[(size_t)(g0 + g) * np + e] << (8 * g);
+        s_mask[e] = m;
+    }
+    for (int s = 0; s < 8 * ng; ++s) s_x[s][threadIdx.x] = 0.0f;
+    const uint32_t e0 = ptr[min(i0, (int64_t)catalogue)], e1 = ptr[min(i0 + kTileEvents, (int64_t)catalogue)];
+    auto loss_of = [&](const SparseEntry& en) {
+        return fin_f32(en.loss, terms[en.elt], terms[np + en.elt], terms[2 * np + en.elt]);
+    };
+    const bool ahead = e1 - e0 <= (uint32_t)kTileEntries;
+    if (ahead)
+        for (uint32_t k = threadIdx.x; k < e1 - e0; k += kTileEvents) {
+            const SparseEntry en = entries[e0 + k];
+            s_elt[k] = (uint16_t)en.elt;
+            s_f[k] = loss_of(en);
+        }
+    __syncthreads();
+    if (i < catalogue) {
+        const uint32_t q1 = ptr[i + 1];
+        for (uint32_t q = ptr[i]; q < q1; ++q) {
+            uint32_t mask;
+            float f;
+            if (ahead) {
+                mask = s_mask[s_elt[q - e0]];
+                f = s_f[q - e0];
+            } else {
+                const SparseEntry en = entries[q];
+                mask = s_mask[en.elt];
+                f = loss_of(en);
+            }
+            for (; mask; mask &= mask - 1) s_x[__ffs((int)mask) - 1][threadIdx.x] += f;
+        }
+    }
+    for (int g = 0; g < ng; ++g) {
+        const OccBuildGroup& grp = groups[g0 + g];
+        float o[8];
+        bool nz = false;
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            o[s] = 0.0f;
+            if (s < grp.n_layers) {
+                const int32_t j = grp.layer[s];
+                o[s] = xl_f32(s_x[8 * g + s][threadIdx.x], occ_terms[2 * j], occ_terms[2 * j + 1]);
+                nz |= o[s] > 0.0f;
+                o[s] = table_entry(o[s], whole ? lbuild[j].fix_scale : 0.0f);
+            }
+        }
+        if (i < catalogue) {
+            float4* dst = reinterpret_cast<float4*>(grp.occ + i * 8);
+            dst[0] = make_float4(o[0], o[1], o[2], o[3]);
+            dst[1] = make_float4(o[4], o[5], o[6], o[7]);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, i < catalogue && nz);
+        if ((threadIdx.x & 31) == 0 && (i >> 5) < words) grp.occ_bits[i >> 5] = m;
+    }
+}
+
 template <int LT, int LP>
 cudaError_t launch_group(const OccGroupArgs& g, const YetArgs& y, int num_sms, int32_t catalogue, bool early,
                          double* ylt, uint8_t* branch, int* flags, cudaStream_t s) {
@@ -625,6 +706,14 @@ cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s) {
     // build_occ_csr_kernel)
     if (p->d_slotmask && p->sp_ptr && p->d_elt_terms && p->d_occ && p->d_lbuild) {
         const SparseEntry* en = reinterpret_cast<const SparseEntry*>(p->sp_entries);
+        if (p->og_lp == 8 && p->ogroups.size() > 1 && !p->og_unsorted) {
+            const dim3 tiles((unsigned)(((int64_t)words * 32 + kTileEvents - 1) / kTileEvents),
+                             (unsigned)((p->ogroups.size() + kTileGroups - 1) / kTileGroups));
+            build_occ_tile_kernel<<<tiles, kTileEvents, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask,
+                                                               p->d_occ, p->d_lbuild, p->d_ogroups,
+                                                               (int32_t)p->ogroups.size(), p->catalogue, words, whole);
+            return cudaGetLastError();
+        }
         switch (p->og_lp) {
             case 1: build_occ_csr_kernel<1><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
             case 2: build_occ_csr_kernel<2><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
