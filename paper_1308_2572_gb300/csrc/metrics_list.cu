@@ -4,7 +4,7 @@
 //
 // PML_p and TVaR_p need only a layer's k largest losses, k = ceil((1 - p) n).
 // Where k is a small part of n, three launches do:
-//   1. sample (one CTA per layer): the r-th largest of 8,192 losses at hashed
+//   1. sample (one CTA per layer): the r-th largest of 4,096 losses at hashed
 //      positions is a threshold T below which the k-th largest lies with
 //      overwhelming probability (r is about six standard deviations past the
 //      sample's share of k); the sample's largest loss, if it repeats, is the
@@ -36,7 +36,7 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr unsigned kAll = 0xffffffffu;
-constexpr int kSample = 8192;
+constexpr int kSample = 4096;
 constexpr int kFinishThreads = 1024;
 constexpr int kSmall = 26624;        // keys the finish CTA holds in shared memory (208 KB)
 constexpr int kPassThreads = 256;
