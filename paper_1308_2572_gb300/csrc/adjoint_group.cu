@@ -20,7 +20,7 @@
 // byte counters, K_i, and up to three (column, layers covering it with a
 // middle branch, loss); the few events with more columns are evaluated from
 // their table row. Records come from the CSR of the non-zero losses where the
-// portfolio holds it (an event with three or more of the group's losses from
+// portfolio holds it (an event with more than four of the group's losses from
 // its table row, in the group's order), else from the table rows; the same
 // values either way.
 //
@@ -208,39 +208,54 @@ __global__ void __launch_bounds__(256) adj_records_kernel(const __grid_constant_
         if (!ptr) {
             rel = record_from_row<NP, LT>(g, s_cover, i, r);
         } else {
-            int cnt = 0, ka = 0, kb = 0;
-            float va = 0.0f, vb = 0.0f;
+            // up to four of the group's losses, sorted by column
+            int cnt = 0, k4[4] = {0, 0, 0, 0};
+            float v4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
             const uint32_t q1 = ptr[i + 1];
             for (uint32_t q = ptr[i]; q < q1; ++q) {
                 const SparseEntry en = entries[q];
-                const int k = col[en.elt];
+                int k = col[en.elt];
+                float v = en.loss;
                 if (k == 255) continue;
-                if (cnt == 0) {
-                    ka = k;
-                    va = en.loss;
-                } else {
-                    kb = k;
-                    vb = en.loss;
-                }
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    if (s == cnt || (s < cnt && k < k4[s])) {
+                        const int tk = k4[s];
+                        const float tv = v4[s];
+                        k4[s] = k;
+                        v4[s] = v;
+                        k = tk;
+                        v = tv;
+                        if (s == cnt) break;
+                    }
                 ++cnt;
             }
-            if (cnt > 2) {
+            if (cnt > 4) {
                 rel = record_from_row<NP, LT>(g, s_cover, i, r);
             } else if (cnt) {
-                // one or two losses: their sum is the same in any order
-                const float wa = __fmaf_rn(s_m[ka], va, -s_d[ka]), wb = __fmaf_rn(s_m[kb], vb, -s_d[kb]);
-                const float fa = fminf(fmaxf(wa, 0.0f), s_lim[ka]);
-                const float fb = cnt > 1 ? fminf(fmaxf(wb, 0.0f), s_lim[kb]) : 0.0f;
+                // the sums in column order, as over the row (absent columns add exactly 0)
                 float x[LT];
 #pragma unroll
-                for (int j = 0; j < LT; ++j)
-                    x[j] = ((s_cover[ka] >> j) & 1u ? fa : 0.0f) + (cnt > 1 && ((s_cover[kb] >> j) & 1u) ? fb : 0.0f);
+                for (int j = 0; j < LT; ++j) x[j] = 0.0f;
+                uint32_t u = 0;
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    if (s < cnt) {
+                        const int k = k4[s];
+                        const float w = __fmaf_rn(s_m[k], v4[s], -s_d[k]), lim = s_lim[k];
+                        const float f = fminf(fmaxf(w, 0.0f), lim);
+                        if (w > 0.0f && w < lim) u |= 1u << k;
+                        const uint32_t cover = s_cover[k];
+#pragma unroll
+                        for (int j = 0; j < LT; ++j) x[j] += (cover >> j) & 1u ? f : 0.0f;
+                    }
                 uint32_t mid, cap, n = 0;
                 layer_branches<LT>(g, x, mid, cap);
                 rel = (mid | cap) != 0u;
-                if (wa > 0.0f && wa < s_lim[ka]) add_column(r, n, mid, s_cover[ka], ka, va);
-                if (cnt > 1 && wb > 0.0f && wb < s_lim[kb]) add_column(r, n, mid, s_cover[kb], kb, vb);
-                finish_record(r, n, mid, cap, 0u);
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    if (s < cnt && ((u >> k4[s]) & 1u)) add_column(r, n, mid, s_cover[k4[s]], k4[s], v4[s]);
+                finish_record(r, n, mid, cap, u);
             }
         }
         {  // an event without its bit too: the folded bitmap may gather it
