@@ -134,8 +134,8 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-KERNEL_SOURCES = {"ylt_plain": "ylt_plain.cu", "ylt_skip": "ylt_skip.cu", "ylt_batched": "ylt_batched.cu",
-                  "ylt_skip64": "ylt_skip64.cu", "ylt_sparse": "ylt_sparse.cu", "metrics": "metrics.cu",
+KERNEL_SOURCES = {"ylt_plain": "ylt_plain.cu", "ylt_skip": "ylt_fixed.cu", "ylt_batched": "ylt_batched.cu",
+                  "ylt_skip64": "ylt_skip64.cu", "ylt_sparse": "ylt_sparse.cu", "metrics": "metrics_list.cu",
                   "adjoint_group": "adjoint_group.cu"}
 
 
@@ -914,14 +914,13 @@ def main():
     # kernels of ours launched per step: forward (one per layer for the plain
     # variant; one occurrence-table build plus a trial pass per occurrence
     # group for the skip and all-FP64 variants; one persistent launch
-    # otherwise) + metrics (6 radix passes, each fused with its digit pick,
-    # and the tail sums fused with the final reduction)
+    # otherwise) + metrics (sample, pass, finish)
     n_groups = len(layer_groups(port))
     launches = {"plain": L, "skip": 1 + len(occurrence_groups(port)),
-                "fp64": 1 + len(occurrence_groups(port, 4))}.get(variant, 1) + 7
+                "fp64": 1 + len(occurrence_groups(port, 4))}.get(variant, 1) + 3
     if with_grad:
         # metrics backward (count, weights, grad) + the adjoint: per group the
-        # event masks, a pass and its reduction (group tables), else per layer
+        # event records, a pass and its reduction (group tables), else per layer
         # a pass and its reduction plus one scatter
         launches += 3 + (3 * n_groups if layouts & art.ART_LAYOUT_GROUP else 2 * L + 1)
     config = {"workload": args.config, "description": CONFIG_TEXT.get(args.config, ""),

@@ -57,7 +57,7 @@ struct ListState {
     u64 sum[2];      // fixed-point sum of the row (unit by ref)
     u64 n_tie;
     unsigned int n_list;
-    int ref;         // reference exponent of the sum
+    int ref;         // reference exponent of the pass's sum; 0: the list holds every loss, sum that
     unsigned int beyond;  // a loss with an exponent above ref was seen
     unsigned int pad;
 };
@@ -135,6 +135,25 @@ __device__ __forceinline__ void pick_bin(SelectScratch& s, unsigned int krem) {
     __syncthreads();
 }
 
+// f(key) for the keys get(0) .. get(n - 1), shared out over the block, eight
+// loads in flight per thread (a list or a row that is not held in shared
+// memory comes from L2 or HBM).
+template <class Get, class F>
+__device__ __forceinline__ void for_each_key(Get get, int64_t n, F f) {
+    constexpr int U = 8;
+    for (int64_t i0 = threadIdx.x; i0 < n; i0 += (int64_t)U * kFinishThreads) {
+        u64 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + (int64_t)u * kFinishThreads;
+            v[u] = i < n ? get(i) : 0ULL;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + (int64_t)u * kFinishThreads < n) f(v[u]);
+    }
+}
+
 // The k-th largest (k >= 1) of the n keys that get(i) yields, of which tie
 // counts n_tie more times; n + n_tie >= k. Every thread of the block calls it
 // and receives it. MSD radix select over the offsets from the smallest key lo; once few candidates are left they are ranked directly.
@@ -147,10 +166,10 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
         const int bits = min(11, top), shift = top - bits;
         for (int i = threadIdx.x; i < kBins; i += blockDim.x) s.hist[i] = 0;
         __syncthreads();
-        for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-            const u64 d = get(i) - lo;
+        for_each_key(get, n, [&](u64 v) {
+            const u64 d = v - lo;
             if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], 1u);
-        }
+        });
         if (threadIdx.x == 0 && n_tie) {
             const u64 d = tie - lo;
             if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], (unsigned)n_tie);
@@ -164,10 +183,9 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
         if (in_bin <= kDirect) {
             // few left: list them (ties once, with their count) and rank each
             // against the others
-            for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-                const u64 v = get(i);
+            for_each_key(get, n, [&](u64 v) {
                 if (((v - lo) >> top) == prefix) s.cand[atomicAdd(&s.n_cand, 1u)] = v;
-            }
+            });
             __syncthreads();
             const int m = (int)s.n_cand;
             const bool tie_in = n_tie && ((tie - lo) >> top) == prefix;
@@ -246,9 +264,12 @@ __global__ void __launch_bounds__(kFinishThreads) list_sample_kernel(const doubl
         ListState l{};
         l.threshold = (u64)(lo + (((b1 << (sh1 - sh2)) | (unsigned int)s.bin) << sh2)) << 32;
         l.tie = repeats > 1 && mx ? mx : kNoTie;
-        // the pass's short fixed point wants room below the sum's unit
-        l.ref = min(ref_exp(mx) + 3, 2046);
-        l.beyond = l.ref < 128 ? 1u : 0u;
+        // room for losses 4,096 times the sample's largest; the pass's short
+        // fixed point wants as much below. T = 0: the list (and the ties) will
+        // hold every loss but 0, and the finish sums it (a layer of few losses
+        // has no sample to set a reference by)
+        l.ref = l.threshold ? min(ref_exp(mx) + 12, 2046) : 0;
+        l.beyond = l.threshold && l.ref < 128 ? 1u : 0u;
         st[blockIdx.x] = l;
     }
 }
@@ -313,8 +334,8 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
             for (int u = 0; u < kPassUnroll; ++u)
                 if ((odd >> u) & 1u) {
                     // a key above ref, or below what the list's threshold can tell from 0
-                    if ((int)(kh[u] >> 20) > ref || kh[u] == 0u) beyond = true;
-                    else fix_add(rest, (u64)kh[u] << 32 | kl[u], ref);
+                    if (kh[u] == 0u || (ref && (int)(kh[u] >> 20) > ref)) beyond = true;
+                    else if (ref) fix_add(rest, (u64)kh[u] << 32 | kl[u], ref);
                 }
         }
         if (__any_sync(kAll, in != 0u)) {
@@ -366,11 +387,11 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     int sum_ref = 0;
     if (st) {
         const ListState l = st[j];
-        have_sum = !l.beyond;
+        have_sum = !l.beyond && l.ref;
         total = Fix{l.sum[0], l.sum[1]};
         sum_ref = l.ref;
         // every loss other than 0 that the list leaves out is below T
-        use_list = have_sum && l.n_list <= cap &&
+        use_list = !l.beyond && l.n_list <= cap &&
                    (l.threshold == 0 || (long long)(l.n_list + l.n_tie) >= kmax_rank);
         if (use_list) {
             m = l.n_list;
@@ -406,8 +427,9 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     auto get = [&](int64_t i) { return held ? s_keys[i] : src[i] & 0x7fffffffffffffffULL; };
     if (!have_sum) {
         Fix f{0, 0};
-        for (int64_t i = threadIdx.x; i < m; i += kFinishThreads) fix_add(f, get(i), e_ref);
+        for_each_key(get, m, [&](u64 v) { fix_add(f, v, e_ref); });
         total = block_fix(f, s.red);
+        if (n_tie) fix_add_times(total, tie, e_ref, n_tie);
         sum_ref = e_ref;
     }
     if (threadIdx.x == 0) {
@@ -423,13 +445,12 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
         Fix f{0, 0};
         u64 cnt = 0;
         if (v < mx)
-            for (int64_t i = threadIdx.x; i < m; i += kFinishThreads) {
-                const u64 key = get(i);
+            for_each_key(get, m, [&](u64 key) {
                 if (key > v) {
                     fix_add(f, key, e_ref);
                     ++cnt;
                 }
-            }
+            });
         f = block_fix(f, s.red);
         cnt = block_sum(cnt, s.red);
         if (threadIdx.x == 0) {
