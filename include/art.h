@@ -23,8 +23,10 @@
  *    set, and art_get_device_status reports ART_EID_RANGE.
  *  - Every piecewise-linear term is XL(v; R, L) = min(max(v - R, 0), L);
  *    limits may be +INFINITY (an unlimited cover).
- *  - No entry point waits on other CTAs or other GPUs; there are no spin
- *    waits in any kernel of this library.
+ *  - No entry point waits on other CTAs or other GPUs. The only waits inside a
+ *    kernel are a warp's for its own copies of event ids into shared memory;
+ *    they are bounded (a copy that has not come after four seconds ends the
+ *    pass, and art_get_device_status reports ART_ETIMEOUT).
  *  - A portfolio belongs to the device that was current when it was created;
  *    call the entry points that take it with that device current. A
  *    portfolio is not thread-safe (its graph cache, staging buffers and work
@@ -55,7 +57,7 @@ typedef enum {
     ART_ENOMEM = 2,        /* a device allocation failed                      */
     ART_ECUDA = 3,         /* a CUDA runtime call failed                      */
     ART_EID_RANGE = 4,     /* the device saw an event id outside [0, C)       */
-    ART_ETIMEOUT = 5,      /* reserved: a bounded wait gave up                */
+    ART_ETIMEOUT = 5,      /* a bounded wait on the device gave up            */
     ART_EUNSUPPORTED = 6   /* the portfolio lacks the layout this call needs  */
 } art_status;
 
@@ -308,8 +310,12 @@ ART_API art_status art_run_ylt_host_metrics(art_portfolio* p, int64_t n_trials, 
  *                 of the first event with C_d - AggR >= AggL (the event that
  *                 exhausts the aggregate limit), -1 if none.
  *  ylt_dev        NULL, or [T] FP64: XL(C_K; AggR, AggL), the sum of the p_d.
- * Runs FP64 arithmetic per event: a reporting path, much slower than
- * art_run_ylt. Errors: ART_EINVAL, ART_EUNSUPPORTED, ART_ECUDA.
+ * C_d is exact where the layer's occurrence losses are bounded (a finite
+ * OccL up to 255 times OccR > 0, or finite ELT limits) and the YET has at least
+ * half as many events as the catalogue: they are then evaluated once per
+ * catalogue event as whole numbers (scratch from the stream-ordered allocator).
+ * Otherwise the call runs FP64 arithmetic per event and is several times
+ * slower. Errors: ART_EINVAL, ART_EUNSUPPORTED, ART_ENOMEM, ART_ECUDA.
  */
 ART_API art_status art_run_payouts(art_portfolio* p, int32_t layer, int64_t n_trials, const int32_t* event_ids_dev,
                                    const int64_t* trial_off_dev, int32_t events_per_trial, double* payouts_dev,
@@ -505,8 +511,9 @@ ART_API art_status art_autotune(art_portfolio* p, int64_t n_trials, const int32_
 
 /* Synchronise the stream, then read and clear the portfolio's device error
  * flags: ART_OK, ART_EID_RANGE (an id outside [0, C) was seen; it counted as
- * zero loss: event ids index the direct-access tables of Section III) or
- * ART_EINVAL (decreasing CSR offsets were seen). Errors of the call itself:
+ * zero loss: event ids index the direct-access tables of Section III),
+ * ART_EINVAL (decreasing CSR offsets were seen) or ART_ETIMEOUT (a bounded
+ * wait of a kernel gave up: the outputs of that call are not complete). Errors of the call itself:
  * ART_EINVAL (NULL portfolio), ART_ECUDA. */
 ART_API art_status art_get_device_status(art_portfolio* p, cudaStream_t stream);
 

@@ -625,7 +625,7 @@ void free_portfolio(art_portfolio* p) {
 // The variant of a call over n_trials trials of k events (k = 0: a CSR, whose
 // length is on the device: 500 events per trial are assumed). ids NULL: they
 // will be staged on the device.
-int resolve_variant(const art_portfolio* p, int64_t n_trials, const int32_t* ids, int32_t k) {
+int resolve_variant(const art_portfolio* p, int64_t n_trials, const int32_t* ids, int32_t k, cudaStream_t s) {
     if (p->variant != ART_VARIANT_AUTO) return p->variant;
     // tables of whole numbers: a pass takes about 3.2 ps per event and run of
     // 8 layers where the sparse variant takes 12 (64 layers over 256 ELTs), after
@@ -633,7 +633,8 @@ int resolve_variant(const art_portfolio* p, int64_t n_trials, const int32_t* ids
     // events per catalogue event on
     const bool whole = !p->ogroups.empty() && std::all_of(p->ogroups.begin(), p->ogroups.end(),
                                                           [](const OccGroupArgs& g) { return g.sum_fits > 0; });
-    if (whole && (double)n_trials * (k > 0 ? k : 500) >= 5.0 * p->catalogue && ids_on_device(ids))
+    if (whole && (double)n_trials * (k > 0 ? k : 500) >= 5.0 * p->catalogue && ids_on_device(ids) &&
+        !captured_by_caller(p, s))
         return ART_VARIANT_SKIP;
     // few groups: the YET is streamed once per group, each event row read
     // only when its bit is set; many groups: one pass over a pool table
@@ -905,7 +906,7 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
     if (st) return st;
     if (n_trials == 0) return ART_OK;
     if (!ylt_dev) return ART_EINVAL;
-    const int variant = resolve_variant(p, n_trials, event_ids_dev, trial_off_dev ? 0 : events_per_trial);
+    const int variant = resolve_variant(p, n_trials, event_ids_dev, trial_off_dev ? 0 : events_per_trial, stream);
     if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     YetArgs y{event_ids_dev, trial_off_dev, n_trials, trial_off_dev ? 0 : events_per_trial, p->catalogue};
     cudaError_t e;
@@ -924,7 +925,9 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
             cudaGraph_t g = nullptr;
             e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
             if (!e) {
+                p->own_capture = true;
                 const cudaError_t le = run_forward(p, variant, y, ylt_dev, branch_dev, cap);
+                p->own_capture = false;
                 e = cudaStreamEndCapture(cap, &g);
                 if (!e) e = le;
             }
@@ -1010,7 +1013,7 @@ art_status host_run(art_portfolio* p, int64_t n_trials, const int32_t* event_ids
         for (int64_t t = 0; t < n_trials; ++t)
             if (trial_off_host[t + 1] < trial_off_host[t]) return ART_EINVAL;
     }
-    const int variant = resolve_variant(p, n_trials, nullptr, trial_off_host ? 0 : events_per_trial);
+    const int variant = resolve_variant(p, n_trials, nullptr, trial_off_host ? 0 : events_per_trial, stream);
     if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     if (!(p->flags & ART_FLAG_HOST_STAGED) && one_pass_over_ids(p, variant)) {
         const int32_t* d_ids = device_alias(event_ids_host);

@@ -409,6 +409,7 @@ struct art_portfolio {
     size_t host_scratch_cap = 0;
 
     // cached graph of one batched launch
+    bool own_capture = false;  // the library itself is capturing (its graph is dropped when terms change)
     cudaGraphExec_t graph_exec = nullptr;
     const void* graph_key[4] = {nullptr, nullptr, nullptr, nullptr};
     int64_t graph_key_n[2] = {0, 0};
@@ -430,6 +431,11 @@ cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t
 // unit 2^e; the largest they can be, in units.
 bool whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units);
 bool ids_on_device(const int32_t* ids);
+// Whether a caller is capturing the stream. Its graph may be replayed after
+// art_update_terms, and the FP32 tables' builds read the terms when they run:
+// a captured call keeps those (whole numbers need the pass's units and the
+// build's to agree).
+bool captured_by_caller(const art_portfolio* p, cudaStream_t s);
 // One occurrence group's trial pass over an X of whole numbers (lp slots per row).
 cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, int num_sms, bool early, double* ylt,
                                uint8_t* branch, int* flags, cudaStream_t s);

@@ -352,7 +352,11 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
                     : (fold ? payouts_fixed_kernel<false, true> : payouts_fixed_kernel<false, false>);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
     char* w = nullptr;
-    if ((e = scratch_alloc((void**)&w, xb + sizeof(uint32_t) * padded, s))) return e;
+    if ((e = scratch_alloc((void**)&w, xb + sizeof(uint32_t) * padded, s))) {
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();  // no room for the table: the other form needs none
+        return cudaSuccess;
+    }
     uint32_t* x = reinterpret_cast<uint32_t*>(w);
     uint32_t* bits = reinterpret_cast<uint32_t*>(w + xb);
     a.x = x;

@@ -814,13 +814,22 @@ bool ids_on_device(const int32_t* ids) {
     return a.type == cudaMemoryTypeDevice;
 }
 
+bool captured_by_caller(const art_portfolio* p, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();  // another stream's capture forbids the legacy stream: the launch will say so
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone && !p->own_capture;
+}
+
 cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                         bool build) {
     const bool early = (p->flags & ART_FLAG_EARLY_EXIT) != 0;
     // tables of whole numbers where the ids lie in device memory (the pass
     // over them brings the ids by bulk copies); ids read in place from host
     // memory keep the FP32 tables and the loads of the pass below
-    const bool whole = ids_on_device(y.ids);
+    const bool whole = ids_on_device(y.ids) && !captured_by_caller(p, s);
     // steps 2-3 once per catalogue event, with the terms as they are now
     cudaError_t err = build ? build_occurrence(p, whole, s) : cudaSuccess;
     if (err != cudaSuccess || y.n_trials == 0) return err;

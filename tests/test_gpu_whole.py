@@ -93,6 +93,59 @@ def test_skip_sums_are_exact(n_layers, catalogue):
         port.close()
 
 
+@pytest.mark.parametrize("n_layers", [1, 8])
+def test_long_trials(n_layers):
+    """Trials of more than 2^20 events: the lanes' counts outgrow the short
+    reduction."""
+    w, rng = _case(n_layers, 97, seed=41)
+    p = w.portfolio
+    p.agg_ret[:] *= 1e4
+    p.agg_lim[:] *= 1e5
+    o = _occ_losses(p)
+    k = (1 << 20) + 1237
+    ids = rng.integers(0, 97, size=3 * k, dtype=np.int32)
+    port = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER, variant=art.ART_VARIANT_SKIP)
+    try:
+        y = torch.empty((n_layers, 3), dtype=torch.float64, device="cuda")
+        art.art_run_ylt(port, 3, torch.from_numpy(ids).cuda(), None, k, y)
+        # the FP64 sum of whole numbers of one unit: exact below 2^53 units
+        np.testing.assert_array_equal(y.cpu().numpy(), _expected(o, p, ids, np.arange(4) * k))
+    finally:
+        port.close()
+
+
+@pytest.mark.parametrize("variant", ["ART_VARIANT_SKIP", "ART_VARIANT_FP64", "ART_VARIANT_AUTO"])
+def test_captured_call_takes_new_occurrence_terms(variant):
+    """A call captured by the caller and replayed after art_update_terms builds
+    its tables from the terms as they are then, whatever their units."""
+    w, rng = _case(17, 5000, seed=3)
+    p = w.portfolio
+    ids = torch.from_numpy(rng.integers(0, 5000, size=400 * 100, dtype=np.int32)).cuda()
+    port = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER | art.ART_LAYOUT_SPARSE | art.ART_LAYOUT_OCC64,
+                                       variant=getattr(art, variant))
+    try:
+        y = torch.zeros((17, 400), dtype=torch.float64, device="cuda")
+        want = torch.zeros_like(y)
+        art.art_run_ylt(port, 400, ids, None, 100, y)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            art.art_run_ylt(port, 400, ids, None, 100, y)
+        m, d, l, t = art.art_get_terms(port)
+        t2 = t.copy()
+        t2[:, 0] *= 37.0
+        t2[:, 1] = np.where(np.arange(17) % 2 == 0, t[:, 1] * 900.0, np.inf)
+        for terms in (t, t2, t):
+            art.art_update_terms(port, terms=terms)
+            y.fill_(-1.0)
+            g.replay()
+            art.art_run_ylt(port, 400, ids, None, 100, want)
+            torch.cuda.synchronize()
+            np.testing.assert_allclose(y.cpu().numpy(), want.cpu().numpy(), rtol=1e-11, atol=1e-9)
+    finally:
+        port.close()
+
+
 def test_unbounded_losses_keep_the_fp32_tables():
     """A group with a layer whose losses are not bounded takes the compensated
     pass; the other groups' results stay exact."""
