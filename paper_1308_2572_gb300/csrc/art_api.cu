@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <limits>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -572,9 +573,39 @@ size_t batched_smem(const art_portfolio* p, bool fp64) {
     return 3 * (size_t)p->pool_np * (fp64 ? 8 : 4) + (size_t)p->n_tiles * p->pool_np * 32;
 }
 
+// The persisting L2 area is reserved while a portfolio with ART_FLAG_L2_PERSIST
+// lives: every other access of the process has that much less L2 (payouts of
+// 100,000 trials 0.84 against 0.35 ms). The last one puts back the limit that
+// the first found, and demotes the lines that the passes left persisting.
+std::mutex g_persist_mutex;
+struct PersistArea {
+    int users = 0;
+    size_t before = 0;
+} g_persist[64];  // per device
+
+cudaError_t reserve_persisting(int device, size_t bytes) {
+    std::lock_guard<std::mutex> lock(g_persist_mutex);
+    PersistArea& a = g_persist[device & 63];
+    cudaError_t e;
+    if (a.users == 0 && (e = cudaDeviceGetLimit(&a.before, cudaLimitPersistingL2CacheSize))) return e;
+    if ((e = cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, bytes))) return e;
+    ++a.users;
+    return cudaSuccess;
+}
+
+void release_persisting(int device) {
+    std::lock_guard<std::mutex> lock(g_persist_mutex);
+    PersistArea& a = g_persist[device & 63];
+    int current = -1;
+    if (--a.users || cudaGetDevice(&current) != cudaSuccess || current != device) return;
+    cudaCtxResetPersistingL2Cache();
+    cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, a.before);
+}
+
 void free_portfolio(art_portfolio* p) {
     if (!p) return;
     cudaDeviceSynchronize();
+    if (p->persisted) release_persisting(p->device);
     for (float* t : p->layer_tab) cudaFree(t);
     for (float* t : p->group_tab) cudaFree(t);
     for (uint32_t* b : p->group_bitmap) cudaFree(b);
@@ -812,7 +843,10 @@ art_status art_create_portfolio(int32_t catalogue_size, int32_t n_elt, const flo
         if (p->flags & ART_FLAG_L2_PERSIST) {
             int persist_max = 0;
             cudaDeviceGetAttribute(&persist_max, cudaDevAttrMaxPersistingL2CacheSize, p->device);
-            if (persist_max > 0 && (e = cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, (size_t)persist_max))) break;
+            if (persist_max > 0) {
+                if ((e = reserve_persisting(p->device, (size_t)persist_max))) break;
+                p->persisted = true;
+            }
         }
         e = cudaStreamSynchronize(stream);
     } while (0);

@@ -320,6 +320,7 @@ struct art_portfolio {
     int32_t layouts = 0, variant = ART_VARIANT_AUTO, flags = 0;
     int32_t trial_tile = 0, cta_threads = 0;
     int num_sms = 0;
+    bool persisted = false;  // created with ART_FLAG_L2_PERSIST: its passes leave persisting lines in L2
 
     // terms as applied (after rounding)
     std::vector<float> mult, ded, lim, occ_ret, occ_lim;

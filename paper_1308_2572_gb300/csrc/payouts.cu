@@ -158,8 +158,9 @@ __device__ __forceinline__ double units_f64(uint32_t u, float unit) {
     return u ? __hiloint2double((int)((f >> 3) + 0x38000000u), (int)(f << 29)) : 0.0;
 }
 
+// Streaming stores: the payouts must not push the table out of L2.
 __device__ __forceinline__ void st_payouts4(double* p, const double (&v)[4]) {
-    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+    asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
                  : "memory");
 }
 
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
                     } else {
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
-                            if (d + i >= cur.head() && d + i < cur.n) pay[d + i] = v[i];
+                            if (d + i >= cur.head() && d + i < cur.n) __stcs(pay + d + i, v[i]);
                     }
                 }
             }
