@@ -630,7 +630,7 @@ cudaError_t launch_lt(const art_portfolio* p, const GroupArgs& g, const GroupInd
 cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& yet, const uint8_t* branch, const double* g,
                                   double* grad_terms, double* grad_mult, cudaStream_t s) {
     YetArgs y = yet;
-    y.by_id = !ids_on_device(y.ids);
+    y.by_id = !ids_on_device(y);
     const size_t C = (size_t)p->catalogue;
     const size_t rec_bytes = sizeof(AdjRecord) * C;
     const size_t bit_bytes = 16 * ((C / 32 + 1 + 3) / 4);

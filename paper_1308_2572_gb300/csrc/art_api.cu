@@ -1141,6 +1141,7 @@ art_status host_run(art_portfolio* p, int64_t n_trials, const int32_t* event_ids
         YetArgs y{p->stage_ids[slot] - i0, trial_off_host ? p->stage_off[slot] : nullptr, nt,
                   trial_off_host ? 0 : events_per_trial, p->catalogue};
         if (!trial_off_host) y.ids = p->stage_ids[slot];
+        y.staged = true;
         if ((e = run_forward(p, variant, y, p->stage_ylt[slot], nullptr, stream, !tables))) break;
         if (ylt_dev && (e = cudaMemcpy2DAsync(ylt_dev + t0, sizeof(double) * n_trials, p->stage_ylt[slot],
                                               sizeof(double) * nt, sizeof(double) * nt, p->n_layers,

@@ -68,6 +68,8 @@ struct YetArgs {
     int32_t k;            // events per trial when dense
     int32_t catalogue;
     bool by_id = false;   // ids to be read one by one (not in device memory: no bulk copies)
+    bool staged = false;  // ids of a chunk that the library copied to the device itself: `ids` is then
+                          // shifted back by the chunk's first index and may point outside any allocation
 };
 
 __device__ __forceinline__ void trial_range(const YetArgs& y, int64_t t, int64_t& b, int64_t& e, bool& bad) {
@@ -432,6 +434,7 @@ cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t
 // unit 2^e; the largest they can be, in units.
 bool whole_losses(float occ_ret, float occ_lim, double elt_lim_sum, int* e, double* max_units);
 bool ids_on_device(const int32_t* ids);
+inline bool ids_on_device(const YetArgs& y) { return y.staged || ids_on_device(y.ids); }
 // Whether a caller is capturing the stream. Its graph may be replayed after
 // art_update_terms, and the FP32 tables' builds read the terms when they run:
 // a captured call keeps those (whole numbers need the pass's units and the

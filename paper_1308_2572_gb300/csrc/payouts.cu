@@ -323,7 +323,7 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
     int e2;
     double top;
     const double events = (double)y.n_trials * (y.off ? 500.0 : (double)y.k);
-    if (events < 0.5 * p->catalogue || !ids_on_device(y.ids) ||
+    if (events < 0.5 * p->catalogue || !ids_on_device(y) ||
         !whole_losses(la.occ_ret, la.occ_lim, lims, &e2, &top))
         return cudaSuccess;
     PayArgs a;

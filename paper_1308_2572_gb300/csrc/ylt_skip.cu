@@ -829,7 +829,7 @@ cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t
     // tables of whole numbers where the ids lie in device memory (the pass
     // over them brings the ids by bulk copies); ids read in place from host
     // memory keep the FP32 tables and the loads of the pass below
-    const bool whole = ids_on_device(y.ids) && !captured_by_caller(p, s);
+    const bool whole = ids_on_device(y) && !captured_by_caller(p, s);
     // steps 2-3 once per catalogue event, with the terms as they are now
     cudaError_t err = build ? build_occurrence(p, whole, s) : cudaSuccess;
     if (err != cudaSuccess || y.n_trials == 0) return err;

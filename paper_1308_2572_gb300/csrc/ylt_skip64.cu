@@ -704,7 +704,7 @@ cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8
     // per-layer tables
     const bool csr = p->sp_ptr && p->d_slotmask64 && p->d_elt_terms64 && p->d_occ;
     const SparseEntry* en = reinterpret_cast<const SparseEntry*>(p->sp_entries);
-    const bool whole = p->whole64 && ids_on_device(y.ids) && !captured_by_caller(p, s);
+    const bool whole = p->whole64 && ids_on_device(y) && !captured_by_caller(p, s);
     if (build && whole && csr) {
         const dim3 tiles((unsigned)(((int64_t)words * 32 + kTileEvents - 1) / kTileEvents),
                          (unsigned)((p->ogroups64.size() * p->og_lp64 + kTileSlots - 1) / kTileSlots));
