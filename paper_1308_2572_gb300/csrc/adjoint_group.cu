@@ -37,9 +37,12 @@
 //   - the multipliers: for each (column k, layers S, loss l) of the record the
 //     lane adds l * W[S] to its own FP32 partial of column k in shared memory,
 //     W[S] = sum_{j in S} g_j a_j from two 16-entry tables of the trial's
-//     weights; every kFold batches the partials are summed across the warp
-//     (recursive halving: 31 shuffles for every column at once) and lane k adds
-//     column k's total to its compensated FP32 pair.
+//     weights; at the end of the trial, and every kFold batches of a long one,
+//     the partials are summed across the warp (recursive halving) and lane k
+//     adds column k's total to its compensated FP32 pair. Partials that run on
+//     over many trials cost precision: with a fold every 32 batches only,
+//     2,000,000 trials of 12 events ended 2-9 times as far from the FP64 sums
+//     as with one per trial, which takes 2% of the call (c3).
 // A trial with no layer on the middle branch costs only its branch codes. The
 // lane values are reduced warp -> CTA -> grid in a fixed order (no atomics:
 // deterministic); FP64 arithmetic runs only in that final reduction. Rounding:
@@ -67,7 +70,7 @@ namespace {
 template <int NP>
 constexpr int kAgWarpsFor = NP <= 16 ? 20 : 16;
 constexpr int kAgIds = 8;     // ids per lane and chunk
-constexpr int kFold = 32;     // batches between the folds of the column partials
+constexpr int kFold = 32;     // batches of one trial between the folds of the column partials
 constexpr uint32_t kOverflow = 7u;  // more than three columns: evaluated from the table row
 
 // What the trial pass reads of an event.
@@ -335,14 +338,16 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
         return t;
     };
 
-    // the lanes' partials summed across the warp by recursive halving (31
-    // shuffles for all columns): at distance o a lane keeps the half of its
-    // columns selected by bit o of its index and adds the partner's copy of
-    // that half; lane k ends with column k
+    // the lanes' partials summed across the warp by recursive halving: at
+    // distance o a lane keeps the half of its columns selected by bit o of its
+    // index and adds the partner's copy of that half, so that lane k (and the
+    // lanes that share its low bits) ends with column k; 31 shuffles for 32
+    // columns, 16 for 16
     auto fold_columns = [&]() {
-        float v[32];
+        constexpr int FC = NP <= 4 ? 4 : NP <= 8 ? 8 : NP <= 16 ? 16 : 32;
+        float v[FC];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
+        for (int k = 0; k < FC; ++k) {
             v[k] = 0.0f;
             if (k < NP) {
                 v[k] = part[32 * k];
@@ -350,7 +355,7 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
             }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = FC / 2; o > 0; o >>= 1) {
             const bool upper = (lane & o) != 0;
 #pragma unroll
             for (int i = 0; i < o; ++i) {
@@ -359,6 +364,8 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
                 v[i] = keep + __shfl_xor_sync(kFull, send, o);
             }
         }
+#pragma unroll
+        for (int o = 16; o >= FC; o >>= 1) v[0] += __shfl_xor_sync(kFull, v[0], o);
         if (lane < NP) two_sum_add(col_h, col_l, v[0]);
     };
 
@@ -370,7 +377,7 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
     ids.request(cur, 0, lane);
     bool lost = false;
     uint32_t unused_max = 0;  // ids outside the catalogue were reported by the forward
-    int folds = 0;            // batches since the partials were folded
+    int folds = 0;            // batches of the trial since the partials were folded
     while (t < y.n_trials && !lost) {
         const bool mid_l = cw.code == 1 && cw.g != 0.0f;
         const float gt = cw.g;
@@ -501,8 +508,9 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
         }
         ring.head = ring.tail;
         add_record(rec, rec_id);
-        folds += 1;
         __syncwarp();
+        fold_columns();  // every trial: a partial that ran on over many short trials would lose bits
+        folds = 0;
         flush_counts();
         if (lost) break;
         t = tn;
