@@ -518,11 +518,7 @@ __global__ void __launch_bounds__(32 * kAgWarpsFor<NP>, 1)
         cw = nw;
     }
     fold_columns();
-    if (lost) {
-        ids.phase ^= 1u;
-        ids.wait();  // the copy in flight may still come: shared memory stays until then
-        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
-    }
+    if (lost) ids.give_up(flags, lane);
     __syncthreads();
     double* s_red = reinterpret_cast<double*>(s_part);  // [NWARP][W]
     // the lane values in FP64, reduced warp -> CTA in a fixed order

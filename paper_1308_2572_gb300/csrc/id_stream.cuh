@@ -86,7 +86,7 @@ struct Trials {
 // shared memory by bulk copies (TMA), one in flight while the chunk before it
 // is processed from registers. Loads of the ids through L1 would share its
 // in-order return path with the gathers, which then wait for DRAM instead of
-// L2 (c1 forward 1.27 ms with 16-byte loads of the ids, XX with the copies).
+// L2.
 template <int E>
 struct IdStream {
     uint32_t bar, buf;  // shared-memory addresses of the warp's barrier and buffer
@@ -126,16 +126,25 @@ struct IdStream {
             : "memory");
         return ok != 0;
     }
-    // Wait for the requested chunk; false when it has not come in time.
-    __device__ __forceinline__ bool wait() {
+    // Wait for the requested chunk; false when it has not come in time, for the
+    // whole warp: each lane polls and reads the clock by itself, and lanes that
+    // disagreed would part before the pass's next vote.
+    __device__ __forceinline__ bool wait(uint64_t limit_ns = kWaitNs) {
         bool ok = arrived();
         if (!ok) {
             const uint64_t t0 = now_ns();
-            while (!(ok = arrived()) && now_ns() - t0 < kWaitNs) {
+            while (!(ok = arrived()) && now_ns() - t0 < limit_ns) {
             }
         }
         phase ^= 1u;
-        return ok;
+        return __all_sync(kFull, ok);
+    }
+    // The end of a pass whose wait gave up: the copy in flight may still come,
+    // and shared memory stays until then (again with a limit).
+    __device__ __forceinline__ void give_up(int* flags, int lane, uint64_t limit_ns = kWaitNs) {
+        phase ^= 1u;
+        wait(limit_ns);
+        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
     }
     // The ids of the chunk from position c0 of a span with c0 < n: slot
     // 4 h + i of a lane is position c0 + 128 h + 4 lane + i. What positions

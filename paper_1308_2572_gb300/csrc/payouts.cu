@@ -289,11 +289,7 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
         cur = nxt;
     }
     flush();
-    if (lost) {
-        ids.phase ^= 1u;
-        ids.wait();  // the copy in flight may still come: shared memory stays until then
-        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
-    }
+    if (lost) ids.give_up(flags, lane);
     if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
     if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
 }

@@ -14,7 +14,7 @@
 // launch reads the same addresses.
 #include <algorithm>
 
-#include "art_internal.cuh"
+#include "id_stream.cuh"
 
 namespace art {
 namespace {
@@ -88,10 +88,36 @@ __global__ void fp64_kernel(int iters, double* sink) {
     if (s == -1.0) *sink = s;
 }
 
+// Warps that wait for a copy nobody requested, each lane with a limit of its
+// own, and end as a trial pass does.
+__global__ void __launch_bounds__(128) wait_kernel(uint64_t limit_ns, int* __restrict__ flags,
+                                                   int* __restrict__ disagree) {
+    __shared__ __align__(512) uint32_t s_ids[4 * 32 * 4];
+    __shared__ __align__(8) uint64_t s_bars[4];
+    const int lane = threadIdx.x & 31;
+    IdStream<4> ids;
+    ids.init(s_bars, s_ids, threadIdx.x >> 5, lane);
+    const bool ok = ids.wait(limit_ns * (1 + (lane & 3)));
+    if (__any_sync(kFull, ok != __shfl_sync(kFull, ok, 0)) && lane == 0) atomicOr(disagree, 1);
+    if (!ok) ids.give_up(flags, lane, limit_ns);
+}
+
 }  // namespace
 }  // namespace art
 
 using namespace art;
+
+// For the tests, not part of the C ABI: a bounded wait that runs out, reported
+// through the portfolio's status as a trial pass reports it. *disagree_dev is
+// set when the lanes of a warp did not all get the same answer.
+extern "C" __attribute__((visibility("default"))) art_status art_test_wait(art_portfolio* p, uint64_t limit_ns,
+                                                                          int* disagree_dev, cudaStream_t stream) {
+    if (!p || !disagree_dev || limit_ns > 100000000ULL) return ART_EINVAL;
+    wait_kernel<<<8, 128, 0, stream>>>(limit_ns, p->d_flags, disagree_dev);
+    const cudaError_t e = cudaGetLastError();
+    if (e) set_last_error(e);
+    return e ? ART_ECUDA : ART_OK;
+}
 
 extern "C" art_status art_probe(int32_t kind, int64_t bytes, int32_t reps, double* result) {
     if (!result || reps < 1 || kind < ART_PROBE_STREAM || kind > ART_PROBE_FP64ADD) return ART_EINVAL;

@@ -239,11 +239,7 @@ __global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_narrow_ker
         cur = nxt;
     }
     flush();
-    if (lost) {
-        ids.phase ^= 1u;
-        ids.wait();  // the copy in flight may still come: shared memory stays until then
-        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
-    }
+    if (lost) ids.give_up(flags, lane);
     if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
     if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
 }
@@ -353,11 +349,7 @@ __global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_wide_kerne
         t = tn;
         cur = nxt;
     }
-    if (lost) {
-        ids.phase ^= 1u;
-        ids.wait();  // the copy in flight may still come: shared memory stays until then
-        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
-    }
+    if (lost) ids.give_up(flags, lane);
     if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
     if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
 }

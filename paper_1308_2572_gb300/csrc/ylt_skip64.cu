@@ -470,11 +470,7 @@ __global__ void __launch_bounds__(32 * k64FxWarps<LT, VEC>, 1)
         t = tn;
         cur = nxt;
     }
-    if (lost) {
-        ids.phase ^= 1u;
-        ids.wait();  // the copy in flight may still come: shared memory stays until then
-        if (lane == 0) atomicOr(flags + kFlagTimeout, 1);
-    }
+    if (lost) ids.give_up(flags, lane);
     if (max_id >= C) atomicOr(flags + kFlagIdRange, 1);
     if (lane == 0 && trials.bad) atomicOr(flags + kFlagBadOffsets, 1);
 }
