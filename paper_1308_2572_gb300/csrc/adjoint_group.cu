@@ -607,7 +607,7 @@ cudaError_t launch_one(const art_portfolio* p, const GroupArgs& g, const GroupIn
     const bool vec = !y.by_id && !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
     auto kern = vec ? (fold ? adjoint_pass_kernel<NP, LT, true, true> : adjoint_pass_kernel<NP, LT, true, false>)
                     : (fold ? adjoint_pass_kernel<NP, LT, false, true> : adjoint_pass_kernel<NP, LT, false, false>);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     // a CTA's warps take neighbouring trials (they share the sectors of the
     // branch codes and weights); few trials are spread over the SMs instead
     const bool many = y.n_trials >= (int64_t)p->num_sms * NWARP;

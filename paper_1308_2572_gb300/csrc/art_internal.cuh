@@ -489,6 +489,19 @@ int64_t tail_count(double p, int64_t n);
 
 void set_last_error(cudaError_t e);
 
+// Lets a kernel without static shared memory be launched with all the shared
+// memory that a block may have. The limit belongs to the function on the
+// device, not to the call, so every call sets this one value: a thread that set
+// the size of its own launch could lower another's between its setting and
+// its launch.
+template <class K>
+cudaError_t allow_max_shared(K* kern) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+}
+
 // Stream-ordered scratch of one call (release it with cudaFreeAsync), from a
 // pool that keeps a bounded amount between calls (scratch.cu).
 cudaError_t scratch_alloc(void** out, size_t bytes, cudaStream_t s);

@@ -867,7 +867,9 @@ cudaError_t launch_metric_kernels(const double* ylt, int64_t n, int32_t n_layers
     auto pass_k = n_p <= 1 ? pass_kernel<1> : n_p <= 2 ? pass_kernel<2> : n_p <= 4 ? pass_kernel<4> : pass_kernel<8>;
     auto tail_k = n_p <= 1 ? tail_kernel<1> : n_p <= 2 ? tail_kernel<2> : n_p <= 4 ? tail_kernel<4> : tail_kernel<8>;
     const size_t shm = sizeof(unsigned int) * (size_t)n_p * kMaxBins;
-    if (shm > 48 * 1024 && (err = cudaFuncSetAttribute(pass_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)))
+    // the limit is the function's, not the call's: every call sets the same (as allow_max_shared)
+    if (shm > 48 * 1024 && (err = cudaFuncSetAttribute(pass_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)sizeof(unsigned int) * kMaxProbs * kMaxBins)))
         return err;
     // pass 2, then one launch per digit a layer's list may still need
     for (int i = 0; i < kPasses; ++i) {

@@ -496,7 +496,10 @@ cudaError_t metrics_list_run(const double* ylt, int64_t n, int32_t n_layers, con
     }
     cudaError_t e;
     const int smem = (int)(sizeof(u64) * std::min<int64_t>(n, kSmall));
-    if ((e = cudaFuncSetAttribute(list_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    // the limit is the function's, not the call's: every call sets the same (as allow_max_shared)
+    if ((e = cudaFuncSetAttribute(list_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(u64) * kSmall)))
+        return e;
     ListState* st = nullptr;
     u64* lists = nullptr;
     const unsigned int cap = list_cap(n);

@@ -347,7 +347,7 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
         ((reinterpret_cast<uintptr_t>(payouts) >> 3) - (reinterpret_cast<uintptr_t>(y.ids) >> 2)) % 4 == 0;
     auto kern = vec ? (fold ? payouts_fixed_kernel<true, true> : payouts_fixed_kernel<true, false>)
                     : (fold ? payouts_fixed_kernel<false, true> : payouts_fixed_kernel<false, false>);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     char* w = nullptr;
     if ((e = scratch_alloc((void**)&w, xb + sizeof(uint32_t) * padded, s))) {
         if (e != cudaErrorMemoryAllocation) return e;

@@ -219,7 +219,7 @@ static cudaError_t launch_cfg(art_portfolio* p, const BatchedArgs& a, const YetA
                               uint8_t* branch, cudaStream_t s) {
     auto kern = ylt_batched_kernel<V, EPL, SLOTS, U>;
     const size_t smem = 3 * (size_t)(32 * EPL) * sizeof(V) + (size_t)a.n_tiles * (32 * EPL) * 32;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_max_shared(kern);
     if (err != cudaSuccess) return err;
     const int threads = (p->cta_threads > 0 && p->cta_threads <= 256) ? p->cta_threads : 256;
     int per_sm = 0;

@@ -397,7 +397,7 @@ cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, 
     const FixedKernel kern = vec ? (fold ? pick_kernel<true, true>(lp, pre4) : pick_kernel<true, false>(lp, pre4))
                                  : (fold ? pick_kernel<false, true>(lp, pre4) : pick_kernel<false, false>(lp, pre4));
     if (!kern) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(num_sms, y.n_trials));
     kern<<<(unsigned)grid, 32 * warps, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
     return cudaGetLastError();

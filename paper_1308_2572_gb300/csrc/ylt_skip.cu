@@ -738,7 +738,7 @@ cudaError_t launch_group(const OccGroupArgs& g, const YetArgs& y, int num_sms, i
     const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
     auto kern = vec ? (fold ? ylt_skip_kernel<LT, LP, true, COMPACT, true> : ylt_skip_kernel<LT, LP, true, COMPACT, false>)
                     : (fold ? ylt_skip_kernel<LT, LP, false, COMPACT, true> : ylt_skip_kernel<LT, LP, false, COMPACT, false>);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     const int64_t grid = std::min<int64_t>(num_sms, (y.n_trials + kSkipWarps - 1) / kSkipWarps);
     kern<<<(unsigned)std::max<int64_t>(1, grid), kSkipThreads, smem, s>>>(g, y, smem_words, early, ylt, branch,
                                                                           flags);

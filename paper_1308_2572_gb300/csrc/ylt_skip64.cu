@@ -492,7 +492,7 @@ cudaError_t launch_fixed64(const OccGroupArgs& g, const YetArgs& y, int num_sms,
     const bool fold = words <= 2 * smem_words;
     auto kern = vec ? (fold ? fixed64_kernel<LT, true, true> : fixed64_kernel<LT, true, false>)
                     : (fold ? fixed64_kernel<LT, false, true> : fixed64_kernel<LT, false, false>);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(num_sms, y.n_trials));
     kern<<<(unsigned)grid, 32 * warps, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
     return cudaGetLastError();
@@ -683,7 +683,7 @@ cudaError_t launch_group64(const OccGroupArgs& g, const YetArgs& y, int num_sms,
     const bool vec = !y.off && y.k % 4 == 0 && (reinterpret_cast<uintptr_t>(y.ids) & 15) == 0;
     auto kern = vec ? (fold ? ylt_skip64_kernel<LT, true, true> : ylt_skip64_kernel<LT, true, false>)
                     : (fold ? ylt_skip64_kernel<LT, false, true> : ylt_skip64_kernel<LT, false, false>);
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
+    if ((e = allow_max_shared(kern))) return e;
     const int64_t grid = std::min<int64_t>(num_sms, (y.n_trials + k64Warps - 1) / k64Warps);
     kern<<<(unsigned)std::max<int64_t>(1, grid), k64Threads, smem, s>>>(g, y, smem_words, early, ylt, branch, flags);
     return cudaGetLastError();

@@ -187,7 +187,7 @@ cudaError_t launch_scatter(art_portfolio* p, const SparseArgs& a, const YetArgs&
     int warps = (p->cta_threads > 0 && p->cta_threads <= kSparseThreads) ? p->cta_threads / 32 : kSparseThreads / 32;
     while (warps > 1 && base + warps * per_warp > 100 * 1024) --warps;  // at least two CTAs per SM
     const size_t smem = base + warps * per_warp;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_max_shared(kern);
     if (err != cudaSuccess) return err;
     const int threads = 32 * warps;
     int per_sm = 0;
@@ -323,7 +323,7 @@ cudaError_t launch_bcast(art_portfolio* p, const SparseArgs& a, const YetArgs& y
                          cudaStream_t s) {
     auto kern = ylt_sparse_bcast_kernel<SLOTS>;
     const size_t smem = (size_t)a.pool_np * sizeof(float4) + (size_t)a.n_tiles * a.pool_np * 32;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_max_shared(kern);
     if (err != cudaSuccess) return err;
     const int threads = (p->cta_threads > 0 && p->cta_threads <= kSparseThreads) ? p->cta_threads : kSparseThreads;
     int per_sm = 0;
