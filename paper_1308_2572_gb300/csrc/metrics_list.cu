@@ -285,6 +285,8 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
     const unsigned int thr = max((unsigned int)(st[j].threshold >> 32), 1u);
     const unsigned int tie_hi = (unsigned int)(st[j].tie >> 32), tie_lo = (unsigned int)st[j].tie;
     const int ref = st[j].ref;
+    // no reference: every loss is out of the short sum's range, a subnormal too
+    const unsigned int dref = ref ? (unsigned int)ref : 0x7fffffffu;
     // The sum as four 32-bit words, the highest a carry: a key within 31
     // binades below ref is its mantissa at the top of 96 bits, shifted down
     // (three shifts and four adds; no bit is lost, so the unit is 2^-96 of
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
         unsigned in = 0, odd = 0;  // bit u: listed; summed the long way
 #pragma unroll
         for (int u = 0; u < kPassUnroll; ++u) {
-            const unsigned int d = (unsigned int)ref - (kh[u] >> 20);
+            const unsigned int d = dref - (kh[u] >> 20);
             const unsigned int hi = __funnelshift_l(kl[u], kh[u], 11) | 0x80000000u, lo = kl[u] << 11;
             const unsigned int x2 = hi >> (d & 31), x1 = __funnelshift_r(lo, hi, d), x0 = __funnelshift_r(0u, lo, d);
             asm("{\n.reg .pred p;\nsetp.lt.u32 p, %4, 32;\n"

@@ -47,3 +47,26 @@ def test_metrics_match_a_full_sort(n):
             np.testing.assert_allclose(got[2], ot, rtol=1e-12, atol=1e-320)
         for a, b in zip(outs[0], outs[2]):
             np.testing.assert_array_equal(a, b)  # repeatable bits
+
+
+@pytest.mark.parametrize("n", [26_625, 60_000, 300_001])
+def test_losses_below_the_normal_range(n):
+    """Losses whose high word is 0 (below 2^-1042), beside trials without a
+    loss and beside ordinary ones: selected and summed as any other."""
+    rng = np.random.default_rng(n)
+    tiny = 5e-324 * rng.integers(1, 1 << 31, n)
+    ln = rng.lognormal(15.0, 2.0, n)
+    y = np.stack([np.where(np.arange(n) % 50 == 0, tiny, 0.0), np.where(rng.random(n) < 0.004, tiny, 0.0), tiny,
+                  np.where(rng.random(n) < 0.3, ln, tiny), np.where(rng.random(n) < 0.001, ln, 0.0) + (np.arange(n) == 7) * 5e-324])
+    dev = torch.from_numpy(y).cuda()
+    for probs in ([0.99], [0.96, 0.999]):
+        L, n_p = y.shape[0], len(probs)
+        om, op, ot = oracle.metrics(y, probs)
+        mean = torch.full((L,), -1.0, dtype=torch.float64, device="cuda")
+        pml = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+        tvar = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+        art.art_metrics(dev, n, L, probs, mean, pml, tvar)
+        np.testing.assert_array_equal(pml.cpu().numpy(), op)
+        # the oracle's sums are exact here or round as above; a subnormal quotient rounds to its unit
+        np.testing.assert_allclose(mean.cpu().numpy(), om, rtol=1e-12, atol=1e-323)
+        np.testing.assert_allclose(tvar.cpu().numpy(), ot, rtol=1e-12, atol=1e-323)
