@@ -11,12 +11,16 @@
 //      tie key (the aggregate cap, the value that repeats most).
 //   2. pass (the only read of the YLT): each layer's exact sum, the number of
 //      losses equal to the tie key, and a list of the other losses >= T that
-//      are not 0.
+//      are not 0. Where the r-th largest of the sample repeats too (a layer
+//      whose events mostly pay their full limit: whole multiples of it), that
+//      value is a second tie key; listed, it took the list's room, and the
+//      finish read the row (1,000,000 trials at three probabilities: 5.3 ms).
 //   3. finish (one CTA per layer): the k-th largest of list and ties by a
 //      radix select in shared memory, the exact sum of the losses above it,
 //      mean, PML and TVaR. If the list holds fewer than k losses and T > 0, or
-//      overflowed, or a loss lay far above the sample's largest, the CTA takes
-//      the row instead: slower, the same results.
+//      overflowed, or some loss is subnormal beside T > 0, the CTA takes the row
+//      instead (for the sum alone where a loss lay far above the sample's
+//      largest): slower, the same results.
 // A YLT of at most kSmall trials skips 1 and 2: its rows fit shared memory.
 //
 // What bounds it: HBM (8 bytes per loss, once); the general path's two full
@@ -26,6 +30,7 @@
 // metrics 40 us against 90 (eight dependent launches).
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "art_internal.cuh"
 
@@ -44,6 +49,11 @@ constexpr int kPassUnroll = 8;       // values per thread whose loads are in fli
 constexpr u64 kNoTie = ~0ULL;
 constexpr int kBins = 2048;          // 11-bit digits
 constexpr int kDirect = 128;         // candidates that are ranked by comparison
+constexpr int kTies = 2;             // keys per layer that are counted, not listed
+constexpr unsigned kAtom = 32;       // sample keys in one of 2^22 bins that make a repeating key likely
+// why a layer's row is read again
+constexpr unsigned kSumOut = 1;      // a loss above the short sum's range: the sum only
+constexpr unsigned kUnlisted = 2;    // a loss that no list can hold (or no reference for any): everything
 
 struct Ranks {
     long long k[kMaxProbs];
@@ -53,12 +63,12 @@ struct Ranks {
 // Per-layer state, written by the sample.
 struct ListState {
     u64 threshold;   // T (its low word is 0)
-    u64 tie;         // the tie key (kNoTie: none)
+    u64 tie[kTies];  // the tie keys (kNoTie: none)
     u64 sum[2];      // fixed-point sum of the row (unit by ref)
-    u64 n_tie;
+    u64 n_tie[kTies];
     unsigned int n_list;
     int ref;         // reference exponent of the pass's sum; 0: the list holds every loss, sum that
-    unsigned int beyond;  // a loss with an exponent above ref was seen
+    unsigned int again;   // kSumOut, kUnlisted
     unsigned int pad;
 };
 
@@ -154,11 +164,15 @@ __device__ __forceinline__ void for_each_key(Get get, int64_t n, F f) {
     }
 }
 
-// The k-th largest (k >= 1) of the n keys that get(i) yields, of which tie
-// counts n_tie more times; n + n_tie >= k. Every thread of the block calls it
-// and receives it. MSD radix select over the offsets from the smallest key lo; once few candidates are left they are ranked directly.
+// Keys that a list leaves out, with their counts (0: none).
+struct Ties {
+    u64 key[kTies], n[kTies];
+};
+
+// The k-th largest (k >= 1) of the n keys that get(i) yields and of the ties;
+// they are k or more. Every thread of the block calls it and receives it. MSD radix select over the offsets from the smallest key lo; once few candidates are left they are ranked directly.
 template <class Get>
-__device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 hi, long long k, SelectScratch& s) {
+__device__ u64 kth_largest(Get get, int64_t n, const Ties& ties, u64 lo, u64 hi, long long k, SelectScratch& s) {
     int top = 64 - __clzll((long long)(hi - lo));  // bits of the largest offset
     u64 prefix = 0;                               // of the offset, in units of 2^top
     long long krem = k;
@@ -170,10 +184,13 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
             const u64 d = v - lo;
             if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], 1u);
         });
-        if (threadIdx.x == 0 && n_tie) {
-            const u64 d = tie - lo;
-            if ((d >> top) == prefix) atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], (unsigned)n_tie);
-        }
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int i = 0; i < kTies; ++i) {
+                const u64 d = ties.key[i] - lo;
+                if (ties.n[i] && (d >> top) == prefix)
+                    atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], (unsigned)ties.n[i]);
+            }
         __syncthreads();
         pick_bin(s, (unsigned int)krem);
         const u64 in_bin = s.hist[s.bin];
@@ -188,18 +205,20 @@ __device__ u64 kth_largest(Get get, int64_t n, u64 tie, u64 n_tie, u64 lo, u64 h
             });
             __syncthreads();
             const int m = (int)s.n_cand;
-            const bool tie_in = n_tie && ((tie - lo) >> top) == prefix;
-            for (int c = threadIdx.x; c < m + (tie_in ? 1 : 0); c += blockDim.x) {
-                const u64 v = c < m ? s.cand[c] : tie;
+            for (int c = threadIdx.x; c < m + kTies; c += blockDim.x) {
+                const u64 v = c < m ? s.cand[c] : c == m ? ties.key[0] : ties.key[1];
+                if (c >= m && !((c == m ? ties.n[0] : ties.n[1]) && ((v - lo) >> top) == prefix)) continue;
                 u64 gt = 0, ge = 0;
                 for (int j = 0; j < m; ++j) {
                     gt += s.cand[j] > v;
                     ge += s.cand[j] >= v;
                 }
-                if (tie_in) {
-                    gt += tie > v ? n_tie : 0ULL;
-                    ge += tie >= v ? n_tie : 0ULL;
-                }
+#pragma unroll
+                for (int i = 0; i < kTies; ++i)
+                    if (((ties.key[i] - lo) >> top) == prefix) {
+                        gt += ties.key[i] > v ? ties.n[i] : 0ULL;
+                        ge += ties.key[i] >= v ? ties.n[i] : 0ULL;
+                    }
                 if ((long long)gt < krem && krem <= (long long)ge) s.found = v;  // the same value from equal candidates
             }
             __syncthreads();
@@ -260,21 +279,53 @@ __global__ void __launch_bounds__(kFinishThreads) list_sample_kernel(const doubl
     }
     __syncthreads();
     pick_bin(s, (unsigned int)rank - above);
+    u64 threshold = (u64)(lo + (((b1 << (sh1 - sh2)) | (unsigned int)s.bin) << sh2)) << 32;
+    // Many sample keys in the r-th largest's bin: a value that repeats, such as
+    // one full limit of a layer whose events mostly pay theirs. Its exact key
+    // becomes a tie key too, or the list would take every one of it.
+    u64 atom = kNoTie;
+    if (s.hist[s.bin] > kAtom && threshold && repeats < (u64)rank) {
+        const u64 base = threshold;
+        const int width = sh2 + 32;
+        unsigned int krem = (unsigned int)rank - above - s.above, same = 0;
+        u64 prefix = 0;
+        for (int left = width; left > 0;) {
+            const int bits = min(11, left), shift = left - bits;
+            __syncthreads();
+            for (int i = threadIdx.x; i < kBins; i += kFinishThreads) s.hist[i] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const u64 d = v[i] - base;  // wraps below the bin
+                if (!(d >> width) && (d >> left) == prefix)
+                    atomicAdd(&s.hist[(d >> shift) & ((1u << bits) - 1)], 1u);
+            }
+            __syncthreads();
+            pick_bin(s, krem);
+            prefix = prefix << bits | (u64)s.bin;
+            krem -= s.above;
+            same = s.hist[s.bin];
+            left = shift;
+        }
+        threshold = (base + prefix) & ~0xffffffffULL;
+        if (same > 1) atom = base + prefix;
+    }
     if (threadIdx.x == 0) {
         ListState l{};
-        l.threshold = (u64)(lo + (((b1 << (sh1 - sh2)) | (unsigned int)s.bin) << sh2)) << 32;
-        l.tie = repeats > 1 && mx ? mx : kNoTie;
+        l.threshold = threshold;
+        l.tie[0] = repeats > 1 && mx ? mx : atom;
+        l.tie[1] = l.tie[0] != atom ? atom : kNoTie;
         // room for losses 4,096 times the sample's largest; the pass's short
         // fixed point wants as much below. T = 0: the list (and the ties) will
         // hold every loss but 0, and the finish sums it (a layer of few losses
         // has no sample to set a reference by)
         l.ref = l.threshold ? min(ref_exp(mx) + 12, 2046) : 0;
-        l.beyond = l.threshold && l.ref < 128 ? 1u : 0u;
+        l.again = l.threshold && l.ref < 128 ? kUnlisted : 0u;
         st[blockIdx.x] = l;
     }
 }
 
-__global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* __restrict__ ylt, int64_t n,
+__global__ void __launch_bounds__(kPassThreads, 5) list_pass_kernel(const double* __restrict__ ylt, int64_t n,
                                                                  ListState* __restrict__ st, u64* __restrict__ lists,
                                                                  unsigned int cap) {
     const int j = blockIdx.y;
@@ -283,7 +334,8 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
     u64* list = lists + (size_t)j * cap;
     // keys of a high word from thr on are listed; zeros never are
     const unsigned int thr = max((unsigned int)(st[j].threshold >> 32), 1u);
-    const unsigned int tie_hi = (unsigned int)(st[j].tie >> 32), tie_lo = (unsigned int)st[j].tie;
+    const unsigned int tie_hi = (unsigned int)(st[j].tie[0] >> 32), tie_lo = (unsigned int)st[j].tie[0];
+    const unsigned int tie2_hi = (unsigned int)(st[j].tie[1] >> 32), tie2_lo = (unsigned int)st[j].tie[1];
     const int ref = st[j].ref;
     // no reference: every loss is out of the short sum's range, a subnormal too
     const unsigned int dref = ref ? (unsigned int)ref : 0x7fffffffu;
@@ -294,80 +346,94 @@ __global__ void __launch_bounds__(kPassThreads) list_pass_kernel(const double* _
     // key (rare) goes the long way in `rest`.
     unsigned int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
     Fix rest{0, 0};
-    unsigned int n_tie = 0;
-    bool beyond = false;
-    for (int64_t i0 = (int64_t)blockIdx.x * kPassThreads * kPassUnroll; i0 < n;
-         i0 += (int64_t)gridDim.x * kPassThreads * kPassUnroll) {
-        unsigned int kh[kPassUnroll], kl[kPassUnroll];  // 0 past the end
-        if (i0 + kPassThreads * kPassUnroll <= n) {
+    unsigned int n_tie = 0, n_tie2 = 0;
+    unsigned int again = 0;
+    // two: the layer has a second tie key (few layers do; the others are
+    // spared its comparison)
+    auto read_row = [&](auto two) {
+        for (int64_t i0 = (int64_t)blockIdx.x * kPassThreads * kPassUnroll; i0 < n;
+             i0 += (int64_t)gridDim.x * kPassThreads * kPassUnroll) {
+            unsigned int kh[kPassUnroll], kl[kPassUnroll];  // 0 past the end
+            if (i0 + kPassThreads * kPassUnroll <= n) {
+#pragma unroll
+                for (int u = 0; u < kPassUnroll; ++u) {
+                    const u64 v = key_at(row, i0 + u * kPassThreads + threadIdx.x);
+                    kh[u] = (unsigned int)(v >> 32);
+                    kl[u] = (unsigned int)v;
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < kPassUnroll; ++u) {
+                    const int64_t i = i0 + (int64_t)u * kPassThreads + threadIdx.x;
+                    const u64 v = i < n ? key_at(row, i) : 0ULL;
+                    kh[u] = (unsigned int)(v >> 32);
+                    kl[u] = (unsigned int)v;
+                }
+            }
+            unsigned in = 0, odd = 0;  // bit u: listed; summed the long way
 #pragma unroll
             for (int u = 0; u < kPassUnroll; ++u) {
-                const u64 v = key_at(row, i0 + u * kPassThreads + threadIdx.x);
-                kh[u] = (unsigned int)(v >> 32);
-                kl[u] = (unsigned int)v;
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < kPassUnroll; ++u) {
-                const int64_t i = i0 + (int64_t)u * kPassThreads + threadIdx.x;
-                const u64 v = i < n ? key_at(row, i) : 0ULL;
-                kh[u] = (unsigned int)(v >> 32);
-                kl[u] = (unsigned int)v;
-            }
-        }
-        unsigned in = 0, odd = 0;  // bit u: listed; summed the long way
-#pragma unroll
-        for (int u = 0; u < kPassUnroll; ++u) {
-            const unsigned int d = dref - (kh[u] >> 20);
-            const unsigned int hi = __funnelshift_l(kl[u], kh[u], 11) | 0x80000000u, lo = kl[u] << 11;
-            const unsigned int x2 = hi >> (d & 31), x1 = __funnelshift_r(lo, hi, d), x0 = __funnelshift_r(0u, lo, d);
-            asm("{\n.reg .pred p;\nsetp.lt.u32 p, %4, 32;\n"
-                "@p add.cc.u32 %0, %0, %5;\n@p addc.cc.u32 %1, %1, %6;\n"
-                "@p addc.cc.u32 %2, %2, %7;\n@p addc.u32 %3, %3, 0;\n}"
-                : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3)
-                : "r"(d), "r"(x0), "r"(x1), "r"(x2));
-            if (d >= 32u && (kh[u] | kl[u])) odd |= 1u << u;
-            const bool eq = kh[u] == tie_hi && kl[u] == tie_lo;
-            n_tie += eq;
-            if (kh[u] >= thr && !eq) in |= 1u << u;
-        }
-        if (odd) {
-#pragma unroll
-            for (int u = 0; u < kPassUnroll; ++u)
-                if ((odd >> u) & 1u) {
-                    // a key above ref, or below what the list's threshold can tell from 0
-                    if (kh[u] == 0u || (ref && (int)(kh[u] >> 20) > ref)) beyond = true;
-                    else if (ref) fix_add(rest, (u64)kh[u] << 32 | kl[u], ref);
+                const unsigned int d = dref - (kh[u] >> 20);
+                const unsigned int hi = __funnelshift_l(kl[u], kh[u], 11) | 0x80000000u, lo = kl[u] << 11;
+                const unsigned int x2 = hi >> (d & 31), x1 = __funnelshift_r(lo, hi, d), x0 = __funnelshift_r(0u, lo, d);
+                asm("{\n.reg .pred p;\nsetp.lt.u32 p, %4, 32;\n"
+                    "@p add.cc.u32 %0, %0, %5;\n@p addc.cc.u32 %1, %1, %6;\n"
+                    "@p addc.cc.u32 %2, %2, %7;\n@p addc.u32 %3, %3, 0;\n}"
+                    : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3)
+                    : "r"(d), "r"(x0), "r"(x1), "r"(x2));
+                if (d >= 32u && (kh[u] | kl[u])) odd |= 1u << u;
+                const bool eq = kh[u] == tie_hi && kl[u] == tie_lo;
+                n_tie += eq;
+                bool eq2 = false;
+                if constexpr (decltype(two)::value) {
+                    eq2 = kh[u] == tie2_hi && kl[u] == tie2_lo;
+                    n_tie2 += eq2;
                 }
-        }
-        if (__any_sync(kAll, in != 0u)) {
-            // one counter update per warp and step: a scan of the lanes' counts
-            const unsigned c = __popc(in);
-            unsigned incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned v = __shfl_up_sync(kAll, incl, o);
-                if (lane >= (unsigned)o) incl += v;
+                if (kh[u] >= thr && !eq && !eq2) in |= 1u << u;
             }
-            unsigned base = 0;
-            if (lane == 31) base = atomicAdd(&st[j].n_list, incl);
-            base = __shfl_sync(kAll, base, 31) + incl - c;
+            if (odd) {
 #pragma unroll
-            for (int u = 0; u < kPassUnroll; ++u)
-                if ((in >> u) & 1u) {
-                    if (base < cap) list[base] = (u64)kh[u] << 32 | kl[u];
-                    ++base;
+                for (int u = 0; u < kPassUnroll; ++u)
+                    if ((odd >> u) & 1u) {
+                        // a key above ref, or below what the list's threshold can tell from 0
+                        if (kh[u] == 0u) again |= kUnlisted;
+                        else if (ref && (int)(kh[u] >> 20) > ref) again |= kSumOut;
+                        else if (ref) fix_add(rest, (u64)kh[u] << 32 | kl[u], ref);
+                    }
+            }
+            if (__any_sync(kAll, in != 0u)) {
+                // one counter update per warp and step: a scan of the lanes' counts
+                const unsigned c = __popc(in);
+                unsigned incl = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned v = __shfl_up_sync(kAll, incl, o);
+                    if (lane >= (unsigned)o) incl += v;
                 }
+                unsigned base = 0;
+                if (lane == 31) base = atomicAdd(&st[j].n_list, incl);
+                base = __shfl_sync(kAll, base, 31) + incl - c;
+#pragma unroll
+                for (int u = 0; u < kPassUnroll; ++u)
+                    if ((in >> u) & 1u) {
+                        if (base < cap) list[base] = (u64)kh[u] << 32 | kl[u];
+                        ++base;
+                    }
+            }
         }
-    }
+    };
+    if (st[j].tie[1] == kNoTie) read_row(std::false_type{});
+    else read_row(std::true_type{});
     // the words hold units of 2^(ref - 1075 - 43): twice kFixBits' unit
     Fix sum{(u64)a1 << 32 | a0, (u64)a3 << 32 | a2};
     sum = Fix{sum.lo << 1, sum.hi << 1 | sum.lo >> 63};
     fix_add2(sum, rest.lo, rest.hi);
     fix_block_atomic(st[j].sum, sum);
     n_tie = __reduce_add_sync(kAll, n_tie);
-    if (lane == 0 && n_tie) atomicAdd(&st[j].n_tie, (u64)n_tie);
-    if (beyond) atomicOr(&st[j].beyond, 1u);
+    if (lane == 0 && n_tie) atomicAdd(&st[j].n_tie[0], (u64)n_tie);
+    n_tie2 = __reduce_add_sync(kAll, n_tie2);
+    if (lane == 0 && n_tie2) atomicAdd(&st[j].n_tie[1], (u64)n_tie2);
+    if (again) atomicOr(&st[j].again, again);
 }
 
 // st NULL: the whole row is in shared memory.
@@ -383,27 +449,34 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     long long kmax_rank = 0;
     for (int q = 0; q < rk.n_p; ++q) kmax_rank = max(kmax_rank, rk.k[q]);
     bool use_list = false, have_sum = false;
-    u64 tie = 0, n_tie = 0;
+    Ties ties{};
     int64_t m = n;  // keys of the source
     Fix total{0, 0};
     int sum_ref = 0;
     if (st) {
         const ListState l = st[j];
-        have_sum = !l.beyond && l.ref;
+        have_sum = !l.again && l.ref;
         total = Fix{l.sum[0], l.sum[1]};
         sum_ref = l.ref;
         // every loss other than 0 that the list leaves out is below T
-        use_list = !l.beyond && l.n_list <= cap &&
-                   (l.threshold == 0 || (long long)(l.n_list + l.n_tie) >= kmax_rank);
+        use_list = !(l.again & kUnlisted) && l.n_list <= cap &&
+                   (l.threshold == 0 || (long long)(l.n_list + l.n_tie[0] + l.n_tie[1]) >= kmax_rank);
         if (use_list) {
             m = l.n_list;
-            tie = l.tie;
-            n_tie = l.n_tie;
+#pragma unroll
+            for (int i = 0; i < kTies; ++i) {
+                ties.key[i] = l.n_tie[i] ? l.tie[i] : 0ULL;
+                ties.n[i] = l.n_tie[i];
+            }
         }
     }
+    const u64 n_ties = ties.n[0] + ties.n[1];
     const u64* src = use_list ? lists + (size_t)j * cap : row;
     const bool held = m <= kSmall;
-    u64 mx = n_tie ? tie : 0ULL, mn = n_tie ? tie : ~0ULL;
+    u64 mx = max(ties.key[0], ties.key[1]), mn = ~0ULL;
+#pragma unroll
+    for (int i = 0; i < kTies; ++i)
+        if (ties.n[i]) mn = min(mn, ties.key[i]);
     constexpr int U = 8;  // loads in flight per thread
     for (int64_t i0 = threadIdx.x; i0 < m; i0 += (int64_t)U * kFinishThreads) {
         u64 v[U];
@@ -428,10 +501,17 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     const int e_ref = ref_exp(mx);
     auto get = [&](int64_t i) { return held ? s_keys[i] : src[i] & 0x7fffffffffffffffULL; };
     if (!have_sum) {
+        // from the list where it holds every loss but 0; where only some loss lay
+        // above the sum's range, from the row (its largest key is the list's)
         Fix f{0, 0};
-        for_each_key(get, m, [&](u64 v) { fix_add(f, v, e_ref); });
+        if (use_list && st[j].ref)
+            for_each_key([&](int64_t i) { return row[i] & 0x7fffffffffffffffULL; }, n, [&](u64 v) { fix_add(f, v, e_ref); });
+        else for_each_key(get, m, [&](u64 v) { fix_add(f, v, e_ref); });
         total = block_fix(f, s.red);
-        if (n_tie) fix_add_times(total, tie, e_ref, n_tie);
+        if (!(use_list && st[j].ref))
+#pragma unroll
+            for (int i = 0; i < kTies; ++i)
+                if (ties.n[i]) fix_add_times(total, ties.key[i], e_ref, ties.n[i]);
         sum_ref = e_ref;
     }
     if (threadIdx.x == 0) {
@@ -442,8 +522,8 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     for (int q = 0; q < rk.n_p; ++q) {
         const long long k = rk.k[q];
         u64 v = 0;  // fewer than k losses above 0
-        if ((long long)(m + n_tie) >= k)
-            v = mn == mx || (tie == mx && n_tie >= (u64)k) ? mx : kth_largest(get, m, tie, n_tie, mn, mx, k, s);
+        if ((long long)(m + n_ties) >= k)
+            v = mn == mx || (ties.key[0] == mx && ties.n[0] >= (u64)k) ? mx : kth_largest(get, m, ties, mn, mx, k, s);
         Fix f{0, 0};
         u64 cnt = 0;
         if (v < mx)
@@ -456,10 +536,12 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
         f = block_fix(f, s.red);
         cnt = block_sum(cnt, s.red);
         if (threadIdx.x == 0) {
-            if (n_tie && tie > v) {
-                fix_add_times(f, tie, e_ref, n_tie);
-                cnt += n_tie;
-            }
+#pragma unroll
+            for (int i = 0; i < kTies; ++i)
+                if (ties.n[i] && ties.key[i] > v) {
+                    fix_add_times(f, ties.key[i], e_ref, ties.n[i]);
+                    cnt += ties.n[i];
+                }
             const double x = __longlong_as_double((long long)v);
             const size_t w = (size_t)j * rk.n_p + q;
             if (pml) pml[w] = x;

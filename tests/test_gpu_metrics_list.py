@@ -70,3 +70,39 @@ def test_losses_below_the_normal_range(n):
         # the oracle's sums are exact here or round as above; a subnormal quotient rounds to its unit
         np.testing.assert_allclose(mean.cpu().numpy(), om, rtol=1e-12, atol=1e-323)
         np.testing.assert_allclose(tvar.cpu().numpy(), ot, rtol=1e-12, atol=1e-323)
+
+
+def _atom_rows(n, rng):
+    """Rows whose sample threshold falls on a value that repeats (a layer whose
+    events mostly pay their full limit), with other values around it."""
+    ln = rng.lognormal(15.0, 1.0, n)
+    pick = rng.random(n)
+    count = rng.poisson(0.2, n)
+    rows = [5e6 * count, 5e6 * rng.poisson(0.6, n), 5e6 * rng.poisson(3.0, n), 5e6 * np.minimum(count, 2),
+            5e6 * count + np.where(pick < 0.01, ln, 0.0),                      # losses between the multiples
+            np.where(pick < 0.3, 7e6, ln),                                    # one atom inside the losses
+            np.where(pick < 0.2, 7e6, np.where(pick < 0.4, 7e6 * (1 + 2.0 ** -40), 0.0)),  # two atoms in one bin
+            np.where(pick < 0.2, 7e6, np.where(pick < 0.4, 7e6 * (1 + 2.0 ** -18), 0.0)),
+            np.where(pick < 0.15, 7e6, np.where(pick < 0.16, ln, 0.0)),        # an atom and few others
+            np.where(pick < 0.5, 7e6, 0.0) + (np.arange(n) == 5) * 1e7,        # the largest is no tie
+            np.where(pick < 0.2, 1e-320, 0.0), np.where(pick < 0.2, 1e-320, ln)]  # subnormal atom
+    return np.stack(rows)
+
+
+@pytest.mark.parametrize("n", [12_288, 12_289, 26_625, 50_003, 300_001])
+def test_repeating_values_at_the_threshold(n):
+    rng = np.random.default_rng(n)
+    y = _atom_rows(n, rng)
+    dev = torch.from_numpy(y).cuda()
+    for probs in ([0.99], [0.955], [0.99, 0.996, 0.999], [0.951, 0.98, 0.9999]):
+        L, n_p = y.shape[0], len(probs)
+        om, op, ot = oracle.metrics(y, probs)
+        for fn in (art.art_metrics, art.art_metrics_noalloc):
+            mean = torch.full((L,), -1.0, dtype=torch.float64, device="cuda")
+            pml = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+            tvar = torch.full((L, n_p), -1.0, dtype=torch.float64, device="cuda")
+            fn(dev, n, L, probs, mean, pml, tvar)
+            np.testing.assert_array_equal(pml.cpu().numpy(), op)
+            # one or two roundings against the oracle's sequential FP64 sums; subnormal units
+            np.testing.assert_allclose(mean.cpu().numpy(), om, rtol=1e-12, atol=1e-323)
+            np.testing.assert_allclose(tvar.cpu().numpy(), ot, rtol=1e-12, atol=1e-323)
