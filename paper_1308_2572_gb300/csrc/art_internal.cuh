@@ -468,8 +468,9 @@ cudaError_t metrics_run_k(const double* ylt, int64_t n, int32_t n_layers, const 
                           void* scratch = nullptr, size_t scratch_bytes = 0);
 size_t metrics_scratch_bytes(int64_t n, int32_t n_layers, int32_t n_p);
 // The one-read form of the metrics (metrics_list.cu): whether it takes ranks
-// up to k_max of n_layers layers of n trials, its scratch, and the call.
-bool metrics_listable(int64_t n, int32_t n_layers, int64_t k_max);
+// up to k_max of n_layers layers of n trials at n_p probabilities, its scratch,
+// and the call.
+bool metrics_listable(int64_t n, int32_t n_layers, int64_t k_max, int32_t n_p);
 size_t metrics_list_bytes(int64_t n, int32_t n_layers);
 cudaError_t metrics_list_run(const double* ylt, int64_t n, int32_t n_layers, const int64_t* k, int32_t n_p, double* mean,
                              double* pml, double* tvar, double* sum_out, cudaStream_t s, void* scratch);

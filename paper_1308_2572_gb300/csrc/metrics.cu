@@ -902,7 +902,7 @@ cudaError_t metrics_run_k(const double* ylt, int64_t n, int32_t n_layers, const 
     char* w = static_cast<char*>(scratch);
     int64_t k_max = 1;
     for (int q = 0; q < n_p; ++q) k_max = std::max(k_max, k[q]);
-    if (metrics_listable(n, n_layers, k_max)) {
+    if (metrics_listable(n, n_layers, k_max, n_p)) {
         const size_t bytes = metrics_list_bytes(n, n_layers);
         const bool own = !w || scratch_bytes < bytes;
         cudaError_t err = own ? scratch_alloc((void**)&w, bytes, s) : cudaSuccess;
@@ -1054,7 +1054,7 @@ extern "C" art_status art_metrics_noalloc(const double* ylt_dev, int64_t n_trial
         k[q] = tail_count(probs_host[q], n_trials);
         k_max = std::max(k_max, k[q]);
     }
-    if (metrics_listable(n_trials, n_layers, k_max) &&
+    if (metrics_listable(n_trials, n_layers, k_max, n_p) &&
         metrics_list_bytes(n_trials, n_layers) <= (size_t)ART_METRICS_NOALLOC_SCRATCH_BYTES) {
         err = metrics_list_run(ylt_dev, n_trials, n_layers, k, n_p, mean_dev, pml_dev, tvar_dev, nullptr, stream, w);
         if (err != cudaSuccess) {

@@ -21,7 +21,7 @@
 //      overflowed, or some loss is subnormal beside T > 0, the CTA takes the row
 //      instead (for the sum alone where a loss lay far above the sample's
 //      largest): slower, the same results.
-// A YLT of at most kSmall trials skips 1 and 2: its rows fit shared memory.
+// A short YLT (metrics_small) skips 1 and 2: its rows fit shared memory.
 //
 // What bounds it: HBM (8 bytes per loss, once); the general path's two full
 // reads and six list passes took 1.04 ms on 128 layers x 1,000,000 trials at
@@ -551,16 +551,42 @@ __global__ void __launch_bounds__(kFinishThreads, 1) list_finish_kernel(const do
     }
 }
 
-unsigned int list_cap(int64_t n) { return (unsigned int)std::max<int64_t>(n / 8, 8192); }
+unsigned int list_cap(int64_t n) { return (unsigned int)((n + 7) / 8); }
+
+// Rank in the sample of the list's threshold: the sample's share of the k
+// largest, six standard deviations and a few more.
+int sample_rank(int64_t n, int64_t k_max) {
+    const double share = (double)k_max * kSample / (double)n;
+    return (int)std::min<double>(kSample, std::ceil(share + 6.0 * std::sqrt(share) + 8.0));
+}
 
 }  // namespace
 
-bool metrics_small(int64_t n) { return n <= kSmall; }
+// Rows that go to the finish whole. It has room for kSmall, but from here on
+// the sample and the pass are faster (12,288 trials, 3 probabilities: 42 us
+// whole and 34 sampled for one layer, 541 and 379 for 2,000; 8,192 trials: 32
+// and 34, 397 and 357; with three atoms in the row whole rows pay more, as
+// their keys meet in few bins: 26,624 trials x 2,000 layers 1.50 ms against 0.69).
+bool metrics_small(int64_t n) { return n <= 12288; }
 
-// The list path takes ranks up to n / 20 (its lists then hold well under the
-// n / 8 losses they have room for).
-bool metrics_listable(int64_t n, int32_t n_layers, int64_t k_max) {
-    return metrics_small(n) || (k_max <= n / 20 && n_layers <= 65535);
+// Whether the list path takes the call. Its lists have room for the ranks up
+// to n / 20 (they then hold well under n / 8), and its finish is one CTA per
+// layer, so few layers with long lists are left to the general path, whose
+// every step is spread over the chip. Both times in us, fitted to 1 to 128
+// layers of 200,000 to 100,000,000 trials at 1 and 3 probabilities (within
+// about a fifth): the pass grows with the YLT, the finish with each list,
+// twice as fast where shared memory holds it. One layer of 1,000,000 trials at
+// 0.95: 133 us by list, 100 in general; at 0.99: 50 and 95; 128 layers at 0.95:
+// 415 and 1,005; one layer of 100,000,000 at 0.99: 2,964 and 702.
+bool metrics_listable(int64_t n, int32_t n_layers, int64_t k_max, int32_t n_p) {
+    if (metrics_small(n)) return true;
+    if (k_max > n / 20 || n_layers > 65535) return false;
+    const double m = (double)n * sample_rank(n, k_max) / kSample, all = 1e-6 * (double)n * n_layers;
+    const double per_key = 1e-3 * (0.3 + (m <= kSmall ? 0.5 : 1.1) * n_p);
+    const double waves = (n_layers + 147) / 148;
+    const double list = 28.0 + std::max(std::min(9.0 * all, 90.0 + 1.2 * all), 3.5e-6 * (double)n) + waves * m * per_key;
+    const double general = 65.0 + 28.0 * n_p + (5.2 + 1.4 * n_p) * all;
+    return list <= general;
 }
 
 size_t metrics_list_bytes(int64_t n, int32_t n_layers) {
@@ -591,10 +617,7 @@ cudaError_t metrics_list_run(const double* ylt, int64_t n, int32_t n_layers, con
         st = reinterpret_cast<ListState*>(scratch);
         lists = reinterpret_cast<u64*>(static_cast<char*>(scratch) +
                                        ((sizeof(ListState) * (size_t)n_layers + 255) & ~(size_t)255));
-        // the sample's share of the k largest, six standard deviations and a few more
-        const double share = (double)k_max * kSample / (double)n;
-        const int rank = (int)std::min<double>(kSample, std::ceil(share + 6.0 * std::sqrt(share) + 8.0));
-        list_sample_kernel<<<(unsigned)n_layers, kFinishThreads, 0, s>>>(ylt, n, rank, st);
+        list_sample_kernel<<<(unsigned)n_layers, kFinishThreads, 0, s>>>(ylt, n, sample_rank(n, k_max), st);
         if ((e = cudaGetLastError())) return e;
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
