@@ -653,27 +653,35 @@ void free_portfolio(art_portfolio* p) {
     scratch_user(-1);
 }
 
-// The variant of a call over n_trials trials of k events (k = 0: a CSR, whose
-// length is on the device: 500 events per trial are assumed). ids NULL: they
-// will be staged on the device.
-int resolve_variant(const art_portfolio* p, int64_t n_trials, const int32_t* ids, int32_t k, cudaStream_t s) {
-    if (p->variant != ART_VARIANT_AUTO) return p->variant;
-    // tables of whole numbers: a pass takes about 3.2 ps per event and run of
-    // 8 layers where the sparse variant takes 12 (64 layers over 256 ELTs), after
-    // a build of about 45 ps per catalogue event and run: it pays from five
-    // events per catalogue event on
-    const bool whole = !p->ogroups.empty() && std::all_of(p->ogroups.begin(), p->ogroups.end(),
-                                                          [](const OccGroupArgs& g) { return g.sum_fits > 0; });
-    if (whole && (double)n_trials * (k > 0 ? k : 500) >= 5.0 * p->catalogue && ids_on_device(ids) &&
-        !captured_by_caller(p, s))
-        return ART_VARIANT_SKIP;
-    // few groups: the YET is streamed once per group, each event row read
-    // only when its bit is set; many groups: one pass over a pool table
-    if (!p->groups.empty() && p->groups.size() <= 2) return ART_VARIANT_SKIP;
-    if (p->sp_ptr && p->n_tiles > 0) return ART_VARIANT_SPARSE;
-    if (p->pool && p->n_tiles > 0) return ART_VARIANT_BATCHED;
-    if (!p->groups.empty()) return ART_VARIANT_SKIP;
-    return ART_VARIANT_PLAIN;
+// Times in us of a forward over n trials of E events in all, for the choice
+// between AUTO's forms (fitted to 1 to 512 layers over pools of 64 and 256 ELTs,
+// 0.01% to 5% of events with a loss per ELT, trials of 5 to 1,000 events: within
+// about a third, where the forms differ by up to 20 times).
+//
+// The skip passes over whole numbers, run by run of 8 layers: the table build
+// (per catalogue event, and per loss of its entries), and per trial its chunks
+// of 256 ids, however few of them it fills; events with a loss cost a row.
+double whole_skip_us(const art_portfolio* p, double n, double E) {
+    const double runs = (double)p->ogroups.size();
+    const double losses = p->sp_ptr ? (double)p->sp_nnz / p->catalogue : 1.0;
+    const double pairs = losses * p->lids.size() / p->n_elt;  // (loss, layer) per event
+    double build = 1e-6 * p->catalogue * runs * (8.0 + 3.3 * losses);
+    if (!(p->d_slotmask && p->sp_ptr)) build = (double)p->layer_bytes / 3.5e6;  // reads every layer's rows
+    const double chunks = std::max(n, E / 256.0 + 0.5 * n);
+    return build + runs * (8.0 + 1e-3 * (0.25 * n + 0.33 * chunks) + 1.1e-6 * E * std::min(1.0, pairs / runs));
+}
+
+// The variants that AUTO takes otherwise.
+double other_us(const art_portfolio* p, int variant, double n, double E) {
+    if (variant == ART_VARIANT_SPARSE) {  // walks each event's losses; a warp takes four trials
+        const double pairs = (double)p->sp_nnz / p->catalogue * p->lids.size() / p->n_elt;
+        const double ps = 10.5 + 0.02 * p->n_layers + 10.0 * std::pow(pairs, 0.85);
+        return 15.0 + (1.2e-3 * n + 1e-6 * ps * E) * std::max(1.0, 9728.0 / std::max(1.0, n));
+    }
+    if (variant == ART_VARIANT_BATCHED) return 15.0 + 1e-3 * n + 0.8e-6 * p->pool_np * E;
+    double ps = 0.0;  // a row of each layer's table per event
+    for (int32_t np : p->layer_np) ps += 1.1 * np;
+    return p->n_layers * (5.0 + 0.3e-3 * n) + 1e-6 * ps * E;
 }
 
 bool variant_available(const art_portfolio* p, int v) {
@@ -685,6 +693,41 @@ bool variant_available(const art_portfolio* p, int v) {
         return !p->ogroups64.empty() ||
                (p->pool64 != nullptr && p->n_tiles > 0 && batched_smem(p, true) <= 200 * 1024);
     return false;
+}
+
+// The variant of a call; other >= 0: a CSR whose event count decides, on the
+// device, between the variant (from `split` events on) and that one.
+struct Route {
+    int variant;
+    int other = -1;
+    int64_t split = 0;
+};
+
+// events: how many the YET holds, where the host knows (a CSR's length is on
+// the device otherwise: -1). y.ids NULL: they will be staged on the device.
+Route resolve_variant(const art_portfolio* p, const YetArgs& y, int64_t events, cudaStream_t s) {
+    if (p->variant != ART_VARIANT_AUTO) return {p->variant};
+    // few groups: the YET is streamed once per group, each event row read
+    // only when its bit is set
+    if (!p->groups.empty() && p->groups.size() <= 2) return {ART_VARIANT_SKIP};
+    // many groups: one pass over the CSR or a pool table
+    int other = ART_VARIANT_PLAIN;
+    if (p->sp_ptr && p->n_tiles > 0) other = ART_VARIANT_SPARSE;
+    else if (p->pool && p->n_tiles > 0) other = ART_VARIANT_BATCHED;
+    else if (!p->groups.empty()) return {ART_VARIANT_SKIP};
+    // or, over tables of whole numbers, one short pass per run of 8 layers
+    const bool whole = !p->ogroups.empty() && std::all_of(p->ogroups.begin(), p->ogroups.end(),
+                                                          [](const OccGroupArgs& g) { return g.sum_fits > 0; });
+    if (!whole || !ids_on_device(y) || captured_by_caller(p, s)) return {other};
+    if (!variant_available(p, other)) return {ART_VARIANT_SKIP};
+    const double n = (double)y.n_trials;
+    int64_t split = 0;
+    switch (by_events(y, events, [&](double E) { return other_us(p, other, n, E); },
+                      [&](double E) { return whole_skip_us(p, n, E); }, &split)) {
+        case ByEvents::few: return {other};
+        case ByEvents::many: return {ART_VARIANT_SKIP};
+        default: return {ART_VARIANT_SKIP, other, split};
+    }
 }
 
 art_status validate_yet(int64_t n_trials, const int32_t* ids, const int64_t* off, int32_t k) {
@@ -705,6 +748,17 @@ cudaError_t run_forward(art_portfolio* p, int variant, const YetArgs& y, double*
     if (variant == ART_VARIANT_SPARSE) return launch_sparse(p, y, ylt, branch, s);
     if (variant == ART_VARIANT_FP64 && !p->ogroups64.empty()) return launch_skip64(p, y, ylt, branch, s, build_tables);
     return launch_batched(p, y, ylt, branch, variant == ART_VARIANT_FP64, s);
+}
+
+// Both forms of a route that the device decides, each behind its gate.
+cudaError_t run_route(art_portfolio* p, const Route& r, YetArgs y, double* ylt, uint8_t* branch, cudaStream_t s) {
+    if (r.other >= 0) {
+        y.gate = EventGate{y.off, y.n_trials, std::numeric_limits<int64_t>::min(), r.split};
+        const cudaError_t e = run_forward(p, r.other, y, ylt, branch, s);
+        if (e) return e;
+        y.gate = EventGate{y.off, y.n_trials, r.split, std::numeric_limits<int64_t>::max()};
+    }
+    return run_forward(p, r.variant, y, ylt, branch, s);
 }
 
 }  // namespace
@@ -940,9 +994,10 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
     if (st) return st;
     if (n_trials == 0) return ART_OK;
     if (!ylt_dev) return ART_EINVAL;
-    const int variant = resolve_variant(p, n_trials, event_ids_dev, trial_off_dev ? 0 : events_per_trial, stream);
-    if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     YetArgs y{event_ids_dev, trial_off_dev, n_trials, trial_off_dev ? 0 : events_per_trial, p->catalogue};
+    const Route route = resolve_variant(p, y, -1, stream);
+    const int variant = route.variant;
+    if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     cudaError_t e;
     const bool use_graph = (p->flags & ART_FLAG_GRAPH) != 0;
     if (use_graph) {
@@ -960,7 +1015,7 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
             e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
             if (!e) {
                 p->own_capture = true;
-                const cudaError_t le = run_forward(p, variant, y, ylt_dev, branch_dev, cap);
+                const cudaError_t le = run_route(p, route, y, ylt_dev, branch_dev, cap);
                 p->own_capture = false;
                 e = cudaStreamEndCapture(cap, &g);
                 if (!e) e = le;
@@ -984,7 +1039,7 @@ art_status art_run_ylt(art_portfolio* p, int64_t n_trials, const int32_t* event_
                         variant != ART_VARIANT_SKIP;
     if (window) set_window(stream, variant == ART_VARIANT_FP64 ? (const void*)p->pool64 : (const void*)p->pool,
                            variant == ART_VARIANT_FP64 ? p->pool64_bytes : p->pool_bytes);
-    e = run_forward(p, variant, y, ylt_dev, branch_dev, stream);
+    e = run_route(p, route, y, ylt_dev, branch_dev, stream);
     if (window) set_window(stream, nullptr, 0);
     return e ? fail(e) : ART_OK;
 }
@@ -1047,7 +1102,8 @@ art_status host_run(art_portfolio* p, int64_t n_trials, const int32_t* event_ids
         for (int64_t t = 0; t < n_trials; ++t)
             if (trial_off_host[t + 1] < trial_off_host[t]) return ART_EINVAL;
     }
-    const int variant = resolve_variant(p, n_trials, nullptr, trial_off_host ? 0 : events_per_trial, stream);
+    const YetArgs whole_yet{nullptr, trial_off_host, n_trials, trial_off_host ? 0 : events_per_trial, p->catalogue};
+    const int variant = resolve_variant(p, whole_yet, trial_off_host ? trial_off_host[n_trials] : -1, stream).variant;
     if (!variant_available(p, variant)) return ART_EUNSUPPORTED;
     if (!(p->flags & ART_FLAG_HOST_STAGED) && one_pass_over_ids(p, variant)) {
         const int32_t* d_ids = device_alias(event_ids_host);

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -61,6 +62,19 @@ struct LayerArgs {
     int32_t layer;        // layer index (row of the YLT)
 };
 
+// A CSR call whose better form hangs on the number of its events, which only
+// the device knows: the host launches both forms, and the kernels of the one
+// whose range does not hold that number leave at once. Open by default.
+struct EventGate {
+    const int64_t* off = nullptr;
+    int64_t n_trials = 0, lo = 0, hi = 0;  // runs when lo <= events < hi
+    __device__ __forceinline__ bool closed() const {
+        if (!off) return false;
+        const int64_t events = off[n_trials] - off[0];
+        return events < lo || events >= hi;
+    }
+};
+
 struct YetArgs {
     const int32_t* ids;
     const int64_t* off;   // NULL: dense
@@ -70,6 +84,7 @@ struct YetArgs {
     bool by_id = false;   // ids to be read one by one (not in device memory: no bulk copies)
     bool staged = false;  // ids of a chunk that the library copied to the device itself: `ids` is then
                           // shifted back by the chunk's first index and may point outside any allocation
+    EventGate gate;
 };
 
 __device__ __forceinline__ void trial_range(const YetArgs& y, int64_t t, int64_t& b, int64_t& e, bool& bad) {
@@ -448,7 +463,7 @@ cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8
 cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap, cudaStream_t s);
 // Write every occurrence group's X and bitmap (one launch); whole: as whole
 // numbers in the groups whose losses allow it.
-cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s);
+cudaError_t build_occurrence(art_portfolio* p, bool whole, const EventGate& gate, cudaStream_t s);
 cudaError_t launch_batched(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, bool fp64,
                            cudaStream_t s);
 cudaError_t launch_adjoint(art_portfolio* p, const YetArgs& y, const uint8_t* branch, const double* g,
@@ -511,6 +526,34 @@ cudaError_t scratch_alloc(void** out, size_t bytes, cudaStream_t s);
 void scratch_user(int delta);
 // Id of the current device's context; 0 if the driver cannot tell.
 unsigned long long current_context_id();
+// Bytes from a device address to the end of its allocation; the largest
+// int64_t if the driver cannot tell.
+int64_t bytes_behind(const void* p);
+// Which of two forms of a call over n trials is the faster one, where the first
+// is for few events (few(E) and many(E): their times over E events). A CSR's
+// number of events is on the device unless the host has it (events >= 0):
+// then `split` is the number from which on the second form is taken there.
+enum class ByEvents { few, many, device };
+template <class Few, class Many>
+ByEvents by_events(const YetArgs& y, int64_t events, Few few, Many many, int64_t* split) {
+    if (!y.off) events = y.n_trials * (int64_t)y.k;
+    if (events >= 0) return few((double)events) < many((double)events) ? ByEvents::few : ByEvents::many;
+    const int64_t most = bytes_behind(y.ids) / (int64_t)sizeof(int32_t);
+    int64_t lo = std::min<int64_t>(most, (int64_t)1 << 40), hi;
+    if (few((double)lo) < many((double)lo)) return ByEvents::few;
+    do {  // down by halves to the last number that is still better off with the second form
+        hi = lo;
+        lo = hi / 2;
+    } while (hi > 0 && few((double)lo) >= many((double)lo));
+    if (hi == 0) return ByEvents::many;
+    while (hi - lo > 1 + lo / 64) {
+        const int64_t mid = lo + (hi - lo) / 2;
+        if (few((double)mid) < many((double)mid)) lo = mid;
+        else hi = mid;
+    }
+    *split = hi;
+    return ByEvents::device;
+}
 
 // Set (bytes > 0) or clear (bytes == 0) a persisting L2 access-policy window
 // over a hot table on a stream.

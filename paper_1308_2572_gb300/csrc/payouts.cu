@@ -40,6 +40,7 @@ template <int NP>
 __global__ void __launch_bounds__(256) payouts_kernel(const LayerArgs la, const YetArgs y,
                                                       double* __restrict__ payouts, int32_t* __restrict__ exhaust,
                                                       double* __restrict__ ylt, int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -124,7 +125,8 @@ struct PayArgs {
 template <int NP>
 __global__ void __launch_bounds__(256) payouts_table_kernel(const LayerArgs la, int32_t catalogue, float scale,
                                                             int32_t words, uint32_t* __restrict__ x,
-                                                            uint32_t* __restrict__ bits) {
+                                                            uint32_t* __restrict__ bits, const EventGate gate) {
+    if (gate.closed()) return;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t u = 0;
     if (i < catalogue) {
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(kPayThreads, 1) payouts_fixed_kernel(const Pay
                                                                       int32_t* __restrict__ exhaust,
                                                                       double* __restrict__ ylt,
                                                                       int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr int E = kPayIds;
     extern __shared__ __align__(128) uint32_t s_dyn[];
     uint32_t* s_ids = s_dyn + 64;  // [kPayWarps][32 * E], after the warps' barriers
@@ -308,20 +311,26 @@ unsigned long long first_units(double unit, F f) {
     return lo;
 }
 
-// The whole-number form of the call. The table costs one read of the layer's
-// rows, an occurrence evaluated by itself about a row's gather (24 us per
-// million against 3): it is built from C / 2 events on (a CSR's trials are
-// taken as 500 events each, its length being on the device). done: false where
-// the call keeps the other form.
-cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double lims, const YetArgs& y, double* payouts,
-                         int32_t* exhaust, double* ylt, cudaStream_t s, bool* done) {
+// The whole-number form of the call, where it is the faster one. Its table
+// costs one read of the layer's rows; its pass then takes 0.55 ns per trial and
+// 256 ids (and 1.2 ps per event), the other form 0.79 ns per trial and 32 ids
+// (2,000,000 events of 16 ELTs: 36 us for the table; 2,000 trials of 300 events
+// 26 us without it and 37 with it, 200,000 trials of 50 316 and 175). A CSR whose
+// length alone decides is launched in both forms, one of which leaves on the
+// device: `rest` then holds the other's gate. done: the other is not needed.
+cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double lims, YetArgs y, double* payouts,
+                         int32_t* exhaust, double* ylt, cudaStream_t s, bool* done, YetArgs* rest) {
     *done = false;
     int e2;
     double top;
-    const double events = (double)y.n_trials * (y.off ? 500.0 : (double)y.k);
-    if (events < 0.5 * p->catalogue || !ids_on_device(y) ||
-        !whole_losses(la.occ_ret, la.occ_lim, lims, &e2, &top))
-        return cudaSuccess;
+    if (!ids_on_device(y) || !whole_losses(la.occ_ret, la.occ_lim, lims, &e2, &top)) return cudaSuccess;
+    const double n = (double)y.n_trials, table_us = (double)p->catalogue * np * 4.0 / 3.5e6;
+    auto steps = [&](double E, double ids) { return std::max(n, E / ids + 0.5 * n); };
+    int64_t split = 0;
+    const ByEvents form = by_events(
+        y, -1, [&](double E) { return 5.0 + 0.79e-3 * steps(E, 32.0); },
+        [&](double E) { return 5.0 + table_us + 1e-3 * (0.1 * n + 0.45 * steps(E, 256.0)) + 1.2e-6 * E; }, &split);
+    if (form == ByEvents::few) return cudaSuccess;
     PayArgs a;
     a.unit = std::ldexp(1.0, e2);
     a.unit_f = (float)a.unit;
@@ -354,6 +363,10 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
         cudaGetLastError();  // no room for the table: the other form needs none
         return cudaSuccess;
     }
+    if (form == ByEvents::device) {
+        rest->gate = EventGate{y.off, y.n_trials, std::numeric_limits<int64_t>::min(), split};
+        y.gate = EventGate{y.off, y.n_trials, split, std::numeric_limits<int64_t>::max()};
+    }
     uint32_t* x = reinterpret_cast<uint32_t*>(w);
     uint32_t* bits = reinterpret_cast<uint32_t*>(w + xb);
     a.x = x;
@@ -361,11 +374,11 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
     const float scale = (float)std::ldexp(1.0, -e2);
     const unsigned blocks = (unsigned)((padded * 32 + 255) / 256);
     switch (np) {
-        case 4: payouts_table_kernel<4><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
-        case 8: payouts_table_kernel<8><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
-        case 16: payouts_table_kernel<16><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
-        case 24: payouts_table_kernel<24><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
-        default: payouts_table_kernel<32><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits); break;
+        case 4: payouts_table_kernel<4><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits, y.gate); break;
+        case 8: payouts_table_kernel<8><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits, y.gate); break;
+        case 16: payouts_table_kernel<16><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits, y.gate); break;
+        case 24: payouts_table_kernel<24><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits, y.gate); break;
+        default: payouts_table_kernel<32><<<blocks, 256, 0, s>>>(la, C, scale, (int32_t)padded, x, bits, y.gate); break;
     }
     if (!(e = cudaGetLastError())) {
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(p->num_sms, y.n_trials));
@@ -373,15 +386,16 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
         e = cudaGetLastError();
     }
     const cudaError_t e3 = cudaFreeAsync(w, s);
-    *done = true;
+    *done = form == ByEvents::many;
     return e ? e : e3;
 }
 
 }  // namespace
 
-cudaError_t launch_payouts(art_portfolio* p, int32_t j, const YetArgs& y, double* payouts, int32_t* exhaust,
+cudaError_t launch_payouts(art_portfolio* p, int32_t j, const YetArgs& yet, double* payouts, int32_t* exhaust,
                            double* ylt, cudaStream_t s) {
-    if (y.n_trials == 0) return cudaSuccess;
+    if (yet.n_trials == 0) return cudaSuccess;
+    YetArgs y = yet;
     LayerArgs la;
     la.table = p->layer_tab[j];
     const int32_t b = p->loff[j], n = p->loff[j + 1] - b;
@@ -400,7 +414,7 @@ cudaError_t launch_payouts(art_portfolio* p, int32_t j, const YetArgs& y, double
     double lims = 0.0;
     for (int k = 0; k < n; ++k) lims += la.lim[k];
     bool done = false;
-    const cudaError_t err = launch_whole(p, la, p->layer_np[j], lims, y, payouts, exhaust, ylt, s, &done);
+    const cudaError_t err = launch_whole(p, la, p->layer_np[j], lims, yet, payouts, exhaust, ylt, s, &done, &y);
     if (err || done) return err;
     switch (p->layer_np[j]) {
         case 4: return launch<4>(la, y, payouts, exhaust, ylt, p->d_flags, s);

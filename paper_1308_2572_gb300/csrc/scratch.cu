@@ -41,6 +41,24 @@ unsigned long long current_context_id() {
     return id;
 }
 
+int64_t bytes_behind(const void* p) {
+    typedef int (*GetRange)(unsigned long long*, size_t*, unsigned long long);
+    static GetRange get_range = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get_range = reinterpret_cast<GetRange>(f);
+    });
+    unsigned long long base = 0;
+    size_t bytes = 0;
+    const unsigned long long a = reinterpret_cast<uintptr_t>(p);
+    if (!get_range || get_range(&base, &bytes, a) != 0 || a < base || a > base + bytes) return INT64_MAX;
+    return (int64_t)(base + bytes - a);
+}
+
 namespace {
 
 constexpr uint64_t kScratchKeep = 256ULL << 20;  // bytes a device's pool keeps between calls

@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(256) ylt_batched_kernel(const BatchedArgs a, c
                                                           double* __restrict__ ylt,
                                                           uint8_t* __restrict__ branch,
                                                           int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr int NPOOL = 32 * EPL;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];

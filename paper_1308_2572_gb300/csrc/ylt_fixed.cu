@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_narrow_ker
                                                                     double* __restrict__ ylt,
                                                                     uint8_t* __restrict__ branch,
                                                                     int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr int E = kFxIds;
     constexpr int NWARP = kFxWarpsFor<LP, VEC>;
     extern __shared__ __align__(512) uint32_t s_dyn[];
@@ -254,6 +255,7 @@ __global__ void __launch_bounds__(32 * kFxWarpsFor<LP, VEC>, 1) fixed_wide_kerne
                                                                   double* __restrict__ ylt,
                                                                   uint8_t* __restrict__ branch,
                                                                   int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr int E = kFxIds;
     constexpr int NWARP = kFxWarpsFor<LP, VEC>;
     extern __shared__ __align__(512) uint32_t s_dyn[];

@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(256) ylt_plain_kernel(const LayerArgs la, cons
                                                         uint8_t* __restrict__ branch,
                                                         int* __restrict__ flags) {
     static_assert(NP % 4 == 0 && NP <= kMaxLayerElts, "row width");
+    if (y.gate.closed()) return;
     const int lane = threadIdx.x & 31;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= y.n_trials) return;  // whole warp leaves together

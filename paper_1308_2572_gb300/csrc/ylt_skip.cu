@@ -444,7 +444,8 @@ __device__ __forceinline__ float table_entry(float o, float scale) {
 template <int LP>
 __global__ void __launch_bounds__(256) build_occ_kernel(const LayerBuildArgs* __restrict__ lbuild,
                                                         const OccBuildGroup* __restrict__ groups, int32_t catalogue,
-                                                        int32_t words, const bool whole) {
+                                                        int32_t words, const bool whole, const EventGate gate) {
+    if (gate.closed()) return;
     __shared__ LayerBuildArgs s_lb[LP];
     const OccBuildGroup& grp = groups[blockIdx.y];
     const int nl = grp.n_layers;
@@ -515,7 +516,8 @@ __global__ void __launch_bounds__(256) build_occ_csr_kernel(const uint32_t* __re
                                                             const float* __restrict__ occ_terms,
                                                             const LayerBuildArgs* __restrict__ lbuild,
                                                             const OccBuildGroup* __restrict__ groups, int32_t catalogue,
-                                                            int32_t words, const bool whole) {
+                                                            int32_t words, const bool whole, const EventGate gate) {
+    if (gate.closed()) return;
     const OccBuildGroup& grp = groups[blockIdx.y];
     const uint8_t* sm = slotmask + (size_t)blockIdx.y * np;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -584,7 +586,8 @@ __global__ void __launch_bounds__(256) build_occ_csr1_kernel(const uint32_t* __r
                                                              const float* __restrict__ occ_terms,
                                                              const LayerBuildArgs* __restrict__ lbuild,
                                                              const OccBuildGroup* __restrict__ groups, int32_t catalogue,
-                                                             int32_t words, const bool whole) {
+                                                             int32_t words, const bool whole, const EventGate gate) {
+    if (gate.closed()) return;
     const OccBuildGroup& grp = groups[0];
     const int lane = threadIdx.x & 31;
     const int64_t i0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
@@ -654,7 +657,8 @@ __global__ void __launch_bounds__(kTileEvents) build_occ_tile_kernel(
     const uint32_t* __restrict__ ptr, const SparseEntry* __restrict__ entries, const float* __restrict__ terms,
     int32_t np, const uint8_t* __restrict__ slotmask, const float* __restrict__ occ_terms,
     const LayerBuildArgs* __restrict__ lbuild, const OccBuildGroup* __restrict__ groups, int32_t n_groups,
-    int32_t catalogue, int32_t words, const bool whole) {
+    int32_t catalogue, int32_t words, const bool whole, const EventGate gate) {
+    if (gate.closed()) return;
     __shared__ float s_x[8 * kTileGroups][kTileEvents];
     __shared__ uint32_t s_mask[kMaxPoolElts];  // the tile's slots of each ELT
     __shared__ float s_f[kTileEntries];
@@ -764,7 +768,7 @@ cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np
     return cudaGetLastError();
 }
 
-cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s) {
+cudaError_t build_occurrence(art_portfolio* p, bool whole, const EventGate& gate, cudaStream_t s) {
     const int32_t words = (int32_t)(((int64_t)p->catalogue + 31) / 32);
     const dim3 grid((unsigned)(((int64_t)words * 32 + 255) / 256), (unsigned)p->ogroups.size());
     // from the CSR of the non-zero losses where the portfolio holds it (see
@@ -776,27 +780,27 @@ cudaError_t build_occurrence(art_portfolio* p, bool whole, cudaStream_t s) {
                              (unsigned)((p->ogroups.size() + kTileGroups - 1) / kTileGroups));
             build_occ_tile_kernel<<<tiles, kTileEvents, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask,
                                                                p->d_occ, p->d_lbuild, p->d_ogroups,
-                                                               (int32_t)p->ogroups.size(), p->catalogue, words, whole);
+                                                               (int32_t)p->ogroups.size(), p->catalogue, words, whole, gate);
             return cudaGetLastError();
         }
         if (p->og_lp == 1 && p->catalogue >= (1 << 19)) {
-            build_occ_csr1_kernel<<<(grid.x + 3) / 4, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole);
+            build_occ_csr1_kernel<<<(grid.x + 3) / 4, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate);
             return cudaGetLastError();
         }
         switch (p->og_lp) {
-            case 1: build_occ_csr_kernel<1><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-            case 2: build_occ_csr_kernel<2><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-            case 4: build_occ_csr_kernel<4><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-            case 8: build_occ_csr_kernel<8><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+            case 1: build_occ_csr_kernel<1><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+            case 2: build_occ_csr_kernel<2><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+            case 4: build_occ_csr_kernel<4><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+            case 8: build_occ_csr_kernel<8><<<grid, 256, 0, s>>>(p->sp_ptr, en, p->d_elt_terms, p->pool_np, p->d_slotmask, p->d_occ, p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
             default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
     }
     switch (p->og_lp) {
-        case 1: build_occ_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-        case 2: build_occ_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-        case 4: build_occ_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
-        case 8: build_occ_kernel<8><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole); break;
+        case 1: build_occ_kernel<1><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+        case 2: build_occ_kernel<2><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+        case 4: build_occ_kernel<4><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
+        case 8: build_occ_kernel<8><<<grid, 256, 0, s>>>(p->d_lbuild, p->d_ogroups, p->catalogue, words, whole, gate); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -831,7 +835,7 @@ cudaError_t launch_skip(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t
     // memory keep the FP32 tables and the loads of the pass below
     const bool whole = ids_on_device(y) && !captured_by_caller(p, s);
     // steps 2-3 once per catalogue event, with the terms as they are now
-    cudaError_t err = build ? build_occurrence(p, whole, s) : cudaSuccess;
+    cudaError_t err = build ? build_occurrence(p, whole, y.gate, s) : cudaSuccess;
     if (err != cudaSuccess || y.n_trials == 0) return err;
     // ART_FLAG_L2_PERSIST: a persisting window over the table each group
     // pass gathers from, so that the id stream does not evict it

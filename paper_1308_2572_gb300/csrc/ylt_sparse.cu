@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(kSparseThreads) ylt_sparse_scatter_kernel(cons
                                                                    double* __restrict__ ylt,
                                                                    uint8_t* __restrict__ branch,
                                                                    int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int LT = 32 * SLOTS;  // layers per tile
     constexpr int XS = LT + 1;      // row stride of the accumulator block (bank spread)
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kSparseThreads) ylt_sparse_bcast_kernel(const 
                                                                    double* __restrict__ ylt,
                                                                    uint8_t* __restrict__ branch,
                                                                    int* __restrict__ flags) {
+    if (y.gate.closed()) return;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     float4* s_terms = reinterpret_cast<float4*>(smem);                       // [pool_np] m, D, Lim
