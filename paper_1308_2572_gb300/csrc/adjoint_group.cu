@@ -22,7 +22,8 @@
 // their table row. Records come from the CSR of the non-zero losses where the
 // portfolio holds it (an event with more than four of the group's losses from
 // its table row, in the group's order), else from the table rows; the same
-// values either way.
+// values either way. Groups whose events mostly have more columns, and calls
+// with no room for the records, go to adjoint_rows.cu.
 //
 // The trial pass is shaped like the forward's (ylt_fixed.cu): a persistent CTA
 // per SM, the bitmap folded into shared memory, a warp per trial streaming its
@@ -93,14 +94,6 @@ __device__ __forceinline__ AdjRecord ld_record(const AdjRecord* p) {
 
 // Bits 0-3 of m to the lowest bits of four bytes.
 __device__ __forceinline__ uint32_t spread4(uint32_t m) { return ((m & 15u) * 0x00204081u) & 0x01010101u; }
-
-// (h, l) += v, keeping the rounding error of the FP32 add (two-sum)
-__device__ __forceinline__ void two_sum_add(float& h, float& l, float v) {
-    const float t = h + v;
-    const float bp = t - h;
-    l += (h - (t - bp)) + (v - bp);
-    h = t;
-}
 
 // The layers covering column k, as the group's membership lists them.
 __device__ __forceinline__ uint32_t layers_of(const GroupArgs& g, int k) {
@@ -584,10 +577,10 @@ struct Scratch {
     uint8_t* col;        // the group's column of each pool ELT (NULL without the CSR)
 };
 
+// Records and pass of one group; *nblk CTA partials are left in the scratch.
 template <int NP, int LT>
-cudaError_t launch_one(const art_portfolio* p, const GroupArgs& g, const GroupIndex& gix, const YetArgs& y,
-                       const uint8_t* branch, const double* gw, const Scratch& sc, double* grad_terms,
-                       double* grad_mult, cudaStream_t s) {
+cudaError_t launch_one(const art_portfolio* p, const GroupArgs& g, const YetArgs& y, const uint8_t* branch,
+                       const double* gw, const Scratch& sc, int* nblk, cudaStream_t s) {
     const int32_t C = y.catalogue;
     const int32_t words_w = (int32_t)(((int64_t)C + 31) / 32);  // words the record kernel writes
     adj_records_kernel<NP, LT><<<(unsigned)(((int64_t)words_w * 32 + 255) / 256), 256, 0, s>>>(
@@ -611,22 +604,33 @@ cudaError_t launch_one(const art_portfolio* p, const GroupArgs& g, const GroupIn
     // a CTA's warps take neighbouring trials (they share the sectors of the
     // branch codes and weights); few trials are spread over the SMs instead
     const bool many = y.n_trials >= (int64_t)p->num_sms * NWARP;
-    const int64_t nblk = many ? p->num_sms : std::max<int64_t>(1, std::min<int64_t>(p->num_sms, y.n_trials));
-    kern<<<(unsigned)nblk, 32 * NWARP, smem, s>>>(g, y, sc.records, sc.bits, smem_words, many ? 1 : nblk,
+    const int64_t blocks = many ? p->num_sms : std::max<int64_t>(1, std::min<int64_t>(p->num_sms, y.n_trials));
+    kern<<<(unsigned)blocks, 32 * NWARP, smem, s>>>(g, y, sc.records, sc.bits, smem_words, many ? 1 : blocks,
                                                   many ? NWARP : 1, branch, gw, sc.partial, p->d_flags);
-    if ((e = cudaGetLastError())) return e;
-    group_scatter_kernel<<<1, 1024, 0, s>>>(sc.partial, (int)nblk, LT, NP, gix, grad_terms, grad_mult);
+    *nblk = (int)blocks;
     return cudaGetLastError();
 }
 
 template <int NP>
-cudaError_t launch_lt(const art_portfolio* p, const GroupArgs& g, const GroupIndex& gix, const YetArgs& y,
-                      const uint8_t* branch, const double* gw, const Scratch& sc, double* gt, double* gm,
-                      cudaStream_t s) {
-    if (g.n_layers <= 1) return launch_one<NP, 1>(p, g, gix, y, branch, gw, sc, gt, gm, s);
-    if (g.n_layers <= 2) return launch_one<NP, 2>(p, g, gix, y, branch, gw, sc, gt, gm, s);
-    if (g.n_layers <= 4) return launch_one<NP, 4>(p, g, gix, y, branch, gw, sc, gt, gm, s);
-    return launch_one<NP, 8>(p, g, gix, y, branch, gw, sc, gt, gm, s);
+cudaError_t launch_lt(const art_portfolio* p, const GroupArgs& g, const YetArgs& y, const uint8_t* branch,
+                      const double* gw, const Scratch& sc, int* nblk, int* lt, cudaStream_t s) {
+    *lt = g.n_layers <= 1 ? 1 : g.n_layers <= 2 ? 2 : g.n_layers <= 4 ? 4 : 8;
+    switch (*lt) {
+        case 1: return launch_one<NP, 1>(p, g, y, branch, gw, sc, nblk, s);
+        case 2: return launch_one<NP, 2>(p, g, y, branch, gw, sc, nblk, s);
+        case 4: return launch_one<NP, 4>(p, g, y, branch, gw, sc, nblk, s);
+        default: return launch_one<NP, 8>(p, g, y, branch, gw, sc, nblk, s);
+    }
+}
+
+// Whether a group takes the rows' form: its losses per catalogue event reach
+// the number at which both forms took the same time (500,000 catalogue events,
+// 30,000 trials of 1,000): 1.3 for one layer of 8 or 16 ELTs, 1.9 of 24, 2.6 of
+// 32; 2.5 for eight layers over 16. Up to four ELTs never do.
+bool dense(const art_portfolio* p, size_t gi) {
+    const int np = p->group_np[gi];
+    const float by_layers = 1.3f + 0.17f * (float)(p->groups[gi].n_layers - 1);
+    return np > 4 && p->group_losses[gi] > std::max(by_layers, np >= 32 ? 2.6f : np >= 24 ? 1.9f : 0.0f);
 }
 
 }  // namespace
@@ -635,23 +639,35 @@ cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& yet, const ui
                                   double* grad_terms, double* grad_mult, cudaStream_t s) {
     YetArgs y = yet;
     y.by_id = !ids_on_device(y);
+    std::vector<bool> rows(p->groups.size());
+    bool any_records = false;
+    for (size_t gi = 0; gi < rows.size(); ++gi) {
+        rows[gi] = dense(p, gi);
+        any_records = any_records || !rows[gi];
+    }
     const size_t C = (size_t)p->catalogue;
-    const size_t rec_bytes = sizeof(AdjRecord) * C;
-    const size_t bit_bytes = 16 * ((C / 32 + 1 + 3) / 4);
+    const size_t bit_bytes = (16 * ((C / 32 + 1 + 3) / 4) + 255) & ~(size_t)255;
     const size_t part_bytes = sizeof(double) * (size_t)p->num_sms * (4 * kMaxGroupLayers + kMaxLayerElts);
-    const size_t a1 = (rec_bytes + 255) & ~(size_t)255, a2 = (bit_bytes + 255) & ~(size_t)255;
+    const size_t mask_bytes = (sizeof(uint2) * (C + 1) + 255) & ~(size_t)255;
+    size_t event_bytes = any_records ? std::max(mask_bytes, (sizeof(AdjRecord) * C + 255) & ~(size_t)255) : mask_bytes;
     char* w = nullptr;
-    cudaError_t err = scratch_alloc((void**)&w, a1 + a2 + part_bytes, s);
+    cudaError_t err = scratch_alloc((void**)&w, event_bytes + bit_bytes + part_bytes, s);
+    if (err == cudaErrorMemoryAllocation && any_records) {
+        cudaGetLastError();  // no room for 32 bytes per catalogue event: the rows' form takes 8
+        rows.assign(rows.size(), true);
+        event_bytes = mask_bytes;
+        err = scratch_alloc((void**)&w, event_bytes + bit_bytes + part_bytes, s);
+    }
     if (err) return err;
-    Scratch sc{reinterpret_cast<AdjRecord*>(w), reinterpret_cast<uint32_t*>(w + a1),
-               reinterpret_cast<double*>(w + a1 + a2), nullptr};
+    Scratch sc{reinterpret_cast<AdjRecord*>(w), reinterpret_cast<uint32_t*>(w + event_bytes),
+               reinterpret_cast<double*>(w + event_bytes + bit_bytes), nullptr};
     do {
         if ((err = cudaMemsetAsync(grad_terms, 0, sizeof(double) * 4 * p->n_layers, s))) break;
         if ((err = cudaMemsetAsync(grad_mult, 0, sizeof(double) * p->n_elt, s))) break;
         if (y.n_trials == 0) break;
         // the bitmap's padding words stay zero for every group
-        if ((err = cudaMemsetAsync(sc.bits, 0, a2, s))) break;
-        for (size_t gi = 0; gi < p->groups.size() && !err; ++gi) {
+        if ((err = cudaMemsetAsync(sc.bits, 0, bit_bytes, s))) break;
+        for (size_t gi = 0; gi < p->groups.size(); ++gi) {
             const GroupArgs& ga = p->groups[gi];
             GroupIndex gix{};
             gix.n_elt = (int32_t)p->group_elts[gi].size();
@@ -659,16 +675,23 @@ cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& yet, const ui
             for (int k = 0; k < gix.n_elt; ++k) gix.elt[k] = p->group_elts[gi][k];
             for (int j = 0; j < gix.n_layers; ++j) gix.layer[j] = p->group_layers[gi][j];
             sc.col = p->d_group_col ? p->d_group_col + gi * (size_t)p->pool_np : nullptr;
-            double* gt = grad_terms;
-            double* gm = grad_mult;
-            switch (p->group_np[gi]) {
-                case 4: err = launch_lt<4>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
-                case 8: err = launch_lt<8>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
-                case 16: err = launch_lt<16>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
-                case 24: err = launch_lt<24>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
-                case 32: err = launch_lt<32>(p, ga, gix, y, branch, g, sc, gt, gm, s); break;
-                default: err = cudaErrorInvalidValue;
+            int nblk = 0, lt = 0;
+            if (rows[gi]) {
+                err = launch_adjoint_rows(p, gi, y, branch, g, reinterpret_cast<uint2*>(w), sc.bits, sc.partial, &nblk,
+                                          &lt, s);
+            } else {
+                switch (p->group_np[gi]) {
+                    case 4: err = launch_lt<4>(p, ga, y, branch, g, sc, &nblk, &lt, s); break;
+                    case 8: err = launch_lt<8>(p, ga, y, branch, g, sc, &nblk, &lt, s); break;
+                    case 16: err = launch_lt<16>(p, ga, y, branch, g, sc, &nblk, &lt, s); break;
+                    case 24: err = launch_lt<24>(p, ga, y, branch, g, sc, &nblk, &lt, s); break;
+                    case 32: err = launch_lt<32>(p, ga, y, branch, g, sc, &nblk, &lt, s); break;
+                    default: err = cudaErrorInvalidValue;
+                }
             }
+            if (err) break;
+            group_scatter_kernel<<<1, 1024, 0, s>>>(sc.partial, nblk, lt, p->group_np[gi], gix, grad_terms, grad_mult);
+            if ((err = cudaGetLastError())) break;
         }
     } while (0);
     const cudaError_t e2 = cudaFreeAsync(w, s);

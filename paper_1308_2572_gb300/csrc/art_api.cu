@@ -522,8 +522,16 @@ cudaError_t build_groups(art_portfolio* p, const float* losses, cudaStream_t str
     p->group_tab.assign(ng, nullptr);
     p->group_bitmap.assign(ng, nullptr);
     int32_t* d_el = nullptr;
+    unsigned long long* d_n = nullptr;  // per group: non-zero losses
+    std::vector<unsigned long long> n_losses(ng, 0);
     cudaError_t e = cudaMalloc(&d_el, sizeof(int32_t) * kMaxLayerElts * ng);
-    if (e) return e;
+    if (!e) e = cudaMalloc(&d_n, sizeof(unsigned long long) * ng);
+    if (!e) e = cudaMemsetAsync(d_n, 0, sizeof(unsigned long long) * ng, stream);
+    if (e) {
+        cudaFree(d_el);
+        cudaFree(d_n);
+        return e;
+    }
     for (size_t gi = 0; gi < ng && !e; ++gi) {
         const std::vector<int32_t>& el = p->group_elts[gi];
         const int np = pad_np((int)el.size());
@@ -539,14 +547,19 @@ cudaError_t build_groups(art_portfolio* p, const float* losses, cudaStream_t str
         if ((e = build_layer_table(losses, p->catalogue, d_el + gi * kMaxLayerElts, (int32_t)el.size(), np,
                                    p->group_tab[gi], stream)))
             break;
-        if ((e = build_group_bitmap(p->group_tab[gi], p->catalogue, np, p->group_bitmap[gi], stream))) break;
+        if ((e = build_group_bitmap(p->group_tab[gi], p->catalogue, np, p->group_bitmap[gi], d_n + gi, stream))) break;
         p->groups[gi].table = p->group_tab[gi];
         p->groups[gi].bitmap = p->group_bitmap[gi];
     }
+    if (!e)
+        e = cudaMemcpyAsync(n_losses.data(), d_n, sizeof(unsigned long long) * ng, cudaMemcpyDeviceToHost, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
     cudaFree(d_el);
+    cudaFree(d_n);
     if (e) return e;
     if (e2) return e2;
+    p->group_losses.resize(ng);
+    for (size_t gi = 0; gi < ng; ++gi) p->group_losses[gi] = (float)((double)n_losses[gi] / p->catalogue);
     if (p->sp_ptr) {  // the adjoint's records come from the CSR
         std::vector<uint8_t> col(ng * p->pool_np, 255);
         for (size_t gi = 0; gi < ng; ++gi)

@@ -38,6 +38,14 @@ __device__ __forceinline__ double fin_f64(double y, double m, double d, double l
     return fmin(fmax(fma(m, y, -d), 0.0), lim);
 }
 
+// (h, l) += v, keeping the rounding error of the FP32 add (two-sum)
+__device__ __forceinline__ void two_sum_add(float& h, float& l, float v) {
+    const float t = h + v;
+    const float bp = t - h;
+    l += (h - (t - bp)) + (v - bp);
+    h = t;
+}
+
 // Aggregate branch code stored for the adjoint: 1 strictly between the
 // retention and retention + limit, 2 strictly above, 0 otherwise.
 __device__ __forceinline__ uint8_t agg_branch(double s, double r, double l) {
@@ -362,6 +370,7 @@ struct art_portfolio {
     std::vector<std::vector<int32_t>> group_layers; // layer ids per group
     std::vector<float*> group_tab;
     std::vector<uint32_t*> group_bitmap;
+    std::vector<float> group_losses;                // mean non-zero losses per catalogue event and group
     uint8_t* d_group_col = nullptr;             // [n_groups][pool_np]: the group's column of an ELT (255: none)
 
     // skip variant (needs ART_LAYOUT_LAYER): occurrence groups and their
@@ -460,7 +469,8 @@ cudaError_t launch_fixed_group(const OccGroupArgs& g, const YetArgs& y, int lp, 
                                uint8_t* branch, int* flags, cudaStream_t s);
 cudaError_t launch_skip64(art_portfolio* p, const YetArgs& y, double* ylt, uint8_t* branch, cudaStream_t s,
                           bool build = true);
-cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap, cudaStream_t s);
+cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap,
+                               unsigned long long* losses, cudaStream_t s);
 // Write every occurrence group's X and bitmap (one launch); whole: as whole
 // numbers in the groups whose losses allow it.
 cudaError_t build_occurrence(art_portfolio* p, bool whole, const EventGate& gate, cudaStream_t s);
@@ -470,6 +480,11 @@ cudaError_t launch_adjoint(art_portfolio* p, const YetArgs& y, const uint8_t* br
                            double* grad_terms, double* grad_mult, cudaStream_t s);
 cudaError_t launch_adjoint_groups(art_portfolio* p, const YetArgs& y, const uint8_t* branch, const double* g,
                                   double* grad_terms, double* grad_mult, cudaStream_t s);
+// One layer group by its table rows (adjoint_rows.cu): masks [catalogue + 1],
+// zero-padded bits, *nblk CTA partials of 4 * *lt + row width values.
+cudaError_t launch_adjoint_rows(const art_portfolio* p, size_t gi, const YetArgs& y, const uint8_t* branch,
+                                const double* gw, uint2* masks, uint32_t* bits, double* partial, int* nblk, int* lt,
+                                cudaStream_t s);
 // The metrics over scratch of at least metrics_scratch_bytes(...) bytes
 // (scratch NULL or smaller: taken from the stream-ordered allocator and
 // released on the stream).

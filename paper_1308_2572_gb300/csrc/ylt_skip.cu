@@ -749,22 +749,26 @@ cudaError_t launch_group(const OccGroupArgs& g, const YetArgs& y, int num_sms, i
     return cudaGetLastError();
 }
 
-// Bitmap of a group table: bit i set when row i has any non-zero entry.
+// Bitmap of a group table (bit i set when row i has any non-zero entry) and the
+// number of its non-zero entries.
 __global__ void build_bitmap_kernel(const float* __restrict__ table, int32_t catalogue, int32_t np,
-                                    uint32_t* __restrict__ bitmap) {
+                                    uint32_t* __restrict__ bitmap, unsigned long long* __restrict__ losses) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool nz = false;
+    unsigned n = 0;
     if (i < catalogue)
-        for (int k = 0; k < np; ++k) nz |= table[i * np + k] != 0.0f;
-    const unsigned m = __ballot_sync(0xffffffffu, nz);
+        for (int k = 0; k < np; ++k) n += table[i * np + k] != 0.0f;
+    const unsigned m = __ballot_sync(0xffffffffu, n != 0);
     if ((threadIdx.x & 31) == 0 && i < catalogue) bitmap[i >> 5] = m;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(losses, (unsigned long long)n);
 }
 
 }  // namespace
 
-cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap, cudaStream_t s) {
+cudaError_t build_group_bitmap(const float* table, int32_t catalogue, int32_t np, uint32_t* bitmap,
+                               unsigned long long* losses, cudaStream_t s) {
     const int64_t n = ((int64_t)catalogue + 31) / 32 * 32;
-    build_bitmap_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(table, catalogue, np, bitmap);
+    build_bitmap_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(table, catalogue, np, bitmap, losses);
     return cudaGetLastError();
 }
 
