@@ -530,6 +530,16 @@ ART_API art_status art_get_footprint(const art_portfolio* p, int64_t* layer_byte
  * first). NULL is a no-op. No counterpart in the paper; never fails. */
 ART_API void art_destroy_portfolio(art_portfolio* p);
 
+/*
+ * art_release_scratch -- give back the device memory that the library keeps
+ * between calls on the current device (the paper has no counterpart). The
+ * metrics, their gradient, the adjoint and the payouts take their scratch from
+ * a pool that keeps up to 256 MB per device; destroying the device's last
+ * portfolio gives it back too. Scratch of work in flight stays. Thread-safe.
+ * Errors: ART_ECUDA.
+ */
+ART_API art_status art_release_scratch(void);
+
 /* Static, human-readable name of a status (an unknown code gets a generic
  * name). No counterpart in the paper; never fails. */
 ART_API const char* art_status_string(art_status s);

@@ -27,7 +27,8 @@ EXPORTS = ("art_create_portfolio", "art_update_terms", "art_get_terms", "art_set
            "art_run_ylt_host", "art_metrics", "art_metrics_backward", "art_run_ylt_backward",
            "art_get_device_status", "art_get_footprint", "art_destroy_portfolio", "art_status_string",
            "art_last_cuda_error", "art_version", "art_metrics_noalloc", "art_probe", "art_autotune",
-           "art_run_payouts", "art_set_flags", "art_run_ylt_host_metrics", "art_topk", "art_merge_topk")
+           "art_run_payouts", "art_set_flags", "art_run_ylt_host_metrics", "art_topk", "art_merge_topk",
+           "art_release_scratch")
 
 
 class LayerTerms(ctypes.Structure):
@@ -90,6 +91,7 @@ def lib():
         "art_status_string": ([st], ctypes.c_char_p),
         "art_last_cuda_error": ([], ctypes.c_char_p),
         "art_version": ([], i32),
+        "art_release_scratch": ([], st),
         "art_probe": ([i32, i64, i32, P], st),
         "art_autotune": ([P, i64, P, P, i32, P, i32, P, P], st),
         "art_run_payouts": ([P, i32, i64, P, P, i32, P, P, P, P], st),
@@ -339,6 +341,12 @@ def art_get_footprint(p):
 
 def art_destroy_portfolio(p) -> None:
     lib().art_destroy_portfolio(_h(p))
+
+
+def art_release_scratch() -> None:
+    """Give back the device memory the library keeps between calls (up to
+    256 MB per device)."""
+    _check(lib().art_release_scratch(), "art_release_scratch")
 
 
 def art_status_string(status: int) -> str:

@@ -662,8 +662,8 @@ void free_portfolio(art_portfolio* p) {
     cudaFree(p->host_scratch);
     if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
+    scratch_user(p->device, -1);
     delete p;
-    scratch_user(-1);
 }
 
 // Times in us of a forward over n trials of E events in all, for the choice
@@ -840,12 +840,12 @@ art_status art_create_portfolio(int32_t catalogue_size, int32_t n_elt, const flo
         delete p;
         return ART_EINVAL;
     }
-    scratch_user(+1);
 
-    cudaError_t e;
+    cudaError_t e = cudaGetDevice(&p->device);
     art_status st = ART_OK;
+    scratch_user(p->device, +1);
     do {
-        if ((e = cudaGetDevice(&p->device))) break;
+        if (e) break;
         if ((e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device))) break;
         if ((e = cudaMalloc(&p->d_flags, sizeof(int) * kNumFlags))) break;
         if ((e = cudaMemsetAsync(p->d_flags, 0, sizeof(int) * kNumFlags, stream))) break;

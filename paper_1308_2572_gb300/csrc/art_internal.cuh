@@ -536,9 +536,9 @@ cudaError_t allow_max_shared(K* kern) {
 // Stream-ordered scratch of one call (release it with cudaFreeAsync), from a
 // pool that keeps a bounded amount between calls (scratch.cu).
 cudaError_t scratch_alloc(void** out, size_t bytes, cudaStream_t s);
-// A portfolio was made (+1) or destroyed (-1): the last one's end trims the
-// current device's pool.
-void scratch_user(int delta);
+// A portfolio of the device was made (+1) or destroyed (-1): the last one's end
+// trims the device's pool.
+void scratch_user(int device, int delta);
 // Id of the current device's context; 0 if the driver cannot tell.
 unsigned long long current_context_id();
 // Bytes from a device address to the end of its allocation; the largest

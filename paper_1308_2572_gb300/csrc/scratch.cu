@@ -6,8 +6,9 @@
 // caller that reads each result paid the mapping of the same scratch on every
 // call (art_metrics on one layer of 1,000,000 trials, each call waited for:
 // 293 us, 111 from this pool; not waited for, both 89). This pool keeps up to
-// kScratchKeep bytes instead; what it keeps is returned when the process's
-// last portfolio is destroyed.
+// kScratchKeep bytes instead; what it keeps is returned when the device's last
+// portfolio is destroyed, or by art_release_scratch (the metrics need no
+// portfolio).
 #include <mutex>
 
 #include "art_internal.cuh"
@@ -69,8 +70,18 @@ struct DevicePool {
     unsigned long long ctx_id = 0;  // the context the pool was made in
 };
 DevicePool g_pools[kMaxDevices];
-int64_t g_portfolios = 0;  // live portfolios of the process
-std::mutex g_mutex;        // guards both
+int64_t g_portfolios[kMaxDevices];  // live portfolios of each device
+std::mutex g_mutex;                 // guards both
+
+// Give back what the current device's pool keeps; memory that work in flight
+// still uses stays. With g_mutex held.
+cudaError_t trim_current() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) return e;
+    if (!g_pools[dev].pool || g_pools[dev].ctx_id != current_context_id()) return cudaSuccess;
+    return cudaMemPoolTrimTo(g_pools[dev].pool, 0);
+}
 
 // The current device's pool; NULL where it cannot be had (the device's
 // default pool serves then). A context recreated after a device reset makes
@@ -115,14 +126,20 @@ cudaError_t scratch_alloc(void** out, size_t bytes, cudaStream_t s) {
     return pool ? cudaMallocFromPoolAsync(out, bytes, pool, s) : cudaMallocAsync(out, bytes, s);
 }
 
-void scratch_user(int delta) {
+void scratch_user(int device, int delta) {
+    if (device < 0 || device >= kMaxDevices) return;
     std::lock_guard<std::mutex> lock(g_mutex);
-    g_portfolios += delta;
-    if (delta > 0 || g_portfolios > 0) return;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
-    // memory that work in flight still uses stays
-    if (g_pools[dev].pool && g_pools[dev].ctx_id == current_context_id()) cudaMemPoolTrimTo(g_pools[dev].pool, 0);
+    g_portfolios[device] += delta;
+    int current = -1;
+    if (delta > 0 || g_portfolios[device] > 0 || cudaGetDevice(&current) != cudaSuccess || current != device) return;
+    trim_current();
 }
 
 }  // namespace art
+
+extern "C" art_status art_release_scratch(void) {
+    std::lock_guard<std::mutex> lock(art::g_mutex);
+    const cudaError_t e = art::trim_current();
+    if (e) art::set_last_error(e);
+    return e ? ART_ECUDA : ART_OK;
+}

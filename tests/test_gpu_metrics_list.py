@@ -106,3 +106,31 @@ def test_repeating_values_at_the_threshold(n):
             # one or two roundings against the oracle's sequential FP64 sums; subnormal units
             np.testing.assert_allclose(mean.cpu().numpy(), om, rtol=1e-12, atol=1e-323)
             np.testing.assert_allclose(tvar.cpu().numpy(), ot, rtol=1e-12, atol=1e-323)
+
+
+def test_repeating_values_take_no_longer():
+    """Full limits only (0, 1, 2, ... times one), where the list would overflow,
+    against losses that do not repeat; and few layers of long lists against
+    ranks that no list serves. Wide bounds: a wrong form takes 3 to 60 times."""
+    def time_us(y, probs):
+        L, n = y.shape
+        out = [torch.empty(s, dtype=torch.float64, device="cuda") for s in (L, (L, len(probs)), (L, len(probs)))]
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            art.art_metrics(y, n, L, probs, *out)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        return min(times)
+
+    g = torch.Generator(device="cuda").manual_seed(3)
+    for L, n in [(1, 1_000_000), (64, 300_000)]:
+        plain = torch.exp(15.0 + torch.randn((L, n), generator=g, device="cuda")).double()
+        atoms = torch.poisson(torch.full((L, n), 0.2, device="cuda"), generator=g).double() * 5e6
+        probs = [0.99, 0.996, 0.999]
+        assert time_us(atoms, probs) <= 4.0 * time_us(plain, probs)
+    long = torch.exp(15.0 + torch.randn((1, 30_000_000), generator=g, device="cuda")).double()
+    probs = [0.951, 0.97, 0.99]
+    assert time_us(long, probs) <= 2.5 * time_us(long, [0.9] + probs[1:])
