@@ -317,8 +317,8 @@ ART_API art_status art_run_ylt_host_metrics(art_portfolio* p, int64_t n_trials, 
  * events that evaluating each catalogue event once, as whole numbers, pays (one
  * or two million of them for a catalogue of two million; for a CSR whose length
  * the host cannot bound the device decides). That takes scratch from the
- * stream-ordered allocator. Otherwise the call runs FP64 arithmetic per event
- * and is several times slower. Errors: ART_EINVAL, ART_EUNSUPPORTED, ART_ENOMEM, ART_ECUDA.
+ * stream-ordered allocator, so a call under a caller's capture does without.
+ * Otherwise the call runs FP64 arithmetic per event and is several times slower. Errors: ART_EINVAL, ART_EUNSUPPORTED, ART_ENOMEM, ART_ECUDA.
  */
 ART_API art_status art_run_payouts(art_portfolio* p, int32_t layer, int64_t n_trials, const int32_t* event_ids_dev,
                                    const int64_t* trial_off_dev, int32_t events_per_trial, double* payouts_dev,

@@ -324,6 +324,9 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
     int e2;
     double top;
     if (!ids_on_device(y) || !whole_losses(la.occ_ret, la.occ_lim, lims, &e2, &top)) return cudaSuccess;
+    // the table would put allocation nodes into a caller's graph, which then
+    // could neither be a child graph nor run twice at a time
+    if (captured_by_caller(p, s)) return cudaSuccess;
     const double n = (double)y.n_trials, table_us = (double)p->catalogue * np * 4.0 / 3.5e6;
     auto steps = [&](double E, double ids) { return std::max(n, E / ids + 0.5 * n); };
     int64_t split = 0;
