@@ -515,7 +515,8 @@ ART_API art_status art_autotune(art_portfolio* p, int64_t n_trials, const int32_
 /* Synchronise the stream, then read and clear the portfolio's device error
  * flags: ART_OK, ART_EID_RANGE (an id outside [0, C) was seen; it counted as
  * zero loss: event ids index the direct-access tables of Section III),
- * ART_EINVAL (decreasing CSR offsets were seen) or ART_ETIMEOUT (a bounded
+ * ART_EINVAL (decreasing CSR offsets were seen, or a trial of more than
+ * 4,294,963,200 events; the trial counts as empty) or ART_ETIMEOUT (a bounded
  * wait of a kernel gave up: the outputs of that call are not complete). Errors of the call itself:
  * ART_EINVAL (NULL portfolio), ART_ECUDA. */
 ART_API art_status art_get_device_status(art_portfolio* p, cudaStream_t stream);

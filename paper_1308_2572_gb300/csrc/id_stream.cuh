@@ -11,6 +11,8 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr uint64_t kWaitNs = 4000000000ULL;  // longest wait for a copy
+// Most events of a trial: positions are 32-bit, and a chunk's end must not wrap.
+constexpr int64_t kMaxTrialIds = 0xfffff000LL;
 
 __device__ __forceinline__ uint64_t now_ns() {
     uint64_t t;
@@ -40,7 +42,7 @@ struct Span {
 template <bool VEC>
 struct Trials {
     int64_t stride = 0;  // VEC: ids from trial to trial
-    bool bad = false;    // a decreasing pair of offsets was seen
+    bool bad = false;    // a decreasing pair of offsets, or one too far apart, was seen
 
     __device__ __forceinline__ Trials(const YetArgs& y, int64_t n_warps) {
         if constexpr (VEC) stride = n_warps * (int64_t)y.k;
@@ -55,6 +57,10 @@ struct Trials {
             int64_t b, e;
             bool bo;
             trial_range(y, t, b, e, bo);
+            if (e - b > kMaxTrialIds) {
+                bo = true;
+                e = b;
+            }
             bad |= bo;
             // ids between the 16-byte boundary before y.ids and y.ids
             const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(y.ids) >> 2) & 3u;
