@@ -588,12 +588,13 @@ size_t batched_smem(const art_portfolio* p, bool fp64) {
 
 // The persisting L2 area is reserved while a portfolio with ART_FLAG_L2_PERSIST
 // lives: every other access of the process has that much less L2 (payouts of
-// 100,000 trials 0.84 against 0.35 ms). The last one puts back the limit that
-// the first found, and demotes the lines that the passes left persisting.
+// 100,000 trials 0.84 against 0.35 ms). The last one demotes the lines that the
+// passes left persisting and puts back the limit that the first found, unless
+// the caller has set another since.
 std::mutex g_persist_mutex;
 struct PersistArea {
     int users = 0;
-    size_t before = 0;
+    size_t before = 0, reserved = 0;  // the limit as the first found it, and as the last set it
 } g_persist[64];  // per device
 
 cudaError_t reserve_persisting(int device, size_t bytes) {
@@ -602,6 +603,7 @@ cudaError_t reserve_persisting(int device, size_t bytes) {
     cudaError_t e;
     if (a.users == 0 && (e = cudaDeviceGetLimit(&a.before, cudaLimitPersistingL2CacheSize))) return e;
     if ((e = cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, bytes))) return e;
+    if ((e = cudaDeviceGetLimit(&a.reserved, cudaLimitPersistingL2CacheSize))) return e;
     ++a.users;
     return cudaSuccess;
 }
@@ -611,8 +613,10 @@ void release_persisting(int device) {
     PersistArea& a = g_persist[device & 63];
     int current = -1;
     if (--a.users || cudaGetDevice(&current) != cudaSuccess || current != device) return;
+    size_t now = 0;
     cudaCtxResetPersistingL2Cache();
-    cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, a.before);
+    if (cudaDeviceGetLimit(&now, cudaLimitPersistingL2CacheSize) == cudaSuccess && now == a.reserved)
+        cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, a.before);
 }
 
 void free_portfolio(art_portfolio* p) {
