@@ -684,7 +684,7 @@ double whole_skip_us(const art_portfolio* p, double n, double E) {
     const double pairs = losses * p->lids.size() / p->n_elt;  // (loss, layer) per event
     double build = 1e-6 * p->catalogue * runs * (8.0 + 3.3 * losses);
     if (!(p->d_slotmask && p->sp_ptr)) build = (double)p->layer_bytes / 3.5e6;  // reads every layer's rows
-    const double chunks = std::max(n, E / 256.0 + 0.5 * n);
+    const double chunks = std::max(n, E / 256.0 + 0.5 * n) * std::max(1.0, 1800.0 / std::max(1.0, n));
     return build + runs * (8.0 + 1e-3 * (0.25 * n + 0.33 * chunks) + 1.1e-6 * E * std::min(1.0, pairs / runs));
 }
 

@@ -328,7 +328,9 @@ cudaError_t launch_whole(art_portfolio* p, const LayerArgs& la, int np, double l
     // could neither be a child graph nor run twice at a time
     if (captured_by_caller(p, s)) return cudaSuccess;
     const double n = (double)y.n_trials, table_us = (double)p->catalogue * np * 4.0 / 3.5e6;
-    auto steps = [&](double E, double ids) { return std::max(n, E / ids + 0.5 * n); };
+    // a warp takes a trial; below about 2,000 of them it waits for its own loads
+    const double alone = std::max(1.0, 2000.0 / n);
+    auto steps = [&](double E, double ids) { return alone * std::max(n, E / ids + 0.5 * n); };
     int64_t split = 0;
     const ByEvents form = by_events(
         y, -1, [&](double E) { return 5.0 + 0.79e-3 * steps(E, 32.0); },

@@ -115,3 +115,16 @@ def test_default_variant_is_near_the_faster_form(n_layers, nnz, trials, k, room)
         assert t["AUTO"] <= 1.5 * min(t["SKIP"], t["SPARSE"]) + 20.0 + 5.0 * ((n_layers + 7) // 8), t
     finally:
         p.close()
+
+
+def test_payouts_of_a_few_long_trials():
+    """One warp per trial: evaluated event by event one trial of 400,000 events
+    takes about 19 ms, over the table of whole losses about 2."""
+    w = _case(1, 1_000_000, 0.02)
+    ids = torch.from_numpy(np.random.default_rng(2).integers(0, 1_000_000, 400_000, dtype=np.int32)).cuda()
+    p = art.portfolio_from_workload(w, layouts=art.ART_LAYOUT_LAYER)
+    try:
+        pay = torch.empty(400_000, dtype=torch.float64, device="cuda")
+        assert _time_us(lambda: art.art_run_payouts(p, 0, 1, ids, None, 400_000, pay)) <= 8000.0
+    finally:
+        p.close()
