@@ -24,6 +24,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -140,11 +141,18 @@ KERNEL_SOURCES = {"ylt_plain": "ylt_plain.cu", "ylt_skip": "ylt_fixed.cu", "ylt_
 
 
 def kernel_source_hash(kernel: str) -> str:
-    """Hash of the kernel's own source file and the shared device header."""
+    """Hash of the kernel's own source file and of every device header that it
+    includes, directly or through another."""
+    csrc = os.path.join(ROOT, "paper_1308_2572_gb300", "csrc")
     h = hashlib.sha256()
-    for f in (KERNEL_SOURCES[kernel], "art_internal.cuh"):
-        with open(os.path.join(ROOT, "paper_1308_2572_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
+    files = [KERNEL_SOURCES[kernel]]
+    for f in files:  # grows by the headers found
+        with open(os.path.join(csrc, f), "rb") as fh:
+            text = fh.read()
+        h.update(text)
+        for name in re.findall(r'^#include "([^"]+\.cuh)"', text.decode(), re.M):
+            if name not in files:
+                files.append(name)
     return h.hexdigest()[:16]
 
 

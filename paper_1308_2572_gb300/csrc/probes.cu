@@ -41,17 +41,19 @@ __global__ void stream_kernel(const float4* __restrict__ p, int64_t n4, float* _
 }
 
 // Each thread issues `per` independent reads of `width` floats at hashed,
-// width-aligned positions of a buffer of n floats.
+// width-aligned positions of a buffer of n floats. The hash is brought into
+// range by a multiplication's high word: a 64-bit remainder per read bound the
+// probe by its own arithmetic (64 MB, 32-byte reads: 6.8 TB/s, and 9.1 without).
 template <int WIDTH>
 __global__ void gather_kernel(const float* __restrict__ p, int64_t n, int per, float* __restrict__ sink) {
     const int64_t slots = n / WIDTH;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float acc = 0.0f;
-    for (int r = 0; r < per; r += 4) {
-        float v[4];
+    for (int r = 0; r < per; r += 8) {
+        float v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t slot = (int64_t)(mix64(tid * 1315423911ull + r + u) % (uint64_t)slots);
+        for (int u = 0; u < 8; ++u) {
+            const int64_t slot = (int64_t)__umul64hi(mix64(tid * 1315423911ull + r + u), (uint64_t)slots);
             const float* q = p + slot * WIDTH;
             if constexpr (WIDTH == 16) {
                 float w[8], z[8];
@@ -72,7 +74,8 @@ __global__ void gather_kernel(const float* __restrict__ p, int64_t n, int per, f
                 v[u] = __ldg(q);
             }
         }
-        acc += v[0] + v[1] + v[2] + v[3];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += v[u];
     }
     if (acc == -1.0f) *sink = acc;
 }

@@ -172,3 +172,23 @@ def test_bench_help_renders():
                        timeout=120)
     assert r.returncode == 0, r.stderr[-500:]
     assert "--no-l2-persist" in r.stdout
+
+
+def test_source_hash_covers_the_headers(tmp_path, monkeypatch):
+    """A change in a header that a kernel includes (the id copies and the ring
+    of the whole-number passes live in one) makes a recorded traffic stale."""
+    import shutil
+    src = os.path.join(bench.ROOT, "paper_1308_2572_gb300", "csrc")
+    dst = tmp_path / "paper_1308_2572_gb300" / "csrc"
+    shutil.copytree(src, dst)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    before = bench.kernel_source_hash("ylt_skip")
+    for name in ("id_stream.cuh", "art_internal.cuh", "ylt_fixed.cu"):
+        with open(dst / name, "a") as f:
+            f.write("// changed\n")
+        after = bench.kernel_source_hash("ylt_skip")
+        assert after != before, name
+        before = after
+    with open(dst / "metrics.cu", "a") as f:
+        f.write("// another kernel's\n")
+    assert bench.kernel_source_hash("ylt_skip") == before
