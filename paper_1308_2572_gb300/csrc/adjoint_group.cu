@@ -53,8 +53,10 @@
 //
 // What bounds the pass (ncu, c3): issue (58%; 52 instructions per 32 events,
 // of which the two POPC of the ring take 4 of 23 cycles) with 20 warps per SM.
-// c3, 500,000 trials: 1.24 ms, with the records 1.28, against 1.95 for the form
-// that gathered 64-byte rows and tested 16 columns per queued event.
+// c3, 500,000 trials, records included: 1.15 ms (1.11 without the fold after
+// every trial), against 1.95 for the form that gathered 64-byte rows and tested
+// 16 columns per queued event (adjoint_rows.cu; where most events have more than
+// three columns that one is the faster).
 #include <algorithm>
 #include <limits>
 

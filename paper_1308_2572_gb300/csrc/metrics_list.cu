@@ -27,7 +27,7 @@
 // reads and six list passes took 1.04 ms on 128 layers x 1,000,000 trials at
 // three probabilities, this takes 0.27 ms (floor 0.15: the pass issues 37
 // instructions per 32 losses and runs at 0.73 of the copy rate), and one layer's
-// metrics 40 us against 90 (eight dependent launches).
+// metrics 36 us against 90 (eight dependent launches).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

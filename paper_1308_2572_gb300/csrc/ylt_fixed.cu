@@ -11,11 +11,12 @@
 // operations per entry instead of the seven of a compensated FP32 add, and
 // reduces across the warp in two 32-bit REDUX steps instead of five rounds of
 // compensated shuffles. It is rounded to FP64 once. On c1 (1,000,000 trials x
-// 1,000 events, one layer) the forward takes 0.90 ms against 1.27 with the
-// compensated pass, on a group of 8 of c4's layers 3.3 against 3.95 ms per
-// 1,000,000 trials, on c3 (8 layers, few events with a loss) 1.80 against 2.07. Groups with a layer that
-// does not fit (OccR = 0, very wide covers) keep the FP32 table and the
-// compensated pass of ylt_skip.cu.
+// 1,000 events, one layer) the forward takes 0.87 ms against 1.25 with the
+// compensated pass, on a group of 8 of c4's layers 2.9 against 3.8 ms per
+// 1,000,000 trials, on c3 (8 layers, few events with a loss) 1.36 against 2.07.
+// Groups with a layer that does not fit (OccR = 0, very wide covers), calls
+// under a caller's capture and ids in host or managed memory keep the FP32 table
+// and the compensated pass of ylt_skip.cu.
 //
 // The rest of the mapping is that of ylt_skip.cu: persistent 1024-thread
 // CTAs, the bitmap folded into shared memory, a warp per trial streaming its
